@@ -117,7 +117,8 @@ def tensor_roofline(dom, per_launch_ms, peaks):
     inside a long step)."""
     if not dom.get("tensor_flops"):
         return None
-    fl = dom["tensor_flops"] / dom["launches"]
+    # the library counts 16 sums per target; the MMAs form eight of them
+    fl = 0.5 * dom["tensor_flops"] / dom["launches"]
     pk = float(peaks.get("bf16_tflops_sustained", 1700.0)) * 1e12
     return {"flops_per_launch": fl, "achieved": fl / (per_launch_ms / 1e3) / 1e12,
             "peak": pk / 1e12, "unit": "TFLOP/s", "frac": fl / pk * 1e3 / per_launch_ms,

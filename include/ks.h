@@ -58,10 +58,12 @@ extern "C" {
  * element-wise step into the last one (the fusion of Sec. III-B). */
 #define KS_UNFUSED 0x100
 /* OR-ed into the variant: register rounds of radix 4 (4 points per thread, twice the
- * threads per tile) instead of radix 8; more parallelism for small workloads. */
+ * threads per tile) instead of radix 8. The radix, the schedule and the column tiles below
+ * tell kernels apart at N <= 2^12 (the column tiles nowhere); the larger sizes have one set
+ * of kernels, and accept these flags without effect. */
 #define KS_RADIX4 0x200
 /* OR-ed into the variant: register rounds of radix 16 (16 points per thread, half the
- * threads per tile): fewer shared-memory round trips for large workloads. */
+ * threads per tile): fewer shared-memory round trips. */
 #define KS_RADIX16 0x400
 /* Radix schedule, OR-ed into the variant: the register-round radix of one kernel stage,
  * overriding the plan's for that stage only. Stages: KS_ST_INV (the input iNTT and the
@@ -79,10 +81,9 @@ extern "C" {
 #define KS_R8 2
 #define KS_R16 3
 #define KS_STAGE_RADIX(stage, code) ((code) << (KS_STAGE_SHIFT + 2 * (stage)))
-/* OR-ed into the variant: a stage's column pass (N >= 2^13) uses the alternative column
- * tile (2^11 points instead of 2^10 up to N = 2^15, 2^10 instead of 2^11 above): the
- * inverse NTTs (KS_COLALT_INV), the ModUp BConv pass (KS_COLALT_UPC), the ModDown BConv
- * pass (KS_COLALT_DNC), or all three (KS_COLTILE_ALT). */
+/* OR-ed into the variant: names an alternative column tile for the inverse NTTs
+ * (KS_COLALT_INV), the ModUp BConv pass (KS_COLALT_UPC), the ModDown BConv pass
+ * (KS_COLALT_DNC), or all three (KS_COLTILE_ALT). Accepted without effect (see above). */
 #define KS_COLALT_INV 0x4000000
 #define KS_COLALT_UPC 0x8000000
 #define KS_COLALT_DNC 0x10000000
@@ -95,7 +96,7 @@ extern "C" {
 #define KS_SPLIT_DOWN 0x20000000
 /* OR-ed into a fused variant: the ModUp and ModDown basis conversions (Sec. II-A) run on
  * the tensor cores (tcgen05): both operands split into bytes, exact bf16 x bf16 -> fp32
- * products summed below 2^23, recombined into the exact 128-bit sum and reduced once,
+ * products summed below 2^23, recombined into one exact sum and reduced once,
  * fused with the first forward NTT pass (the inverse column passes write the bytes of
  * their output instead of the output). Same result bits as the integer path. Effective
  * on contexts with ks_info.tc = 1 (2^13 <= N <= 2^17, 2 <= alpha <= 9, dnum <= 64); ignored
@@ -353,12 +354,12 @@ int ks_switch_batch(const ks_job *jobs, int njobs, int flags, void *stream);
  * launched by this process: KS_OK, or KS_ETIMEOUT if a bounded wait gave up. */
 int ks_batch_status(void *stream);
 
-/* Autotuner: times the dataflows {DPOB, DSOB, DPOC c=2, DPOC c=4, DSOC c=2} x
- * {radix 8, radix 4, radix 16} on this job (replicated `batch` times, 1..16, in one
- * launch set); then, for N >= 2^13, refines the winner's schedule one coordinate at a
- * time: each stage's radix (KS_STAGE_RADIX), each column pass's tile (KS_COLALT_*) and,
- * for DPOB, the split ModDown (KS_SPLIT_DOWN), a change kept when the KeySwitch gets
- * more than 1.5% faster (best of six timings each). Stores the result as the
+/* Autotuner: times the dataflows {DPOB, DSOB, DPOC c=2, DPOC c=4, DSOC c=2} (N <= 2^12:
+ * each with radix 8, radix 4 and radix 16) on this job (replicated `batch` times, 1..16, in
+ * one launch set); then, for N >= 2^13, tries the tensor-core basis conversions
+ * (KS_BCONV_TC, else KS_BCONV_TC_DOWN) and, for DPOB, the split ModDown (KS_SPLIT_DOWN) on
+ * the winner, a change kept when the KeySwitch gets more than 1.5% faster (best of six
+ * timings each). Stores the result as the
  * context's KS_AUTO plan and writes it to *variant / *chunks. Writes the switched
  * result to out_dev. Synchronizes `stream`; allocates and frees its own scratch. */
 int ks_tune(ks_context *ctx, const uint64_t *d_dev, const uint64_t *evk_dev, uint64_t *out_dev,
@@ -443,7 +444,9 @@ typedef struct {
                     key multiply) and Montgomery reductions; the rest are Shoup products
                     (butterflies, scalings) */
   double tensor_flops; /* summed tensor-core FLOPs (2 per bf16 multiply-add), counted
-                          apart from ops: the basis conversions of KS_BCONV_TC plans */
+                          apart from ops: the basis conversions of KS_BCONV_TC plans, at
+                          the 16 sums per target of a full byte product (the MMAs form
+                          eight: half of this count) */
 } ks_kernel_stat;
 
 int ks_profile_begin(void);

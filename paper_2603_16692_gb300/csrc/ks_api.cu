@@ -33,7 +33,6 @@ struct Plan {
   bool unfused;
   int rl;        // register-round radix of the plan: 3 (8 points per thread), 2 or 4
   int srl[ST_COUNT];  // per stage (the plan's unless the variant's schedule sets one)
-  int ca[ST_COUNT];   // per stage: 1 = alternative column tile (stages with column passes)
   int code;      // every variant bit that changes the launches (graph-cache key)
   bool split;    // KS_SPLIT_DOWN in effect (fused DPOB, two-pass N)
   bool tc_up;    // KS_BCONV_TC in effect (fused, context with a tensor-core path)
@@ -94,10 +93,6 @@ int make_plan(const ks_context *c, int variant, int chunks, Plan *pl) {
     const int code = (variant >> (KS_STAGE_SHIFT + 2 * st)) & 3;  // 0: the plan's radix
     pl->srl[st] = code == 0 ? pl->rl : code + 1;
   }
-  for (int st = 0; st < ST_COUNT; ++st) pl->ca[st] = 0;
-  pl->ca[ST_INV] = (variant & KS_COLALT_INV) ? 1 : 0;
-  pl->ca[ST_UPC] = (variant & KS_COLALT_UPC) ? 1 : 0;
-  pl->ca[ST_DNC] = (variant & KS_COLALT_DNC) ? 1 : 0;
   pl->code = variant & ~0xff;
   pl->split = (variant & KS_SPLIT_DOWN) && base == KS_DPOB && !pl->unfused && c->loga > 0;
   pl->tc_up = (variant & KS_BCONV_TC) && !pl->unfused && c->tc_ap > 0;
@@ -205,7 +200,7 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
   const double NJ = (double)N * J;
   const bool single = c->loga == 0;
   auto stage = [&](int st) -> const LaunchTable & {
-    return *c->ltab[pl.srl[st] - 2][pl.ca[st]];
+    return *c->ltab[pl.srl[st] - 2];
   };
   const LaunchTable &L = stage(ST_INV), &LU = stage(ST_UPC), &LK = stage(ST_KM),
                     &LDC = stage(ST_DNC), &LDR = stage(ST_DNR);
@@ -251,8 +246,7 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
       Tasks tg = up;
       tg.mode = TASK_TARGET;
       const int nconv = L.count(c, up);
-      // tc_tg: the targets the tensor-core form converts (each digit's in groups of
-      // kTcTargets)
+      // tc_tg: the targets the tensor-core form converts (each digit's, in pairs)
       double src_b = 0, conv_ops = 0, tc_tg = 0;
       for (int j = up.j0; j < up.j1; ++j) src_b += dsize(j) * W;
       {
@@ -262,15 +256,16 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
           one.j1 = j + 1;
           const int cnt = L.count(c, one);
           conv_ops += (double)cnt * NJ * (dsize(j) + 1);
-          tc_tg += (cnt + kTcTargets - 1) / kTcTargets * kTcTargets;
+          tc_tg += (cnt + 1) / 2 * 2;
         }
       }
       const double nt = t1 - t0, nd = up.j1 - up.j0;
       const double own = nd * nt - nconv;
       if (!pl.unfused) {
         // the tensor-core form reads the sources as bytes (16 per residue), runs the
-        // products on the tensor cores (tc_ap * 256 FLOPs per target point) and one REDC
-        // per output on the integer pipes
+        // products on the tensor cores (counted as tc_ap * 256 FLOPs per target point: the
+        // 16 slots of a full byte product; the MMAs do half of them) and one REDC per
+        // output on the integer pipes
         if (!single && pl.tc_up)
           KS_TRY(timed(
               "modup_col", nconv * W + 2 * src_b, nconv * (NJ + BF_A), nconv * NJ, s,
@@ -351,7 +346,7 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
         KS_TRY(timed(
             "moddown_col", n * W + 2 * vp_b, n * (NJ + BF_A), n * NJ, s,
             [&] { return launch_bconv_tc(c, js, wo, dn, false, s); },
-            2.0 * ((i1 - i0 + kTcTargets - 1) / kTcTargets * kTcTargets) * NJ * c->tc_ap *
+            2.0 * ((i1 - i0 + 1) / 2 * 2) * NJ * c->tc_ap *
                 256));
       else if (!single)
         KS_TRY(timed("moddown_col", n * W + vp_b, conv + n * BF_A, conv, s,
@@ -506,17 +501,16 @@ int create_context(int dnum, int logn, int L, const u64 *q, const u64 *p, int al
   c->loga = ks::geo_loga(logn);
   c->logb = logn - c->loga;
   c->loggr = ks::geo_loggr(logn);
-  for (int r = 0; r < 3; ++r)
-    for (int ca = 0; ca < 2; ++ca) {
-      const LaunchTable *t = ks::launch_table(logn, r + 2, ca);
-      if (!t || t->prepare() != cudaSuccess) {
-        cudaGetLastError();
-        delete c;
-        return KS_ECUDA;
-      }
-      c->ltab[r][ca] = t;
+  for (int r = 0; r < 3; ++r) {
+    const LaunchTable *t = ks::launch_table(logn, r + 2);
+    if (!t || t->prepare() != cudaSuccess) {
+      cudaGetLastError();
+      delete c;
+      return KS_ECUDA;
     }
-  c->lt = c->ltab[1][0];
+    c->ltab[r] = t;
+  }
+  c->lt = c->ltab[1];
   if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
@@ -1414,12 +1408,11 @@ int ks_tune(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *out
   const int bases[][2] = {{KS_DPOB, 0}, {KS_DSOB, 0}, {KS_DPOC, 2}, {KS_DPOC, 4}, {KS_DSOC, 2}};
   size_t ws_max = 0;
   const int radix[3] = {0, KS_RADIX4, KS_RADIX16};
-  for (auto &b : bases)
-    for (int r : radix) {
-      Plan pl;
-      if (make_plan(c, b[0] | r | KS_BCONV_TC, b[1], &pl) == KS_OK)
-        ws_max = std::max(ws_max, pl.total * 8);
-    }
+  for (auto &b : bases) {
+    Plan pl;
+    if (make_plan(c, b[0] | KS_BCONV_TC, b[1], &pl) == KS_OK)
+      ws_max = std::max(ws_max, pl.total * 8);
+  }
   const size_t out_b = (size_t)2 * c->nq * c->N * 8;
   void *mem = nullptr;
   if (cudaMalloc(&mem, batch * (ws_max + out_b)) != cudaSuccess) {
@@ -1457,11 +1450,11 @@ int ks_tune(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *out
     }
     return ms_min;
   };
-  // 1) dataflow x radix
+  // 1) dataflow, and the radix where it names different kernels (N <= 2^12)
   float best = 1e30f;
   int best_v = KS_DPOB, best_c = 0;
   for (auto &b : bases)
-    for (int ri = 0; ri < 3 && rc == KS_OK; ++ri) {
+    for (int ri = 0; ri < (c->loga > 0 ? 1 : 3) && rc == KS_OK; ++ri) {
       const int v = b[0] | radix[ri];
       const float ms = time_plan(v, b[1], 3);
       if (ms < best) {
@@ -1470,52 +1463,22 @@ int ks_tune(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *out
         best_c = b[1];
       }
     }
-  // 2) the schedule of the winner, one coordinate at a time: each stage's radix, then the
-  // tensor-core basis conversions (both, else the ModDown one alone; a column pass they
-  // replace drops its radix), then each remaining column pass's tile, then the split
-  // ModDown. The winner is re-timed with the same number of repetitions, and a change is
-  // kept only if the whole KeySwitch gets faster by more than the timing noise (1.5%).
+  // 2) two-pass sizes: the tensor-core basis conversions (both, else the ModDown one alone),
+  // then the split ModDown. The winner is re-timed with the same number of repetitions, and
+  // a change is kept only if the whole KeySwitch gets faster by more than the timing noise
+  // (1.5%).
   if (rc == KS_OK && c->loga > 0) {
     best = time_plan(best_v, best_c, 6);
-    const int plan_code3 = (best_v & KS_RADIX4) ? KS_R4 : (best_v & KS_RADIX16) ? KS_R16 : KS_R8;
-    for (int st = 0; st < ST_COUNT && rc == KS_OK; ++st)
-      for (int code = KS_R4; code <= KS_R16 && rc == KS_OK; ++code) {
-        if (code == plan_code3) continue;
-        const int cur = (best_v >> (KS_STAGE_SHIFT + 2 * st)) & 3;
-        if (cur == code) continue;
-        const int v = (best_v & ~KS_STAGE_RADIX(st, 3)) | KS_STAGE_RADIX(st, code);
-        const float ms = time_plan(v, best_c, 6);
-        if (ms < 0.985f * best) {
-          best = ms;
-          best_v = v;
-        }
-      }
-    if (rc == KS_OK && c->tc_ap > 0 && !(best_v & KS_UNFUSED)) {
-      const int up_dn = KS_STAGE_RADIX(ST_UPC, 3) | KS_STAGE_RADIX(ST_DNC, 3);
-      const int cand[2] = {(best_v & ~up_dn) | KS_BCONV_TC,
-                           (best_v & ~KS_STAGE_RADIX(ST_DNC, 3)) | KS_BCONV_TC_DOWN};
-      for (int v : cand) {
-        if (rc != KS_OK) break;
-        const float ms = time_plan(v, best_c, 6);
-        if (ms < 0.985f * best) {
-          best = ms;
-          best_v = v;
-          break;
-        }
-      }
-    }
-    const bool tc_up = (best_v & KS_BCONV_TC) != 0;
-    const bool tc_down = (best_v & (KS_BCONV_TC | KS_BCONV_TC_DOWN)) != 0;
-    for (int bit : {KS_COLALT_INV, KS_COLALT_UPC, KS_COLALT_DNC, KS_SPLIT_DOWN}) {
-      if (rc != KS_OK) break;
-      if ((tc_up && bit == KS_COLALT_UPC) || (tc_down && bit == KS_COLALT_DNC)) continue;
-      if (bit == KS_SPLIT_DOWN && ((best_v & 0xff) != KS_DPOB || (best_v & KS_UNFUSED))) continue;
-      const float ms = time_plan(best_v ^ bit, best_c, 6);
-      if (ms < 0.985f * best) {
-        best = ms;
-        best_v ^= bit;
-      }
-    }
+    auto attempt = [&](int v) {
+      if (rc != KS_OK) return false;
+      const float ms = time_plan(v, best_c, 6);
+      if (ms >= 0.985f * best) return false;
+      best = ms;
+      best_v = v;
+      return true;
+    };
+    if (c->tc_ap > 0 && !attempt(best_v | KS_BCONV_TC)) attempt(best_v | KS_BCONV_TC_DOWN);
+    if ((best_v & 0xff) == KS_DPOB) attempt(best_v | KS_SPLIT_DOWN);
   }
   g_prof.on = prof;
   cudaEventDestroy(e0);

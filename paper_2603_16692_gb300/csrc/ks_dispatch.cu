@@ -41,57 +41,24 @@ const LaunchTable &launch_table_11_4_0();
 const LaunchTable &launch_table_12_3_0();
 const LaunchTable &launch_table_12_2_0();
 const LaunchTable &launch_table_12_4_0();
-const LaunchTable &launch_table_13_3_0();
-const LaunchTable &launch_table_13_3_1();
-const LaunchTable &launch_table_13_2_0();
-const LaunchTable &launch_table_13_2_1();
-const LaunchTable &launch_table_13_4_0();
-const LaunchTable &launch_table_13_4_1();
-const LaunchTable &launch_table_14_3_0();
-const LaunchTable &launch_table_14_3_1();
-const LaunchTable &launch_table_14_2_0();
-const LaunchTable &launch_table_14_2_1();
-const LaunchTable &launch_table_14_4_0();
-const LaunchTable &launch_table_14_4_1();
-const LaunchTable &launch_table_15_3_0();
-const LaunchTable &launch_table_15_3_1();
-const LaunchTable &launch_table_15_2_0();
-const LaunchTable &launch_table_15_2_1();
-const LaunchTable &launch_table_15_4_0();
-const LaunchTable &launch_table_15_4_1();
-const LaunchTable &launch_table_16_3_0();
-const LaunchTable &launch_table_16_3_1();
-const LaunchTable &launch_table_16_2_0();
-const LaunchTable &launch_table_16_2_1();
-const LaunchTable &launch_table_16_4_0();
-const LaunchTable &launch_table_16_4_1();
-const LaunchTable &launch_table_17_3_0();
-const LaunchTable &launch_table_17_3_1();
-const LaunchTable &launch_table_17_2_0();
-const LaunchTable &launch_table_17_2_1();
-const LaunchTable &launch_table_17_4_0();
-const LaunchTable &launch_table_17_4_1();
+const LaunchTable &launch_table_13();
+const LaunchTable &launch_table_14();
+const LaunchTable &launch_table_15();
+const LaunchTable &launch_table_16();
+const LaunchTable &launch_table_17();
 
 namespace {
-// [log N][radix log 2..4][column tile 0/1]; sizes with one pass (N <= 2^12) have no
-// column pass, so both column-tile entries name the same launchers.
+// [log N][radix log 2..4]: the single-pass sizes (N <= 2^12) have kernels per register-round
+// radix; the two-pass sizes have one set, which every radix and column tile names.
 using TableFn = const LaunchTable &(*)();
 struct TableSet {
-  TableFn fn[18][5][2] = {};
+  TableFn fn[18][5] = {};
   TableSet() {
-#define KS_T0(N)                                \
-  for (int c = 0; c < 2; ++c) {                 \
-    fn[N][3][c] = &launch_table_##N##_3_0;      \
-    fn[N][2][c] = &launch_table_##N##_2_0;      \
-    fn[N][4][c] = &launch_table_##N##_4_0;      \
-  }
-#define KS_T1(N)                            \
-  fn[N][3][0] = &launch_table_##N##_3_0;    \
-  fn[N][2][0] = &launch_table_##N##_2_0;    \
-  fn[N][4][0] = &launch_table_##N##_4_0;    \
-  fn[N][3][1] = &launch_table_##N##_3_1;    \
-  fn[N][2][1] = &launch_table_##N##_2_1;    \
-  fn[N][4][1] = &launch_table_##N##_4_1;
+#define KS_T0(N)                       \
+  fn[N][3] = &launch_table_##N##_3_0;  \
+  fn[N][2] = &launch_table_##N##_2_0;  \
+  fn[N][4] = &launch_table_##N##_4_0;
+#define KS_T1(N) fn[N][2] = fn[N][3] = fn[N][4] = &launch_table_##N;
     KS_T0(1) KS_T0(2) KS_T0(3) KS_T0(4) KS_T0(5) KS_T0(6) KS_T0(7) KS_T0(8) KS_T0(9)
     KS_T0(10) KS_T0(11) KS_T0(12)
     KS_T1(13) KS_T1(14) KS_T1(15) KS_T1(16) KS_T1(17)
@@ -101,10 +68,10 @@ struct TableSet {
 };
 }  // namespace
 
-const LaunchTable *launch_table(int logn, int rl, int ca) {
+const LaunchTable *launch_table(int logn, int rl) {
   static const TableSet t;
-  if (logn < 1 || logn > 17 || rl < 2 || rl > 4 || ca < 0 || ca > 1) return nullptr;
-  const TableFn f = t.fn[logn][rl][ca];
+  if (logn < 1 || logn > 17 || rl < 2 || rl > 4) return nullptr;
+  const TableFn f = t.fn[logn][rl];
   return f ? &f() : nullptr;
 }
 

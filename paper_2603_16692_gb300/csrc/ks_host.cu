@@ -124,11 +124,11 @@ bool is_prime_u64(u64 n) { return miller_rabin(n); }
 
 int build_tables(ks_context *c) {
   const int QP = c->qp, nq = c->nq, np = c->np, alpha = c->alpha, beta = c->beta;
-  const int logn = c->logn, loga = c->loga, logb = c->logb, loggr = c->loggr;
+  const int logn = c->logn, loga = c->loga, logb = c->logb;
   const size_t N = (size_t)1 << logn, N1 = (size_t)1 << loga, N2 = (size_t)1 << logb;
-  const size_t GR = (size_t)1 << loggr;
-  const size_t rowlen = (N2 - 1) * N1;
-  const size_t twr_tile = (N2 - 1) * GR;  // entries per row tile
+  // row table: N2 entries per row (row_tw; the last unused), or the N - 1 of a single pass
+  const size_t rowent = loga == 0 ? N2 - 1 : N2;
+  const size_t rowlen = rowent * N1;
 
   std::vector<ModInfo> mod(QP);
   // (the inverse row pass reads the forward row table, mirrored: see ks_ntt.cuh)
@@ -160,19 +160,15 @@ int build_tables(ks_context *c) {
       twc_f[t * N1 + k] = shoup_pair(k ? pw[e] : 1, m);
       twc_i[t * N1 + k] = shoup_pair(k ? pwi[e] : 1, m);
     }
-    // Row table, by row tile b of GR rows (r = b*GR + g), stage-major inside a tile:
-    // entry (b*(N2-1) + 2^ls - 1 + c)*GR + g = psi^brv_logn((N1 + r) 2^ls + c).
-    for (size_t b = 0; b < N1 / GR; ++b)
+    // Row table: stage ls, block c of row r holds psi^brv_logn((N1 + r) 2^ls + c).
+    for (size_t r = 0; r < N1; ++r)
       for (int ls = 0; ls < logb; ++ls)
-        for (size_t cc = 0; cc < ((size_t)1 << ls); ++cc)
-          for (size_t g = 0; g < GR; ++g) {
-            const size_t r = b * GR + g;
-            const size_t k = ((N1 + r) << ls) + cc;
-            const unsigned e = brv((unsigned)k, logn);
-            const size_t idx =
-                t * rowlen + b * twr_tile + ((((size_t)1 << ls) - 1 + cc) << loggr) + g;
-            twr_f[idx] = shoup_pair(pw[e], m);
-          }
+        for (size_t cc = 0; cc < ((size_t)1 << ls); ++cc) {
+          const size_t k = ((N1 + r) << ls) + cc;
+          const unsigned e = brv((unsigned)k, logn);
+          const size_t pos = loga == 0 ? ((size_t)1 << ls) - 1 + cc : (size_t)row_tw(ls, (int)cc);
+          twr_f[t * rowlen + r * rowent + pos] = shoup_pair(pw[e], m);
+        }
   });
 
   // iNTT scales: N^-1 * Qhat_{j,i}^-1 mod q_i for the digit j holding i.
@@ -222,43 +218,47 @@ int build_tables(ks_context *c) {
   }
 
   // Tensor-core basis conversion constants (ks_tc.cu): per (digit, target) / target, a
-  // block [g < 2][k < ap][r < 8][a < 8] of bf16 values, the Toeplitz-shaped B operand:
-  // entry (s = 8g + r, limb k, byte a) = byte s - a of the constant of source k (zero
-  // outside bytes 0..7 and for missing sources), and in slot k = alpha the value 2^23
-  // at a = 0 (it meets the 1.0 the A operand holds there, adding 2^23 to every sum).
+  // block [k < ap][b < 8][a < 8] of bf16 values: byte b of c_k 2^(8a) mod m, where c_k is
+  // the constant of source k times 2^32 (one 32-bit Montgomery step follows; zero for
+  // missing sources), and in slot k = alpha the value 2^23 at a = 0 (it meets the 1.0 the
+  // A operand holds there, adding 2^23 to every sum).
   std::vector<u64> bup, bdown;
   if (c->tc_ap > 0) {
     const int ap = c->tc_ap;
-    const size_t blk = 32 * (size_t)ap;  // words per block (256 ap bytes)
+    const size_t blk = 16 * (size_t)ap;  // words per block (128 ap bytes)
     auto bf16_byte = [](unsigned b) {
       const float f = (float)b;
       uint32_t bits;
       std::memcpy(&bits, &f, 4);
       return (uint16_t)(bits >> 16);
     };
-    auto fill = [&](u64 *dst, const u64 *cst, int ns) {
+    // cst[k] carries a factor that `fix` turns into 2^32 (mod m)
+    auto fill = [&](u64 *dst, const u64 *cst, int ns, u64 fix, u64 m) {
       uint16_t *h = reinterpret_cast<uint16_t *>(dst);
-      for (int g = 0; g < 2; ++g)
-        for (int k = 0; k < ap; ++k)
-          for (int r = 0; r < 8; ++r)
-            for (int a = 0; a < 8; ++a) {
-              const int sl = 8 * g + r, b = sl - a;
-              uint16_t val = 0;
-              if (k < ns && b >= 0 && b <= 7)
-                val = bf16_byte((unsigned)(cst[k] >> (8 * b)) & 0xffu);
-              else if (k == alpha && a == 0)
-                val = 0x4B00;  // 2^23
-              h[((g * ap + k) * 8 + r) * 8 + a] = val;
-            }
+      for (int k = 0; k < ns; ++k) {
+        u64 v = mulm(cst[k], fix, m);
+        for (int a = 0; a < 8; ++a) {
+          for (int b = 0; b < 8; ++b)
+            h[(k * 8 + b) * 8 + a] = bf16_byte((unsigned)(v >> (8 * b)) & 0xffu);
+          v = mulm(v, 256 % m, m);
+        }
+      }
+      for (int b = 0; b < 8; ++b) h[(alpha * 8 + b) * 8] = 0x4B00;  // 2^23
     };
+    // cup carries 2^128 and its result keeps a Montgomery factor 2^64: 2^-32 more turns
+    // the 64-bit step's constant into the 32-bit step's; cdown carries 2^64, likewise
+    std::vector<u64> fix(QP);
+    for (int t = 0; t < QP; ++t) fix[t] = invm(((u64)1 << 32) % c->mods[t], c->mods[t]);
     bup.assign((size_t)beta * QP * blk, 0);
     bdown.assign((size_t)nq * blk, 0);
-    for (int j = 0; j < beta; ++j) {
-      const int lo = j * alpha, ns = std::min(nq, lo + alpha) - lo;
-      for (int t = 0; t < QP; ++t)
-        fill(&bup[((size_t)j * QP + t) * blk], &cup[((size_t)j * QP + t) * alpha], ns);
-    }
-    for (int i = 0; i < nq; ++i) fill(&bdown[(size_t)i * blk], &cdown[(size_t)i * alpha], np);
+    par_for(QP, [&](int t) {
+      for (int j = 0; j < beta; ++j) {
+        const int lo = j * alpha, ns = std::min(nq, lo + alpha) - lo;
+        fill(&bup[((size_t)j * QP + t) * blk], &cup[((size_t)j * QP + t) * alpha], ns, fix[t],
+             c->mods[t]);
+      }
+      if (t < nq) fill(&bdown[(size_t)t * blk], &cdown[(size_t)t * alpha], np, fix[t], c->mods[t]);
+    });
   }
 
   // One device allocation for everything (256-byte aligned pieces).

@@ -1,11 +1,6 @@
-// Kernel instantiations for N = 2^LOGN, LOGN in { 17 }, radix 8, 4 and 16.
-#include "ks_kern.cuh"
+// Kernel instantiations for N = 2^17.
+#include "ks_rows.cuh"
 
 namespace ks {
-#define KS_INST(N, R, C) \
-  const LaunchTable &launch_table_##N##_##R##_##C() { return kern::Launch<N, R, C>::table(); }
-KS_INST(17, 3, 0)
-KS_INST(17, 2, 0)
-KS_INST(17, 4, 0)
-#undef KS_INST
+const LaunchTable &launch_table_17() { return kern::RowFns<17>::table(); }
 }  // namespace ks

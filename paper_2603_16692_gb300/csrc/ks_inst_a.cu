@@ -1,9 +1,9 @@
 // Kernel instantiations for N = 2^LOGN, LOGN in { 1 2 3 4 5 6 }, radix 8, 4 and 16.
-#include "ks_kern.cuh"
+#include "ks_rows.cuh"
 
 namespace ks {
 #define KS_INST(N, R, C) \
-  const LaunchTable &launch_table_##N##_##R##_##C() { return kern::Launch<N, R, C>::table(); }
+  const LaunchTable &launch_table_##N##_##R##_##C() { return kern::LaunchOne<N, R>::table(); }
 KS_INST(1, 3, 0)
 KS_INST(1, 2, 0)
 KS_INST(1, 4, 0)

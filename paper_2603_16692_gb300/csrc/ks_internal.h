@@ -29,6 +29,8 @@ struct ModInfo {
 // Moduli below this take the fast butterflies (no per-stage reduction, approximate
 // Shoup quotients); the bounds they rely on are stated in ks_ntt.cuh.
 constexpr u64 kFastModulus = (u64)1 << 51;
+// ... and below this the mid ones (one conditional subtraction on every other stage).
+constexpr u64 kMidModulus = (u64)1 << 60;
 
 // Work items of one launch, decoded from blockIdx.y (see ks_kern.cuh, decode()).
 // A decoded item packs: bits 0-7 limb, bits 8-15 digit (ModUp) or polynomial
@@ -88,18 +90,19 @@ struct Tables {
   ModInfo *mod;          // [QP]
   ulonglong2 *twc_f;     // [QP][N1]  column-pass forward twiddles (w, w')
   ulonglong2 *twc_i;     // [QP][N1]  column-pass inverse twiddles
-  ulonglong2 *twr_f;     // [QP][N1/GR][N2-1][GR] row-pass twiddles by row tile (the
-                         // inverse row pass reads them mirrored)
+  ulonglong2 *twr_f;     // [QP][N1][N2] row-pass twiddles by row, entries ordered by row_tw
+                         // (ks_ntt.cuh; a single pass: N-1, stage-major); the inverse row
+                         // pass reads them mirrored
   ulonglong2 *iscale_q;  // [nq]  N^-1 * Qhat_{j,i}^-1 mod q_i   (Shoup pair)
   ulonglong2 *iscale_p;  // [np]  N^-1 * Phat_k^-1 mod p_k
   u64 *cup;              // [beta][QP][alpha] (Qhat_{j,i} mod m_t) 2^128 mod m_t
   u64 *cdown;            // [nq][alpha]       (Phat_k mod q_i) 2^64 mod q_i
   ulonglong2 *pinv;      // [nq] P^-1 mod q_i (Shoup pair)
   ulonglong2 *pmod;      // [nq] P mod q_i (Shoup pair), keygen only
-  // Tensor-core basis conversions (ks_tc.cu): the constants of cup / cdown as bf16
-  // bytes in the MMA's B layout, 32 * tc_ap words per (digit, target) / target.
-  u64 *bup;              // [beta][QP][32 tc_ap] (empty when the context has no TC path)
-  u64 *bdown;            // [nq][32 tc_ap]
+  // Tensor-core basis conversions (ks_tc.cu): the conversion constants as bf16 bytes in
+  // the MMA's B layout, 16 * tc_ap words per (digit, target) / target.
+  u64 *bup;              // [beta][QP][16 tc_ap] (empty when the context has no TC path)
+  u64 *bdown;            // [nq][16 tc_ap]
   int *err;              // sticky device error word
 };
 
@@ -108,7 +111,7 @@ constexpr int kTcMaxSets = 64;
 // Tensor-core BConv work items: column tiles of 2^kTcTpLog points, kTcTargets targets
 // (of one source set) per item.
 constexpr int kTcTpLog = 10;
-constexpr int kTcTargets = 2;
+constexpr int kTcTargets = 4;
 // Work of one tensor-core BConv launch: the target groups of every source set, over all
 // column tiles; item = (tile, target group), tile-major (see ks_tc.cu).
 struct TcItems {
@@ -132,10 +135,9 @@ struct ks_context {
   int top_L = -1;  // level of the context whose keys this one uses (-1: itself)
   int N;
   int loga, logb, loggr;  // two-pass split N = 2^loga * 2^logb; rows per row tile 2^loggr
-  // Launchers by register-round radix (index log2 radix - 2: radix 4 has twice the
-  // threads per tile of radix 8, radix 16 half) and column tile (0: default, 1: the
-  // alternative); lt = radix 8, default tiles.
-  const ks::LaunchTable *ltab[3][2] = {};
+  // Launchers by register-round radix (index log2 radix - 2; the two-pass sizes have one
+  // set); lt = radix 8.
+  const ks::LaunchTable *ltab[3] = {};
   const ks::LaunchTable *lt = nullptr;
   int run_up = 1, run_down = 1;  // max terms per exact 128-bit BConv sum
   // Tensor-core basis conversions: K slots per source set (alpha + 1 rounded up to
@@ -250,10 +252,9 @@ int switch_launch_only(ks_context *c, const uint64_t *d, const uint64_t *evk, ui
 // True when ctx's selected plan came from the selector installed now (ks_select.cu).
 bool selected_current(const ks_context *c);
 
-// rl = log2 of the radix of the register rounds (3: 8 points per thread, 2: 4 points
-// per thread, twice the threads per tile; 4: 16 points); ca = 1: the alternative
-// column tile (geo_tile_log_col_alt).
-const LaunchTable *launch_table(int logn, int rl, int ca);
+// rl = log2 of the radix of the register rounds (3: 8 points per thread, 2: 4, 4: 16); it
+// tells kernels apart at N <= 2^12 only.
+const LaunchTable *launch_table(int logn, int rl);
 
 // Tensor-core basis conversion + first forward NTT pass (ks_tc.cu), in place of the
 // fused column passes modup_col (up = true, TASK_UP -> tmp) and moddown_col (TASK_DOWN ->

@@ -226,11 +226,11 @@ template <class GT>
 __device__ __forceinline__ const ulonglong2 *col_table(const ulonglong2 *tab, int prime) {
   return tab + ((size_t)prime << GT::LOGA);
 }
-// Row-pass twiddle slab of (prime, row tile blk): (N2-1)*GR entries, stage-major.
+// Row-pass twiddle slab of (prime, row tile blk): N2 entries per row (a single pass: N-1).
 template <class GT>
 __device__ __forceinline__ const ulonglong2 *row_table(const ulonglong2 *tab, int prime,
                                                        int blk) {
-  return tab + (size_t)prime * (GT::N2 - 1) * GT::N1 + (size_t)blk * GT::TWR;
+  return tab + (size_t)prime * (GT::TWR / GT::GR) * GT::N1 + (size_t)blk * GT::TWR;
 }
 
 __device__ __forceinline__ void stage_consts(u64 *cst, const u64 *__restrict__ src, int n,
@@ -532,18 +532,6 @@ __device__ __forceinline__ void inv_col_body(const KArgs &a, const JobPtr &jp, c
   }
 }
 
-template <int LOGN, int RL, int CA>
-__global__ void __launch_bounds__(GeoT<LOGN, RL, 0, CA>::NT,
-                                  min_blocks(GeoT<LOGN, RL, 0, CA>::NT, RL == 4 ? 512 : 768))
-    k_inv_col(KArgs a, JobSet js, WsOff wo, int which, int split, int pieces) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  int only_o;
-  const int by = inv_grid_row(a, which, split, only_o);
-  inv_col_body<LOGN, RL, CA>(a, js.j[blockIdx.z], wo, which, blockIdx.x, by, raw, only_o,
-                             pieces != 0);
-  pdl_trigger();  // the next kernel may launch once every CTA is here
-}
-
 // Buffers of a forward pass for job jp: the BConv sources and the output buffer.
 template <int PRO>
 __device__ __forceinline__ void fwd_bufs(const JobPtr &jp, const WsOff &wo, int buf,
@@ -561,7 +549,7 @@ __device__ __forceinline__ void fwd_bufs(const JobPtr &jp, const WsOff &wo, int 
 }
 
 // Forward NTT, column pass (global stages 0 .. logN1-1) with a tile producer; the
-// lazy ([0, 4m)) result goes to the output buffer's slot.
+// lazy result goes to the output buffer's slot.
 template <int LOGN, int RL, int PRO, int CA, bool TMA = true>
 __device__ __forceinline__ void fwd_col_body(const KArgs &a, const JobPtr &jp, const WsOff &wo,
                                              const Tasks &tk, int buf, int bx, int by,
@@ -583,21 +571,6 @@ __device__ __forceinline__ void fwd_col_body(const KArgs &a, const JobPtr &jp, c
   tw_ready<TMA>(&twbar, a.tab.err);
   tile_fwd<GT::LOGA, GT::LOGGC, GT::PC, GT::NT, false, RL>(sm, tws, a.tab.mod[t].m);
   store_cols<GT>(dst + (size_t)task_slot(w) * a.N, sm, c0);
-}
-
-// Tiles of 256+ threads: 4 CTAs per SM (64 registers, a few spilled words) measured
-// 1-3% faster on GB300 at N >= 2^16 than the compiler's 78-register choice; smaller
-// tiles keep that choice.
-template <int LOGN, int RL, int PRO, int CA>
-__global__ void __launch_bounds__(GeoT<LOGN, RL, 0, CA>::NT,
-                                  min_blocks(GeoT<LOGN, RL, 0, CA>::NT,
-                                             GeoT<LOGN, RL, 0, CA>::NT >= 256 ? 1024 : 0))
-    k_fwd_col(KArgs a, JobSet js, WsOff wo, Tasks tk, int buf) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  __shared__ u64 cst[kMaxLimbs];
-  fwd_col_body<LOGN, RL, PRO, CA>(a, js.j[blockIdx.z], wo, tk, buf, blockIdx.x, blockIdx.y, raw,
-                                  cst);
-  pdl_trigger();  // the next kernel may launch once every CTA is here
 }
 
 // Plain forward row pass: canonical result back in place.
@@ -636,7 +609,7 @@ __global__ void __launch_bounds__(GeoT<LOGN, RL, 1>::NT)
 // are staged once.
 //
 // The products take ext as the forward pass leaves it (below kFwdLazy * m with the
-// fast butterflies; exact moduli: brought below m by two conditional subtractions),
+// fast butterflies; the other classes: brought below m first),
 // since REDC only needs its input below m 2^64. With at most four elements per
 // thread the products of all digits are summed exactly in 128 bits and reduced once
 // per output word (needs (bound of ext) * (digits) * m < 2^64, checked per CTA; the
@@ -676,7 +649,8 @@ __device__ __forceinline__ void keymult_body(const KArgs &a, const JobPtr &jp, c
   stage_tw<GT, TMA>(tws, row_table<GT>(a.tab.twr_f, t, blk), GT::TWR, &twbar);
   pdl_wait();
   const u64 pol = l2_stream();
-  const bool fast = mi.m < kFastModulus;
+  const int cls = mod_class(mi.m);
+  const bool fast = cls == CLS_FAST;
   // ext stays lazy when the exact digit sum of its products fits one REDC
   const int nd = tk.j1 - tk.j0;
   const bool lazy = fast && (unsigned __int128)(kFwdLazy * (WIDE ? nd : 1)) * mi.m <
@@ -684,8 +658,7 @@ __device__ __forceinline__ void keymult_body(const KArgs &a, const JobPtr &jp, c
   const u64 m2 = 2 * mi.m;
   auto ext_word = [&](u64 y) -> u64 {
     if (lazy) return y;
-    if (!fast) return csub(csub(y, m2), mi.m);  // exact butterflies: below 4m
-    return reduce_full(y, mi.m, mi.mu);
+    return fwd_canon(y, mi.m, mi.mu, cls);
   };
   U128 w0[WIDE ? EPT : 1], w1[WIDE ? EPT : 1];  // exact digit sums (WIDE)
   u64 s0[WIDE ? 1 : EPT], s1[WIDE ? 1 : EPT];    // lazy residue sums in [0, 2m)
@@ -848,7 +821,8 @@ __device__ __forceinline__ void keymult_pipe_body(const KArgs &a, const JobPtr &
   pdl_wait();
   issue_tile(tk.j0, 0);
   cp_async_commit();
-  const bool fast = mi.m < kFastModulus;
+  const int cls = mod_class(mi.m);
+  const bool fast = cls == CLS_FAST;
   const int nd = tk.j1 - tk.j0;
   const bool lazy = fast && (unsigned __int128)(kFwdLazy * (WIDE ? nd : 1)) * mi.m <
                                 (unsigned __int128)1 << 64;
@@ -888,7 +862,7 @@ __device__ __forceinline__ void keymult_pipe_body(const KArgs &a, const JobPtr &
       } else if (lazy) {
         y = x;
       } else {
-        y = fast ? reduce_full(x, mi.m, mi.mu) : csub(csub(x, m2), mi.m);
+        y = fwd_canon(x, mi.m, mi.mu, cls);
       }
       const u64 ka = k0[e], kb = k0[TILE + e];
       if (WIDE) {
@@ -938,12 +912,8 @@ __global__ void __launch_bounds__(GeoT<LOGN, RL, 1>::NT,
   // more NTT per CTA), so starting them first shortens the tail of multi-wave launches
   // (measured on GB300 at (4, 2^16, 35): 125 -> 121 us for this launch).
   const int by = gridDim.y - 1 - blockIdx.y;
-  if constexpr (ROW_PIPE<LOGN, RL>) {
-    keymult_pipe_body<LOGN, RL>(a, js.j[blockIdx.z], wo, tk, blockIdx.x, by, raw);
-  } else {
-    __shared__ u64 cst[GeoT<LOGN, RL, 1>::LOGA == 0 ? kMaxLimbs : 1];
-    keymult_body<LOGN, RL, PRO>(a, js.j[blockIdx.z], wo, tk, blockIdx.x, by, raw, cst);
-  }
+  __shared__ u64 cst[kMaxLimbs];
+  keymult_body<LOGN, RL, PRO>(a, js.j[blockIdx.z], wo, tk, blockIdx.x, by, raw, cst);
   pdl_trigger();  // the next kernel may launch once every CTA is here
 }
 
@@ -965,10 +935,12 @@ __device__ __forceinline__ void moddown_body(const KArgs &a, const JobPtr &jp, c
   const size_t N = a.N;
   const size_t off0 = (size_t)r0 << GT::LOGB;
   // The NTT output z enters the scaling lazy: below kFwdLazy * m (fast butterflies) or,
-  // after one conditional subtraction, below 2m (exact); acc + zb - z is then positive
-  // and below (kFwdLazy + 1) m < 2^64, and the Shoup product by P^-1 takes any word.
-  const bool fast = m < kFastModulus;
-  const u64 m2 = 2 * m, zb = fast ? kFwdLazy * m : m2;
+  // after one conditional subtraction, below 8m (mid) or 2m (exact); acc + zb - z is then
+  // positive and below (kFwdLazy + 1) m, 9m or 3m < 2^64, and the Shoup product by P^-1
+  // takes any word.
+  const int cls = mod_class(m);
+  const bool fast = cls == CLS_FAST;
+  const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
   if (threadIdx.x == 0)
     for (int c = 0; c < 2; ++c) prefetch_l2(acc + ((size_t)c * a.qp + i) * N + off0, GT::TILE * 8);
   __shared__ u64 twbar;
@@ -993,7 +965,7 @@ __device__ __forceinline__ void moddown_body(const KArgs &a, const JobPtr &jp, c
         const int e = threadIdx.x + k * GT::NT;
         if (GT::TILE % GT::NT != 0 && e >= GT::TILE) break;
         const int g = e >> GT::LOGB, x = e & (GT::N2 - 1);
-        const u64 z = fast ? sm[x * GT::PR + g] : csub(sm[x * GT::PR + g], m2);
+        const u64 z = fast ? sm[x * GT::PR + g] : csub(sm[x * GT::PR + g], zs);
         o[e] = addmod(csub(shoup(ac[e] + zb - z, pv.x, pv.y, m), m), ad[e], m);
       }
     } else {
@@ -1002,7 +974,7 @@ __device__ __forceinline__ void moddown_body(const KArgs &a, const JobPtr &jp, c
         const int e = threadIdx.x + k * GT::NT;
         if (GT::TILE % GT::NT != 0 && e >= GT::TILE) break;
         const int g = e >> GT::LOGB, x = e & (GT::N2 - 1);
-        const u64 z = fast ? sm[x * GT::PR + g] : csub(sm[x * GT::PR + g], m2);
+        const u64 z = fast ? sm[x * GT::PR + g] : csub(sm[x * GT::PR + g], zs);
         o[e] = csub(shoup(ac[e] + zb - z, pv.x, pv.y, m), m);
       }
     }
@@ -1042,8 +1014,9 @@ __device__ __forceinline__ void moddown_pipe_body(const KArgs &a, const JobPtr &
   const size_t N = a.N;
   const size_t off0 = (size_t)r0 << GT::LOGB;
   // the NTT output enters the scaling lazy, as in moddown_body
-  const bool fast = m < kFastModulus;
-  const u64 m2 = 2 * m, zb = fast ? kFwdLazy * m : m2;
+  const int cls = mod_class(m);
+  const bool fast = cls == CLS_FAST;
+  const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
   __shared__ u64 twbar;
   stage_tw<GT, TMA>(tws, row_table<GT>(a.tab.twr_f, i, blk), GT::TWR, &twbar);
   pdl_wait();
@@ -1088,7 +1061,7 @@ __device__ __forceinline__ void moddown_pipe_body(const KArgs &a, const JobPtr &
       const int e = threadIdx.x + k * NT;
       if (TILE % NT != 0 && e >= TILE) break;
       const u64 zr = sm[(e & (GT::N2 - 1)) * GT::PR + (e >> GT::LOGB)];
-      const u64 z = fast ? zr : csub(zr, m2);
+      const u64 z = fast ? zr : csub(zr, zs);
       u64 r = csub(shoup(sa[e] + zb - z, pv.x, pv.y, m), m);
       if (add) r = addmod(r, ad[e], m);
       o[e] = r;
@@ -1105,12 +1078,8 @@ __global__ void __launch_bounds__(GeoT<LOGN, RL, 1>::NT,
   // does not wait for this kernel before it ends) start while this one writes its result
   // to host memory
   if (js.j[blockIdx.z].dsrc) pdl_trigger();
-  if constexpr (ROW_PIPE<LOGN, RL>) {
-    moddown_pipe_body<LOGN, RL>(a, js.j[blockIdx.z], wo, tk, blockIdx.x, blockIdx.y, raw);
-  } else {
-    __shared__ u64 cst[GeoT<LOGN, RL, 1>::LOGA == 0 ? kMaxLimbs : 1];
-    moddown_body<LOGN, RL, PRO>(a, js.j[blockIdx.z], wo, tk, blockIdx.x, blockIdx.y, raw, cst);
-  }
+  __shared__ u64 cst[kMaxLimbs];
+  moddown_body<LOGN, RL, PRO>(a, js.j[blockIdx.z], wo, tk, blockIdx.x, blockIdx.y, raw, cst);
   pdl_trigger();  // the next kernel may launch once every CTA is here
 }
 
@@ -1125,128 +1094,6 @@ inline cudaError_t smem_attr(K kernel, int bytes) {
 }
 
 inline KArgs args_of(const ks_context *c) { return make_args(c); }
-
-// Below four CTAs per SM of a GB300 (152 SMs) a launch is latency-bound on its few
-// CTAs' serial work (measured at (2, 2^15, 10): the accumulator iNTT passes 12.1 ->
-// 10.1 us and 12.0 -> 10.8 us with one CTA per polynomial).
-constexpr int kSplitCtas = 4 * 152;
-
-template <int LOGN, int RL, int CA = 0>
-struct Launch {
-  using GTC = GeoT<LOGN, RL, 0, CA>;  // column-pass geometry (CA: alternative tile)
-  using GTR = GeoT<LOGN, RL, 1>;  // row-pass geometry
-  static constexpr int GRID_COL = GTC::LOGA == 0 ? 1 : GTC::N2 / GTC::GC;
-  static constexpr int GRID_ROW = GTR::N1 / GTR::GR;
-  static constexpr int PRO_ROW_UP = GTR::LOGA == 0 ? PRO_UP : PRO_LOAD;
-  static constexpr int PRO_ROW_DOWN = GTR::LOGA == 0 ? PRO_DOWN : PRO_LOAD;
-  // the pipelined row kernels reserve their double buffers
-  static constexpr int SMEM_KM = ROW_PIPE<LOGN, RL> ? KmSmem<GTR>::BYTES : GTR::SMEM_ROW;
-  static constexpr int SMEM_MD = ROW_PIPE<LOGN, RL> ? MdSmem<GTR>::BYTES : GTR::SMEM_ROW;
-
-  static cudaError_t prepare() {
-    cudaError_t e;
-    if ((e = smem_attr(k_inv_row<LOGN, RL>, GTR::SMEM_ROW))) return e;
-    if ((e = smem_attr(k_fwd_row_store<LOGN, RL>, GTR::SMEM_ROW))) return e;
-    if ((e = smem_attr(k_fwd_row_keymult<LOGN, RL, PRO_ROW_UP>, SMEM_KM))) return e;
-    if ((e = smem_attr(k_fwd_row_moddown<LOGN, RL, PRO_ROW_DOWN>, SMEM_MD))) return e;
-    if (GTC::LOGA > 0) {
-      if ((e = smem_attr(k_inv_col<LOGN, RL, CA>, GTC::SMEM_COL))) return e;
-      if ((e = smem_attr(k_fwd_col<LOGN, RL, PRO_LOAD, CA>, GTC::SMEM_COL))) return e;
-      if ((e = smem_attr(k_fwd_col<LOGN, RL, PRO_UP, CA>, GTC::SMEM_COL))) return e;
-      if ((e = smem_attr(k_fwd_col<LOGN, RL, PRO_DOWN, CA>, GTC::SMEM_COL))) return e;
-    }
-    return cudaSuccess;
-  }
-
-  static int count(const ks_context *c, const Tasks &tk) { return count_tasks(c, tk); }
-
-  // The accumulator P-limbs (which = 1) hold two polynomials per limb: they get one CTA
-  // each when a CTA per limb would give fewer than kSplitCtas CTAs.
-  static int inv_split(int grid, int inner, int which, int jobs) {
-    return which == 1 && grid * inner * jobs < kSplitCtas ? 1 : 0;
-  }
-
-  static cudaError_t intt_row(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
-                              cudaStream_t s) {
-    const int inner = which == 0 ? c->nq : c->np;
-    if (inner == 0 || js.n == 0) return cudaSuccess;
-    const int split = inv_split(GRID_ROW, inner, which, js.n);
-    return launch_pdl(k_inv_row<LOGN, RL>, dim3(GRID_ROW, inner << split, js.n), dim3(GTR::NT),
-                      GTR::SMEM_ROW, s, args_of(c), js, wo, which, split);
-  }
-
-  static cudaError_t intt_col_p(const ks_context *c, const JobSet &js, const WsOff &wo,
-                                int which, int pieces, cudaStream_t s) {
-    const int inner = which == 0 ? c->nq : c->np;
-    if (GTC::LOGA == 0 || inner == 0 || js.n == 0) return cudaSuccess;
-    const int split = inv_split(GRID_COL, inner, which, js.n);
-    return launch_pdl(k_inv_col<LOGN, RL, CA>, dim3(GRID_COL, inner << split, js.n), dim3(GTC::NT),
-                      GTC::SMEM_COL, s, args_of(c), js, wo, which, split, pieces);
-  }
-  static cudaError_t intt_col(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
-                              cudaStream_t s) {
-    return intt_col_p(c, js, wo, which, 0, s);
-  }
-  static cudaError_t intt_col_tc(const ks_context *c, const JobSet &js, const WsOff &wo,
-                                 int which, cudaStream_t s) {
-    return intt_col_p(c, js, wo, which, 1, s);
-  }
-
-  template <int PRO>
-  static cudaError_t col(const ks_context *c, const JobSet &js, const WsOff &wo,
-                         const Tasks &tk, int buf, cudaStream_t s) {
-    const int n = count_tasks(c, tk);
-    if (GTC::LOGA == 0 || n == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_fwd_col<LOGN, RL, PRO, CA>, dim3(GRID_COL, n, js.n), dim3(GTC::NT),
-                      GTC::SMEM_COL, s, args_of(c), js, wo, tk, buf);
-  }
-
-  static cudaError_t modup_col(const ks_context *c, const JobSet &js, const WsOff &wo,
-                               const Tasks &tk, cudaStream_t s) {
-    return col<PRO_UP>(c, js, wo, tk, BUF_TMP, s);
-  }
-
-  static cudaError_t moddown_col(const ks_context *c, const JobSet &js, const WsOff &wo,
-                                 const Tasks &tk, cudaStream_t s) {
-    return col<PRO_DOWN>(c, js, wo, tk, BUF_TMP2, s);
-  }
-
-  static cudaError_t modup_row(const ks_context *c, const JobSet &js, const WsOff &wo,
-                               const Tasks &tk, cudaStream_t s) {
-    const int n = count_tasks(c, tk);
-    if (n == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_fwd_row_keymult<LOGN, RL, PRO_ROW_UP>, dim3(GRID_ROW, n, js.n),
-                      dim3(GTR::NT), SMEM_KM, s, args_of(c), js, wo, tk);
-  }
-
-  static cudaError_t moddown_row(const ks_context *c, const JobSet &js, const WsOff &wo,
-                                 const Tasks &tk, cudaStream_t s) {
-    const int n = count_tasks(c, tk);
-    if (n == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_fwd_row_moddown<LOGN, RL, PRO_ROW_DOWN>, dim3(GRID_ROW, n, js.n),
-                      dim3(GTR::NT), SMEM_MD, s, args_of(c), js, wo, tk);
-  }
-
-  static cudaError_t ntt_col(const ks_context *c, const JobSet &js, const WsOff &wo,
-                             const Tasks &tk, int buf, cudaStream_t s) {
-    return col<PRO_LOAD>(c, js, wo, tk, buf, s);
-  }
-
-  static cudaError_t ntt_row(const ks_context *c, const JobSet &js, const WsOff &wo,
-                             const Tasks &tk, int buf, cudaStream_t s) {
-    const int n = count_tasks(c, tk);
-    if (n == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_fwd_row_store<LOGN, RL>, dim3(GRID_ROW, n, js.n), dim3(GTR::NT),
-                      GTR::SMEM_ROW, s, args_of(c), js, wo, tk, buf);
-  }
-
-  static const LaunchTable &table() {
-    static const LaunchTable t = {&prepare,     &count,       &intt_row,  &intt_col,
-                                  &intt_col_tc, &modup_col,   &modup_row, &moddown_col,
-                                  &moddown_row, &ntt_col,     &ntt_row};
-    return t;
-  }
-};
 
 }  // namespace kern
 }  // namespace ks

@@ -1,0 +1,805 @@
+// Row passes and the inverse column pass of the two-pass sizes on the register-tile core
+// (ks_core.cuh): the input and accumulator iNTTs, the key multiply, the ModDown row pass
+// and the plain forward row pass. One set of kernels per N serves every radix and column
+// tile a plan may name for these stages (a schedule's radix chooses the integer
+// basis-conversion column passes only; every schedule computes the same bits).
+#pragma once
+#include "ks_core.cuh"
+#include "ks_kern.cuh"
+
+namespace ks {
+namespace kern {
+
+// Row tile of N = 2^LOGN: GP threads, GR rows of N2 points.
+template <int LOGN, int GP_ = 64>
+struct RowGeo {
+  static constexpr int LOGA = geo_loga(LOGN), LOGB = LOGN - LOGA;
+  using SB = core::Sub<LOGB, core::row_rl(LOGN)>;
+  static constexpr int N1 = 1 << LOGA, N2 = 1 << LOGB;
+  static constexpr int GP = GP_, GR = GP / SB::T, TILE = GR * N2;
+  static constexpr int WR = 32 / SB::T;      // rows of a warp
+  static constexpr int RP = core::row_pitch<SB>();  // words of a row in shared memory
+  static constexpr int TILEW = GR * RP;      // words of a tile
+  static constexpr int TWR = N2 * GR;        // twiddle entries of a tile
+  static constexpr int TW_BYTES = TWR * 16;
+  static constexpr int GRID = N1 / GR;
+  static_assert(GRID % 4 == 0, "tiles of a CTA");
+  static_assert(SB::T <= 32, "a row inside a warp");
+};
+
+// The twiddle slab of (prime, row tile) by one bulk copy (see stage_tw); tw_ready waits.
+template <class RG>
+__device__ __forceinline__ void stage_row_tw(ulonglong2 *tws, const ulonglong2 *tab, int prime,
+                                             int blk, u64 *bar) {
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    mbar_expect_tx(bar, RG::TW_BYTES);
+    bulk_g2s(tws, tab + (((size_t)prime << RG::LOGB) << RG::LOGA) + (size_t)blk * RG::TWR,
+             RG::TW_BYTES, bar);
+  }
+}
+
+template <class RG>
+__device__ __forceinline__ void row_fwd_cls(u64 *v, u64 *s, const ulonglong2 *tw, u64 m, int t,
+                                            int cls) {
+  if (cls == CLS_FAST)
+    core::row_fwd<typename RG::SB, CLS_FAST>(v, s, tw, m, t);
+  else if (cls == CLS_MID)
+    core::row_fwd<typename RG::SB, CLS_MID>(v, s, tw, m, t);
+  else
+    core::row_fwd<typename RG::SB, CLS_EXACT>(v, s, tw, m, t);
+}
+template <class RG>
+__device__ __forceinline__ void row_inv_cls(u64 *v, u64 *s, const ulonglong2 *tw, u64 m, int t,
+                                            int cls) {
+  if (cls == CLS_FAST)
+    core::row_inv<typename RG::SB, CLS_FAST>(v, s, tw, m, t);
+  else if (cls == CLS_MID)
+    core::row_inv<typename RG::SB, CLS_MID>(v, s, tw, m, t);
+  else
+    core::row_inv<typename RG::SB, CLS_EXACT>(v, s, tw, m, t);
+}
+
+// Lane-linear 16-byte walk over a warp's own rows: pair k of lane l covers words
+// 2 (l + 32 k) of the warp's WR rows (contiguous in global memory); calls f(word offset in
+// the warp's rows, position in its shared rows).
+template <class RG, class F>
+__device__ __forceinline__ void warp_rows(F f) {
+  constexpr int W = RG::WR * RG::N2;  // words of the warp's rows
+#pragma unroll
+  for (int k = 0; k < W / 64; ++k) {
+    const int e = 2 * ((threadIdx.x & 31) + 32 * k);
+    f(e, (e >> RG::LOGB) * RG::RP + core::row_pos(e & (RG::N2 - 1)));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Inverse row pass: d -> v (which 0, one polynomial) or the P-limbs of acc -> vp (which 1,
+// both polynomials, one group of 64 threads each, sharing the twiddle slab). Canonical
+// output for the column pass. Bound by the integer pipe and the twiddle slab's traffic
+// (16 bytes per point against 8 in and 8 out).
+template <int LOGN>
+__global__ void __launch_bounds__(128, 6)
+    k_inv_row2(KArgs a, JobSet js, WsOff wo, int which) {
+  using RG = RowGeo<LOGN>;
+  using SB = typename RG::SB;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ u64 twbar;
+  ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
+  const JobPtr &jp = js.j[blockIdx.z];
+  const InttSet is = intt_set(a, jp, wo, which);
+  const int o = threadIdx.x / RG::GP, tg = threadIdx.x % RG::GP;
+  const int row = tg / SB::T, t = tg % SB::T, w0 = row / RG::WR * RG::WR;  // warp's first row
+  const int ii = blockIdx.y, prime = is.prime_base + ii, blk = blockIdx.x, r0 = blk * RG::GR;
+  u64 *tile = reinterpret_cast<u64 *>(raw + RG::TW_BYTES) + o * RG::TILEW;
+  const ModInfo &mi = a.tab.mod[prime];
+  const u64 m = mi.m, mu = mi.mu;
+  constexpr size_t N = (size_t)1 << LOGN;
+  stage_row_tw<RG>(tws, a.tab.twr_f, prime, RG::N1 / RG::GR - 1 - blk, &twbar);
+  // (see inv_row_body: an input in host memory is read without waiting for the
+  // predecessor, which is waited for at the end)
+  const bool host_in = which == 0 && jp.dsrc;
+  if (!host_in) pdl_wait();
+  const size_t off = ((size_t)(r0 + w0) << RG::LOGB);
+  const u64 *src = host_in ? jp.dsrc + (size_t)ii * N + off
+                           : is.src + ((size_t)o * is.src_outer + ii) * N + off;
+  u64 *ws = tile + w0 * RG::RP;
+  if (host_in) {
+    u64 *copy = const_cast<u64 *>(jp.d) + (size_t)ii * N + off;
+    warp_rows<RG>([&](int e, int p) {
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(src + e);
+      *reinterpret_cast<ulonglong2 *>(copy + e) = x;
+      *reinterpret_cast<ulonglong2 *>(ws + p) = x;
+    });
+  } else {
+    warp_rows<RG>([&](int e, int p) {
+      *reinterpret_cast<ulonglong2 *>(ws + p) = *reinterpret_cast<const ulonglong2 *>(src + e);
+    });
+  }
+  __syncthreads();  // the warp's rows, and the barrier's initialisation
+  tw_ready<true>(&twbar, a.tab.err);
+  u64 v[SB::E];
+  u64 *s = tile + row * RG::RP;
+  core::get_row<SB>(v, s, t);
+  row_inv_cls<RG>(v, s, tws + (size_t)(RG::GR - 1 - row) * RG::N2, m, t, mod_class(m));
+  u64 *d = is.dst + ((size_t)o * is.dst_outer + ii) * N + ((size_t)(r0 + row) << RG::LOGB);
+#pragma unroll
+  for (int u = 0; u < SB::E; ++u) d[(u << SB::LOGT) + t] = reduce_full(v[u], m, mu);
+  if (host_in) pdl_wait();
+  pdl_trigger();
+}
+
+// ---------------------------------------------------------------------------
+// Inverse column pass, in place, with the per-limb scale; `pieces` writes the bf16 bytes
+// of the result for the tensor-core conversion instead (see store_pieces). Both
+// polynomials of which = 1 run side by side.
+template <int LOGN>
+struct ColGeo {
+  static constexpr int LOGA = geo_loga(LOGN), LOGB = LOGN - LOGA;
+  static constexpr int N1 = 1 << LOGA, N2 = 1 << LOGB;
+  static constexpr int RL = core::col_rl(LOGN), E = 1 << RL, LOGT = LOGA - RL;
+  static constexpr int GC = 8;             // columns per tile: 64-byte row segments
+  static constexpr int GP = GC << LOGT;    // threads of a tile
+  static constexpr int TILEW = core::col_words<LOGA, GC, RL>();
+  static constexpr int KL = core::col_rounds<LOGA, RL>() - 1;  // last round
+  static constexpr int TW_BYTES = N1 * 16;
+  static constexpr int GRID = N2 / GC;
+};
+
+template <int LOGN>
+__global__ void __launch_bounds__(2 * ColGeo<LOGN>::GP, 768 / (2 * ColGeo<LOGN>::GP))
+    k_inv_col2(KArgs a, JobSet js, WsOff wo, int which, int pieces) {
+  using CG = ColGeo<LOGN>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ u64 twbar;
+  ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
+  const JobPtr &jp = js.j[blockIdx.z];
+  const InttSet is = intt_set(a, jp, wo, which);
+  const int o = threadIdx.x / CG::GP, tg = threadIdx.x % CG::GP;
+  const int g = tg % CG::GC, t = tg / CG::GC, c0 = blockIdx.x * CG::GC;
+  const int ii = blockIdx.y, prime = is.prime_base + ii;
+  u64 *tile = reinterpret_cast<u64 *>(raw + CG::TW_BYTES) + o * CG::TILEW;
+  const u64 m = a.tab.mod[prime].m;
+  if (threadIdx.x == 0) {
+    mbar_init(&twbar, 1);
+    mbar_expect_tx(&twbar, CG::TW_BYTES);
+    bulk_g2s(tws, a.tab.twc_i + ((size_t)prime << CG::LOGA), CG::TW_BYTES, &twbar);
+  }
+  pdl_wait();
+  u64 *d = is.dst + ((size_t)o * is.dst_outer + ii) * ((size_t)1 << LOGN);
+  u64 v[CG::E];
+#pragma unroll
+  for (int r = 0; r < CG::E; ++r)
+    v[r] = d[((size_t)core::ColRound<CG::LOGA, CG::RL, CG::KL>::point(t, r) << CG::LOGB) + c0 + g];
+  const ulonglong2 sc = is.scale[ii];
+  __syncthreads();  // the barrier's initialisation
+  tw_ready<true>(&twbar, a.tab.err);
+  const int cls = mod_class(m);
+  auto sync = [] { __syncthreads(); };
+  if (cls == CLS_FAST)
+    core::col_inv<CG::LOGA, CG::RL, CG::GC, CLS_FAST, CG::KL>(v, tile, tws, m, t, g, sync);
+  else if (cls == CLS_MID)
+    core::col_inv<CG::LOGA, CG::RL, CG::GC, CLS_MID, CG::KL>(v, tile, tws, m, t, g, sync);
+  else
+    core::col_inv<CG::LOGA, CG::RL, CG::GC, CLS_EXACT, CG::KL>(v, tile, tws, m, t, g, sync);
+#pragma unroll
+  for (int u = 0; u < CG::E; ++u) v[u] = csub(shoup(v[u], sc.x, sc.y, m), m);
+  const int col = c0 + g;
+  if (pieces) {
+    const size_t limb = which == 0 ? (size_t)ii : (size_t)o * a.np + ii;
+    const int lgc = a.tc_tplog - CG::LOGA;
+    u64 *pb = jp.ws + (which == 0 ? wo.pv : wo.ppv) + (limb << (LOGN + 1)) +
+              2 * (((size_t)(col >> lgc) << a.tc_tplog) + (col & ((1 << lgc) - 1)));
+#pragma unroll
+    for (int u = 0; u < CG::E; ++u)
+      *reinterpret_cast<uint4 *>(pb + ((size_t)((u << CG::LOGT) + t) << (lgc + 1))) =
+          bf16_bytes(v[u]);
+  } else {
+#pragma unroll
+    for (int u = 0; u < CG::E; ++u) d[((size_t)((u << CG::LOGT) + t) << CG::LOGB) + col] = v[u];
+  }
+  pdl_trigger();
+}
+
+// Exact sum of 64 x 64-bit products: value lo + 2^32 mid + 2^64 hi. The middle products
+// are summed on their own, so a term takes four 32x32->64 products and three 64-bit adds
+// (19 cycles a warp against 28.7 for a carry chain over the whole 128 bits). mid must stay
+// below 2^63: at most `fl` terms between two folds (mac_terms).
+struct Mac3 {
+  u64 lo, hi, mid;
+  __device__ __forceinline__ void add(u64 y, u64 k) {
+    const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
+    const uint32_t kl = (uint32_t)k, kh = (uint32_t)(k >> 32);
+    const u64 l = mul_wide(yl, kl), h = mul_wide(yh, kh);
+    mid += mul_wide(yl, kh) + mul_wide(yh, kl);
+    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(lo), "+l"(hi) : "l"(l), "l"(h));
+  }
+  __device__ __forceinline__ void fold() {
+    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;"
+        : "+l"(lo), "+l"(hi)
+        : "l"(mid << 32), "l"(mid >> 32));
+    mid = 0;
+  }
+  // value * 2^-64 mod m, canonical, for a value below m 2^64 and mid below 2^63: two 32-bit
+  // Montgomery steps (inv = m^-1 mod 2^32), each taking off u m with u the low word times
+  // inv; six products against nine and about half the instructions of fold() and a 64-bit
+  // step.
+  __device__ __forceinline__ u64 reduce(u64 m, uint32_t inv) const {
+    const uint32_t ml = (uint32_t)m, mh = (uint32_t)(m >> 32);
+    const uint32_t u0 = (uint32_t)lo * inv;
+    const long long t = (long long)(mid + (lo >> 32) - (mul_wide(u0, ml) >> 32)) -
+                        (long long)mul_wide(u0, mh);
+    const uint32_t u1 = (uint32_t)t * inv;
+    const u64 r = hi + (u64)(t >> 32) - (mul_wide(u1, ml) >> 32) - mul_wide(u1, mh) + m;
+    return csub(r, m);
+  }
+};
+// The canonical residue of a sum; exact moduli, whose mid may pass 2^63, by fold() and the
+// 64-bit step.
+__device__ __forceinline__ u64 mac_reduce(Mac3 &s, const ModInfo &mi, u64 m, uint32_t inv,
+                                          int cls) {
+  if (cls != CLS_EXACT) return s.reduce(m, inv);
+  s.fold();
+  return csub(redc(U128{s.lo, s.hi}, m, mi.minv), m);
+}
+// Terms whose middle products stay below 2^63 - 2^33 in the key multiply: 71 m + 2^33 each
+// with lazy ext (below 70 m, m < 2^51), 2 m + 2^33 otherwise (m < 2^60); exact moduli fold
+// every term.
+__device__ __forceinline__ int mac_terms(int cls) {
+  return cls == CLS_FAST ? 32 : cls == CLS_MID ? 3 : 1;
+}
+
+// Forward column tile: 8 columns, 8 points per thread.
+template <int LOGN>
+struct FwdColGeo {
+  static constexpr int LOGA = geo_loga(LOGN), LOGB = LOGN - LOGA;
+  static constexpr int N1 = 1 << LOGA, N2 = 1 << LOGB;
+  static constexpr int RL = 3, E = 8, GC = 8, GP = GC * N1 / E;
+  static constexpr int TILEW = core::col_words<LOGA, GC, RL>();
+  static constexpr int TW_BYTES = N1 * 16;
+  static constexpr int GRID = N2 / GC, SMEM = TW_BYTES + TILEW * 8;
+};
+
+// ---------------------------------------------------------------------------
+// Forward column pass: the integer basis conversion of a task (PRO_UP, PRO_DOWN) or a plain
+// load (PRO_LOAD, in place), then the first forward NTT pass on the thread's eight points.
+// The conversion's sums are exact (Mac3), four points at a time, and reduced in registers;
+// the tile in shared memory is only the NTT's exchange. Bound by the integer pipe.
+template <int LOGN, int PRO>
+__global__ void __launch_bounds__(FwdColGeo<LOGN>::GP, 768 / FwdColGeo<LOGN>::GP)
+    k_fwd_col2(KArgs a, JobSet js, WsOff wo, Tasks tk, int buf) {
+  using CG = FwdColGeo<LOGN>;
+  using C0 = core::ColRound<CG::LOGA, CG::RL, 0>;
+  using CL = core::ColRound<CG::LOGA, CG::RL, core::col_rounds<CG::LOGA, CG::RL>() - 1>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ u64 twbar;
+  ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
+  u64 *tile = reinterpret_cast<u64 *>(raw + CG::TW_BYTES);
+  const u64 *src;
+  u64 *dst;
+  fwd_bufs<PRO>(js.j[blockIdx.z], wo, buf, src, dst);
+  const uint32_t w = decode(a, tk, blockIdx.y);
+  const int tgt = task_limb(w), dig = task_dig(w);
+  const int g = threadIdx.x % CG::GC, t = threadIdx.x / CG::GC, c0 = blockIdx.x * CG::GC;
+  if (threadIdx.x == 0) {
+    mbar_init(&twbar, 1);
+    mbar_expect_tx(&twbar, CG::TW_BYTES);
+    bulk_g2s(tws, a.tab.twc_f + ((size_t)tgt << CG::LOGA), CG::TW_BYTES, &twbar);
+  }
+  const ModInfo &mi = a.tab.mod[tgt];
+  const u64 m = mi.m;
+  const int cls = mod_class(m);
+  dst += ((size_t)task_slot(w) << LOGN) + c0 + g;
+  u64 v[CG::E];
+  if constexpr (PRO == PRO_LOAD) {
+    pdl_wait();
+#pragma unroll
+    for (int r = 0; r < CG::E; ++r) v[r] = dst[(size_t)C0::point(t, r) << CG::LOGB];
+  } else {
+    // sources: digit dig's limbs of v, or polynomial dig's P-limbs of vp
+    const int i0 = dig * (PRO == PRO_UP ? a.alpha : a.np);
+    const int ns = PRO == PRO_UP ? min(a.nq, i0 + a.alpha) - i0 : a.np;
+    const u64 *cst = PRO == PRO_UP ? a.tab.cup + ((size_t)dig * a.qp + tgt) * a.alpha
+                                   : a.tab.cdown + (size_t)tgt * a.alpha;
+    // run: terms of one reduction (their sum below m 2^64); fl: terms whose middle products
+    // stay below 2^63: source + m + 2^33 each
+    const int run = PRO == PRO_UP ? a.run_up : a.run_down;
+    const int fl = min(run, cls == CLS_FAST && run >= (1 << 13) ? 1 << 10 : run >= 16 ? 3 : 1);
+    const bool exact = cls == CLS_EXACT || run < 16;  // a modulus or source above 2^60
+    const uint32_t inv = 0u - (uint32_t)mi.minv;
+    src += ((size_t)i0 << LOGN) + c0 + g;
+    pdl_wait();
+    constexpr int H = 4;  // points per batch (bounds the live registers)
+#pragma unroll
+    for (int h = 0; h < CG::E; h += H) {
+      Mac3 s[H] = {};
+      u64 x[H];
+#pragma unroll
+      for (int k = 0; k < H; ++k) x[k] = src[(size_t)C0::point(t, h + k) << CG::LOGB];
+      u64 c = __ldg(cst);
+      bool one = true;  // no reduction yet
+      int left = run, fold = fl;
+#pragma unroll 1
+      for (int i = 0; i < ns; ++i) {
+        u64 xn[H], cn = 0;
+        if (i + 1 < ns) {  // the next limb's loads before this one's products
+          const u64 *sn = src + ((size_t)(i + 1) << LOGN);
+#pragma unroll
+          for (int k = 0; k < H; ++k) xn[k] = sn[(size_t)C0::point(t, h + k) << CG::LOGB];
+          cn = __ldg(cst + i + 1);
+        }
+#pragma unroll
+        for (int k = 0; k < H; ++k) s[k].add(x[k], c);
+        --left;
+        if (--fold == 0 || left == 0 || i == ns - 1) {
+          fold = fl;
+          if (left == 0 || i == ns - 1) {
+            left = run;
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+              const u64 z = mac_reduce(s[k], mi, m, inv, exact ? CLS_EXACT : cls);
+              v[h + k] = one ? z : csub(v[h + k] + z, m);
+              s[k] = Mac3{};
+            }
+            one = false;
+          } else {
+#pragma unroll
+            for (int k = 0; k < H; ++k) s[k].fold();
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < H; ++k) x[k] = xn[k];
+        c = cn;
+      }
+    }
+  }
+  __syncthreads();  // the barrier's initialisation
+  tw_ready<true>(&twbar, a.tab.err);
+  auto sync = [] { __syncthreads(); };
+  if (cls == CLS_FAST)
+    core::col_fwd<CG::LOGA, CG::RL, CG::GC, CLS_FAST, 0>(v, tile, tws, m, t, g, sync);
+  else if (cls == CLS_MID)
+    core::col_fwd<CG::LOGA, CG::RL, CG::GC, CLS_MID, 0>(v, tile, tws, m, t, g, sync);
+  else
+    core::col_fwd<CG::LOGA, CG::RL, CG::GC, CLS_EXACT, 0>(v, tile, tws, m, t, g, sync);
+#pragma unroll
+  for (int r = 0; r < CG::E; ++r) dst[(size_t)CL::point(t, r) << CG::LOGB] = v[r];
+  pdl_trigger();
+}
+
+// ---------------------------------------------------------------------------
+// Plain forward row pass (keygen, unfused plans): canonical result back in place.
+template <int LOGN>
+__global__ void __launch_bounds__(64)
+    k_row_store2(KArgs a, JobSet js, WsOff wo, Tasks tk, int buf) {
+  using RG = RowGeo<LOGN>;
+  using SB = typename RG::SB;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ u64 twbar;
+  ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
+  u64 *tile = reinterpret_cast<u64 *>(raw + RG::TW_BYTES);
+  const int row = threadIdx.x / SB::T, t = threadIdx.x % SB::T, w0 = row / RG::WR * RG::WR;
+  const u64 *src;
+  u64 *dst;
+  fwd_bufs<PRO_LOAD>(js.j[blockIdx.z], wo, buf, src, dst);
+  const uint32_t w = decode(a, tk, blockIdx.y);
+  const int p = task_limb(w), blk = blockIdx.x, r0 = blk * RG::GR;
+  const ModInfo &mi = a.tab.mod[p];
+  const u64 m = mi.m, mu = mi.mu;
+  stage_row_tw<RG>(tws, a.tab.twr_f, p, blk, &twbar);
+  pdl_wait();
+  u64 *b = dst + ((size_t)task_slot(w) << LOGN);
+  u64 v[SB::E];
+#pragma unroll
+  for (int u = 0; u < SB::E; ++u)
+    v[u] = b[((size_t)(r0 + row) << RG::LOGB) + (u << SB::LOGT) + t];
+  __syncthreads();
+  tw_ready<true>(&twbar, a.tab.err);
+  u64 *s = tile + row * RG::RP;
+  row_fwd_cls<RG>(v, s, tws + row * RG::N2, m, t, mod_class(m));
+  __syncwarp();
+  core::put_row<SB>(s, v, t);
+  __syncwarp();
+  const u64 *ws = tile + w0 * RG::RP;
+  u64 *o = b + ((size_t)(r0 + w0) << RG::LOGB);
+  warp_rows<RG>([&](int e, int q) {
+    ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(ws + q);
+    x.x = reduce_full(x.x, m, mu);
+    x.y = reduce_full(x.y, m, mu);
+    *reinterpret_cast<ulonglong2 *>(o + e) = x;
+  });
+  pdl_trigger();
+}
+
+// ---------------------------------------------------------------------------
+// Key multiply (TASK_TARGET): one CTA = one row tile of one target limb t, all its digits:
+//   acc_c[t] (+)= sum_j ext_j[t] * evk[j][c][t],  c = 0, 1.
+// Groups of kKmGp threads transform one digit's tile each, side by side on one twiddle slab,
+// and leave ext in shared memory; after one barrier every thread multiplies its points by
+// the key words of all digits (read once, 16 bytes a lane, pulled into L2 by the TMA unit
+// while the digits are transformed) with exact 128-bit sums and one REDC per output word.
+// The CTA's own digit (t's limb inside the digit) is the input itself, put in Montgomery
+// form. Up to `ds` digits fit at a time; more are taken in turns, the accumulators
+// re-read.
+constexpr int kKmDigits = 10;   // most digits of a tile held in shared memory
+constexpr int kKmGroups = 4;    // most groups of threads (one tile each)
+
+// A warp per digit's tile of two 256-point rows (one of 512) at N >= 2^16, two warps per
+// tile of 512 points below: small CTAs, so that several of them mix their transform and
+// multiply phases on an SM. (Several tiles per CTA at one or two digits: 21 -> 23 us per
+// digit launch of (4, 2^16, 35) in four chunks, not kept.)
+__host__ __device__ constexpr int km_gp(int logn) { return logn >= 16 ? 32 : 64; }
+
+template <int LOGN>
+__global__ void __launch_bounds__(km_gp(LOGN) * kKmGroups, 768 / (km_gp(LOGN) * kKmGroups))
+    k_keymult2(KArgs a, JobSet js, WsOff wo, Tasks tk, int ds) {
+  using RG = RowGeo<LOGN, km_gp(LOGN)>;
+  using SB = typename RG::SB;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ u64 twbar;
+  ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
+  u64 *ext = reinterpret_cast<u64 *>(raw + RG::TW_BYTES);
+  const JobPtr &jp = js.j[blockIdx.z];
+  const int grp = threadIdx.x / RG::GP, ngrp = blockDim.x / RG::GP, tg = threadIdx.x % RG::GP;
+  const int row = tg / SB::T, t = tg % SB::T, w0 = row / RG::WR * RG::WR;
+  // targets in reverse: the P-limb targets, listed last, transform every digit (a Q-limb
+  // target's own digit needs no transform), so they start first
+  const int tgt = tk.t0 + (gridDim.y - 1 - blockIdx.y);
+  const ModInfo &mi = a.tab.mod[tgt];
+  const u64 m = mi.m;
+  const uint32_t inv = 0u - (uint32_t)mi.minv;  // m^-1 mod 2^32
+  const int blk = blockIdx.x, off0 = blk * RG::TILE;
+  const int od = tgt < a.nq ? tgt / a.alpha : -1;  // the target's own digit
+  const int nd = tk.j1 - tk.j0;
+  // the tile's key words: digit j, polynomial c at (2j + c) eqp N words further
+  const u64 *evk = jp.evk + ((size_t)(tgt < a.nq ? tgt : a.epb + (tgt - a.nq)) << LOGN) + off0;
+  for (int k = threadIdx.x; k < 2 * nd; k += blockDim.x)
+    prefetch_l2(evk + ((size_t)((2 * tk.j0 + k) * a.eqp) << LOGN), RG::TILE * 8);
+  stage_row_tw<RG>(tws, a.tab.twr_f, tgt, blk, &twbar);
+  const int cls = mod_class(m), fl = mac_terms(cls);
+  // ext stays lazy when the exact digit sum of its products fits one reduction
+  const bool lazy = cls == CLS_FAST && __umul64hi(kFwdLazy * min(nd, ds), m) == 0;
+  pdl_wait();
+  __syncthreads();  // the twiddle barrier's initialisation
+  for (int c0 = tk.j0; c0 < tk.j1; c0 += ds) {
+    const int n = min(ds, tk.j1 - c0);
+    const int oc = od - c0;  // the own digit's index in this turn, if any
+    const bool has = oc >= 0 && oc < n;
+    for (int jj = grp; jj < n; jj += ngrp) {
+      // the digits to transform first, the own digit (cheap) last
+      const int jx = !has ? jj : jj == n - 1 ? oc : jj < oc ? jj : jj + 1;
+      u64 *ex = ext + jx * RG::TILEW;
+      if (has && jx == oc) {
+        const u64 *dt = jp.d + ((size_t)tgt << LOGN) + off0 + (w0 << RG::LOGB);
+        u64 *ws = ex + w0 * RG::RP;
+        const u64 r1 = mi.r1, r1s = mi.r1s;
+        warp_rows<RG>([&](int e, int p) {
+          ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(dt + e);
+          if (lazy) {
+            x.x = shoup4(x.x, r1, r1s, m);  // [0, 4m)
+            x.y = shoup4(x.y, r1, r1s, m);
+          } else {
+            x.x = csub(shoup(x.x, r1, r1s, m), m);
+            x.y = csub(shoup(x.y, r1, r1s, m), m);
+          }
+          *reinterpret_cast<ulonglong2 *>(ws + p) = x;
+        });
+        continue;
+      }
+      const int j = c0 + jx;
+      const u64 *src = jp.ws + wo.tmp +
+                       ((size_t)(j * tk.sm.sj + tgt * tk.sm.st + tk.sm.base) << LOGN) + off0 +
+                       (row << RG::LOGB) + t;
+      u64 v[SB::E];
+#pragma unroll
+      for (int u = 0; u < SB::E; ++u) v[u] = src[u << SB::LOGT];
+      tw_ready<true>(&twbar, a.tab.err);
+      u64 *s = ex + row * RG::RP;
+      row_fwd_cls<RG>(v, s, tws + row * RG::N2, m, t, cls);
+      if (!lazy) {
+        const u64 mu = mi.mu;
+#pragma unroll
+        for (int r = 0; r < SB::E; ++r) v[r] = fwd_canon(v[r], m, mu, cls);
+      }
+      __syncwarp();
+      core::put_row<SB>(s, v, t);
+    }
+    // Multiply: this thread's pairs of points in turn, each over the turn's digits, as one
+    // loop of (pair, digit) steps. The next step's key words (and at a new pair the old
+    // accumulators) are loaded before a step's products, the first ones before the barrier.
+    const u64 pol = l2_stream();
+    const bool first = tk.first && c0 == tk.j0;
+    const size_t cst = (size_t)a.eqp << LOGN;  // words between a digit's two polynomials
+    const int bd = blockDim.x;
+    const u64 *kp = evk + c0 * 2 * cst + 2 * threadIdx.x;
+    u64 *o = jp.ws + wo.acc + ((size_t)tgt << LOGN) + off0 + 2 * threadIdx.x;
+    const size_t oc1 = (size_t)a.qp << LOGN;  // to polynomial 1's accumulators
+    ulonglong2 na = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp), pol);
+    ulonglong2 nb = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp + cst), pol);
+    ulonglong2 no0 = {}, no1 = {}, old0 = {}, old1 = {};
+    if (!first) {
+      no0 = *reinterpret_cast<const ulonglong2 *>(o);
+      no1 = *reinterpret_cast<const ulonglong2 *>(o + oc1);
+    }
+    __syncthreads();
+    tw_ready<true>(&twbar, a.tab.err);  // (a CTA with no digit to transform, too)
+    Mac3 s[4] = {};
+    int jj = 0, fold = fl;
+    for (int e = 2 * threadIdx.x; e < RG::TILE;) {
+      const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(
+          ext + jj * RG::TILEW + (e >> RG::LOGB) * RG::RP + core::row_pos(e & (RG::N2 - 1)));
+      const ulonglong2 ka = na, kb = nb;
+      if (jj == 0) old0 = no0, old1 = no1;
+      const bool last = jj == n - 1;
+      kp += last ? (long long)(2 * bd) - (long long)((n - 1) * 2 * cst) : (long long)(2 * cst);
+      if (!last || e + 2 * bd < RG::TILE) {
+        na = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp), pol);
+        nb = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp + cst), pol);
+        if (last && !first) {
+          no0 = *reinterpret_cast<const ulonglong2 *>(o + 2 * bd);
+          no1 = *reinterpret_cast<const ulonglong2 *>(o + 2 * bd + oc1);
+        }
+      }
+      s[0].add(y.x, ka.x);
+      s[1].add(y.y, ka.y);
+      s[2].add(y.x, kb.x);
+      s[3].add(y.y, kb.y);
+      if (last) {
+        u64 r[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          r[i] = mac_reduce(s[i], mi, m, inv, cls);
+          s[i] = Mac3{};
+        }
+        if (!first) {
+          r[0] = addmod(r[0], old0.x, m);
+          r[1] = addmod(r[1], old0.y, m);
+          r[2] = addmod(r[2], old1.x, m);
+          r[3] = addmod(r[3], old1.y, m);
+        }
+        *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(r[0], r[1]);
+        *reinterpret_cast<ulonglong2 *>(o + oc1) = make_ulonglong2(r[2], r[3]);
+        o += 2 * bd;
+        e += 2 * bd;
+        jj = 0;
+        fold = fl;
+      } else {
+        ++jj;
+        if (--fold == 0) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s[i].fold();
+          fold = fl;
+        }
+      }
+    }
+    if (c0 + ds < tk.j1) __syncthreads();  // ext is free for the next turn
+  }
+  pdl_trigger();
+}
+
+// ---------------------------------------------------------------------------
+// ModDown row pass with the final scaling (TASK_DOWN1):
+//   out_c[i] = (acc_c[i] - NTT(BConv_{P->Q}(c))[i]) * P^-1 mod q_i (+ addend),
+// the two polynomials of limb i side by side in two groups of 64 threads that share the
+// twiddle slab; each warp finishes its own rows (no block barrier after the start).
+template <int LOGN>
+__global__ void __launch_bounds__(128, 6)
+    k_moddown2(KArgs a, JobSet js, WsOff wo, Tasks tk) {
+  using RG = RowGeo<LOGN>;
+  using SB = typename RG::SB;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ u64 twbar;
+  ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
+  const JobPtr &jp = js.j[blockIdx.z];
+  // host-buffer operation: see k_fwd_row_moddown
+  if (jp.dsrc) pdl_trigger();
+  const int c = threadIdx.x / RG::GP, tg = threadIdx.x % RG::GP;
+  const int row = tg / SB::T, t = tg % SB::T, w0 = row / RG::WR * RG::WR;
+  const uint32_t w = decode(a, tk, blockIdx.y);
+  const int i = task_limb(w), blk = blockIdx.x, r0 = blk * RG::GR;
+  u64 *tile = reinterpret_cast<u64 *>(raw + RG::TW_BYTES) + c * RG::TILEW;
+  const u64 m = a.tab.mod[i].m;
+  const ulonglong2 pv = a.tab.pinv[i];
+  constexpr size_t N = (size_t)1 << LOGN;
+  stage_row_tw<RG>(tws, a.tab.twr_f, i, blk, &twbar);
+  const int cls = mod_class(m);
+  const bool fast = cls == CLS_FAST;
+  const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
+  pdl_wait();
+  const size_t woff = (size_t)(r0 + w0) << RG::LOGB;  // the warp's rows
+  const u64 *ac = jp.ws + wo.acc + ((size_t)c * a.qp + i) * N + woff;
+  u64 v[SB::E];
+  {
+    const u64 *src = jp.ws + wo.tmp2 + (size_t)(task_slot(w) + c * tk.span) * N +
+                     ((size_t)(r0 + row) << RG::LOGB) + t;
+#pragma unroll
+    for (int u = 0; u < SB::E; ++u) v[u] = src[u << SB::LOGT];
+  }
+  if ((threadIdx.x & 31) == 0) prefetch_l2(ac, RG::WR * RG::N2 * 8);
+  __syncthreads();  // the twiddle barrier's initialisation
+  tw_ready<true>(&twbar, a.tab.err);
+  u64 *s = tile + row * RG::RP;
+  row_fwd_cls<RG>(v, s, tws + row * RG::N2, m, t, cls);
+  __syncwarp();
+  core::put_row<SB>(s, v, t);
+  __syncwarp();
+  const u64 *ws = tile + w0 * RG::RP;
+  const size_t ob = ((size_t)c * a.nq + i) * N + woff;
+  const bool add = (jp.addmask >> c) & 1;
+  // the NTT output z enters lazy, as in moddown_body
+  warp_rows<RG>([&](int e, int q) {
+    const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(ws + q);
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(ac + e);
+    const u64 z0 = fast ? z.x : csub(z.x, zs), z1 = fast ? z.y : csub(z.y, zs);
+    ulonglong2 r;
+    r.x = csub(shoup(x.x + zb - z0, pv.x, pv.y, m), m);
+    r.y = csub(shoup(x.y + zb - z1, pv.x, pv.y, m), m);
+    if (add) {
+      const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(jp.add + ob + e);
+      r.x = addmod(r.x, y.x, m);
+      r.y = addmod(r.y, y.y, m);
+    }
+    *reinterpret_cast<ulonglong2 *>(jp.out + ob + e) = r;
+  });
+  pdl_trigger();
+}
+
+// ---------------------------------------------------------------------------
+// Launchers of one two-pass N.
+template <int LOGN>
+struct RowFns {
+  using RG = RowGeo<LOGN>;
+  using KG = RowGeo<LOGN, km_gp(LOGN)>;  // the key multiply's tile
+  using CG = ColGeo<LOGN>;
+  using FG = FwdColGeo<LOGN>;
+  static constexpr int smem_row(int tiles) { return RG::TW_BYTES + tiles * RG::TILEW * 8; }
+  static constexpr int smem_km(int ds) { return KG::TW_BYTES + ds * KG::TILEW * 8; }
+  static constexpr int smem_col(int tiles) { return CG::TW_BYTES + tiles * CG::TILEW * 8; }
+
+  static cudaError_t prepare() {
+    cudaError_t e;
+    if ((e = smem_attr(k_inv_row2<LOGN>, smem_row(2)))) return e;
+    if ((e = smem_attr(k_inv_col2<LOGN>, smem_col(2)))) return e;
+    if ((e = smem_attr(k_fwd_col2<LOGN, PRO_LOAD>, FG::SMEM))) return e;
+    if ((e = smem_attr(k_fwd_col2<LOGN, PRO_UP>, FG::SMEM))) return e;
+    if ((e = smem_attr(k_fwd_col2<LOGN, PRO_DOWN>, FG::SMEM))) return e;
+    if ((e = smem_attr(k_row_store2<LOGN>, smem_row(1)))) return e;
+    if ((e = smem_attr(k_keymult2<LOGN>, smem_km(kKmDigits)))) return e;
+    return smem_attr(k_moddown2<LOGN>, smem_row(2));
+  }
+  static cudaError_t intt_row(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
+                              cudaStream_t s) {
+    const int inner = which == 0 ? c->nq : c->np, tiles = which + 1;
+    if (inner == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_inv_row2<LOGN>, dim3(RG::GRID, inner, js.n), dim3(RG::GP * tiles),
+                      smem_row(tiles), s, args_of(c), js, wo, which);
+  }
+  static cudaError_t col(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
+                         int pieces, cudaStream_t s) {
+    const int inner = which == 0 ? c->nq : c->np, tiles = which + 1;
+    if (inner == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_inv_col2<LOGN>, dim3(CG::GRID, inner, js.n), dim3(CG::GP * tiles),
+                      smem_col(tiles), s, args_of(c), js, wo, which, pieces);
+  }
+  static cudaError_t intt_col(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
+                              cudaStream_t s) {
+    return col(c, js, wo, which, 0, s);
+  }
+  static cudaError_t intt_col_tc(const ks_context *c, const JobSet &js, const WsOff &wo,
+                                 int which, cudaStream_t s) {
+    return col(c, js, wo, which, 1, s);
+  }
+  template <int PRO>
+  static cudaError_t fwd_col(const ks_context *c, const JobSet &js, const WsOff &wo,
+                             const Tasks &tk, int buf, cudaStream_t s) {
+    const int n = count_tasks(c, tk);
+    if (n == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_fwd_col2<LOGN, PRO>, dim3(FG::GRID, n, js.n), dim3(FG::GP), FG::SMEM, s,
+                      args_of(c), js, wo, tk, buf);
+  }
+  static cudaError_t modup_col(const ks_context *c, const JobSet &js, const WsOff &wo,
+                               const Tasks &tk, cudaStream_t s) {
+    return fwd_col<PRO_UP>(c, js, wo, tk, BUF_TMP, s);
+  }
+  static cudaError_t moddown_col(const ks_context *c, const JobSet &js, const WsOff &wo,
+                                 const Tasks &tk, cudaStream_t s) {
+    return fwd_col<PRO_DOWN>(c, js, wo, tk, BUF_TMP2, s);
+  }
+  static cudaError_t ntt_col(const ks_context *c, const JobSet &js, const WsOff &wo,
+                             const Tasks &tk, int buf, cudaStream_t s) {
+    return fwd_col<PRO_LOAD>(c, js, wo, tk, buf, s);
+  }
+  static cudaError_t modup_row(const ks_context *c, const JobSet &js, const WsOff &wo,
+                               const Tasks &tk, cudaStream_t s) {
+    const int n = count_tasks(c, tk), nd = tk.j1 - tk.j0;
+    if (n == 0 || js.n == 0 || nd < 1) return cudaSuccess;
+    const int turns = (nd + kKmDigits - 1) / kKmDigits, ds = (nd + turns - 1) / turns;
+    return launch_pdl(k_keymult2<LOGN>, dim3(KG::GRID, n, js.n),
+                      dim3(KG::GP * std::min(ds, kKmGroups)), smem_km(ds), s,
+                      args_of(c), js, wo, tk, ds);
+  }
+  static cudaError_t moddown_row(const ks_context *c, const JobSet &js, const WsOff &wo,
+                                 const Tasks &tk, cudaStream_t s) {
+    const int n = count_tasks(c, tk);
+    if (n == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_moddown2<LOGN>, dim3(RG::GRID, n, js.n), dim3(RG::GP * 2), smem_row(2), s,
+                      args_of(c), js, wo, tk);
+  }
+  static cudaError_t ntt_row(const ks_context *c, const JobSet &js, const WsOff &wo,
+                             const Tasks &tk, int buf, cudaStream_t s) {
+    const int n = count_tasks(c, tk);
+    if (n == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_row_store2<LOGN>, dim3(RG::GRID, n, js.n), dim3(RG::GP), smem_row(1), s,
+                      args_of(c), js, wo, tk, buf);
+  }
+  static const LaunchTable &table() {
+    static const LaunchTable t = {&prepare,     &count_tasks, &intt_row,  &intt_col,
+                                  &intt_col_tc, &modup_col,   &modup_row, &moddown_col,
+                                  &moddown_row, &ntt_col,     &ntt_row};
+    return t;
+  }
+};
+
+// Launchers of a single-pass size (N <= 2^12): the shared-memory tile rounds of radix RL.
+template <int LOGN, int RL>
+struct LaunchOne {
+  using GTR = GeoT<LOGN, RL, 1>;
+
+  static cudaError_t prepare() {
+    cudaError_t e;
+    if ((e = smem_attr(k_inv_row<LOGN, RL>, GTR::SMEM_ROW))) return e;
+    if ((e = smem_attr(k_fwd_row_store<LOGN, RL>, GTR::SMEM_ROW))) return e;
+    if ((e = smem_attr(k_fwd_row_keymult<LOGN, RL, PRO_UP>, GTR::SMEM_ROW))) return e;
+    return smem_attr(k_fwd_row_moddown<LOGN, RL, PRO_DOWN>, GTR::SMEM_ROW);
+  }
+  static cudaError_t intt_row(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
+                              cudaStream_t s) {
+    const int inner = which == 0 ? c->nq : c->np;
+    if (inner == 0 || js.n == 0) return cudaSuccess;
+    // the accumulator P-limbs hold two polynomials: one CTA each (a launch is a few CTAs)
+    return launch_pdl(k_inv_row<LOGN, RL>, dim3(1, inner << which, js.n), dim3(GTR::NT),
+                      GTR::SMEM_ROW, s, args_of(c), js, wo, which, which);
+  }
+  static cudaError_t no_col(const ks_context *, const JobSet &, const WsOff &, int,
+                            cudaStream_t) {
+    return cudaSuccess;
+  }
+  static cudaError_t no_col_task(const ks_context *, const JobSet &, const WsOff &,
+                                 const Tasks &, cudaStream_t) {
+    return cudaSuccess;
+  }
+  static cudaError_t no_ntt_col(const ks_context *, const JobSet &, const WsOff &,
+                                const Tasks &, int, cudaStream_t) {
+    return cudaSuccess;
+  }
+  static cudaError_t modup_row(const ks_context *c, const JobSet &js, const WsOff &wo,
+                               const Tasks &tk, cudaStream_t s) {
+    const int n = count_tasks(c, tk);
+    if (n == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_fwd_row_keymult<LOGN, RL, PRO_UP>, dim3(1, n, js.n), dim3(GTR::NT),
+                      GTR::SMEM_ROW, s, args_of(c), js, wo, tk);
+  }
+  static cudaError_t moddown_row(const ks_context *c, const JobSet &js, const WsOff &wo,
+                                 const Tasks &tk, cudaStream_t s) {
+    const int n = count_tasks(c, tk);
+    if (n == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_fwd_row_moddown<LOGN, RL, PRO_DOWN>, dim3(1, n, js.n), dim3(GTR::NT),
+                      GTR::SMEM_ROW, s, args_of(c), js, wo, tk);
+  }
+  static cudaError_t ntt_row(const ks_context *c, const JobSet &js, const WsOff &wo,
+                             const Tasks &tk, int buf, cudaStream_t s) {
+    const int n = count_tasks(c, tk);
+    if (n == 0 || js.n == 0) return cudaSuccess;
+    return launch_pdl(k_fwd_row_store<LOGN, RL>, dim3(1, n, js.n), dim3(GTR::NT), GTR::SMEM_ROW,
+                      s, args_of(c), js, wo, tk, buf);
+  }
+  static const LaunchTable &table() {
+    static const LaunchTable t = {&prepare,     &count_tasks, &intt_row,    &no_col,
+                                  &no_col,      &no_col_task, &modup_row,   &no_col_task,
+                                  &moddown_row, &no_ntt_col,  &ntt_row};
+    return t;
+  }
+};
+
+}  // namespace kern
+}  // namespace ks

@@ -1,44 +1,49 @@
 // Fast basis conversion (the ModUp and ModDown BConv of Sec. II-A) on the tensor cores
 // (tcgen05, sm_103a), fused with the first forward NTT pass.
 //
-// The conversion of one column tile is an integer matrix product,
-//   S[p][t] = sum_i x_i[p] * c_i[t]    (x_i < 2^62 source residues, c_i < 2^62 constants),
-// that must be exact (128 bits) before its one Montgomery reduction. It runs on the
-// bf16 tensor cores exactly by splitting both operands into bytes:
-//   x_i = sum_a x_ia 2^(8a),  c_i = sum_b c_ib 2^(8b)   (a, b = 0..7),
-//   S = sum_s v_s 2^(8s),  v_s = sum_i sum_{a+b=s} x_ia c_ib   (s = 0..14).
-// Bytes are exact in bf16, every product x_ia c_ib < 2^16 is exact in the fp32
-// accumulator, and v_s <= 16 * 8 * 255^2 < 2^23 for at most 16 sources, so every
-// partial sum is an exact fp32 integer whatever the summation order. The MMA computes
-// all v_s at once as D[p][(t, s)] = sum_(i, a) A[p][(i, a)] B[(i, a)][(t, s)] with
-// A[p][(i, a)] = x_ia (the bytes of the sources, K = 8 per source limb) and the
-// Toeplitz-shaped constant B[(i, a)][(t, s)] = c_i[t]_(s-a) (zero outside 0..7). One
+// The conversion of one column tile is the integer matrix product
+//   S[p][t] = sum_i x_i[p] * c_i[t] mod m_t   (x_i < 2^62 source residues, constants c_i[t]).
+// It runs on the bf16 tensor cores exactly by splitting both operands into bytes, the
+// sources as x_i = sum_a x_ia 2^(8a) and, for each byte a, the constant
+// c_ia[t] = c_i[t] 2^(8a) mod m_t = sum_b c_iab 2^(8b)   (a, b = 0..7):
+//   S = sum_b v_b 2^(8b),  v_b = sum_i sum_a x_ia c_iab   (b = 0..7).
+// Bytes are exact in bf16, every product x_ia c_iab < 2^16 is exact in the fp32
+// accumulator, and v_b <= 16 * 8 * 255^2 < 2^23 for at most 16 sources, so every
+// partial sum is an exact fp32 integer whatever the summation order. Reducing each
+// shifted constant first keeps S below 2^15 m_t: eight accumulators per target instead of
+// the fifteen of the full 128-bit byte product, and one 32-bit Montgomery step (S 2^-32,
+// the constants carry 2^32) instead of a 64-bit one; per converted word that is 4
+// 32x32->64 products against 9 and about half the instructions. The MMA computes all v_b
+// at once as D[p][(t, b)] = sum_(i, a) A[p][(i, a)] B[(i, a)][(t, b)]. One
 // more K row adds 2^23 to every accumulator (A = 1, B = 2^23): the fp32 bits of
-// 2^23 + v_s are then 0x4B000000 + v_s, and v_s needs no float-to-integer conversion.
+// 2^23 + v_b are then 0x4B000000 + v_b, and v_b needs no float-to-integer conversion.
 //
 // Layout (no swizzle, K-major core matrices of 8 rows x 16 bytes):
 //  A  [k < ap][p < TP][8 bf16]     the bytes of source limb k at point p (16 bytes): K
 //     direction stride TP*16 bytes (LBO), M direction 128 bytes (SBO). Written by the
-//     inverse column pass (store_pieces), copied per tile with one bulk copy per limb.
-//  B  [u < 2][g < 2][k < ap][r < 8][8 bf16] per target pair: target u, output slots
-//     s = 8g + r, limb k; K stride 128 bytes (LBO), N stride ap*128 bytes (SBO). A
-//     constant table per (digit, target) / target, built with the context.
-//  D  TMEM lane p (of a 128-point M block), column (u, s): one accumulator of
-//     (TP / 128) x 32 columns per consumer group, so the MMAs of one group's next pair
-//     run while the other group recombines and transforms its own.
+//     inverse column pass, copied per tile with one bulk copy per limb.
+//  B  [u < 4][k < ap][b < 8][8 bf16] per target group: target u, byte b, limb k; K stride
+//     128 bytes (LBO), N stride ap*128 bytes (SBO). A constant table per (digit, target) /
+//     target, built with the context.
+//  D  TMEM lane p (of a 128-point M block), column (u, b): one accumulator of
+//     (TP / 128) x 32 columns per consumer group, so the MMAs of one group's next item
+//     run while the other group reduces and transforms its own.
 //
-// One CTA per SM walks a contiguous range of (column tile, target pair) items; the
+// One CTA per SM walks a contiguous range of (column tile, target group) items; the
 // bytes of a tile's sources stay in shared memory while the CTA converts them onto
-// successive pairs of targets. Roles: one issuer thread (its own warp) copies the
+// successive groups of four targets. Roles: one issuer thread (its own warp) copies the
 // tile's source bytes and issues the MMAs (completion on mbarriers through
 // tcgen05.commit); a loader warp decodes each item's targets (a lane per target) and
 // copies their constants an item ahead, off the issuer's path; two consumer groups
-// take the items in turn: each reads its lanes' 16 sums per target from TMEM,
-// recombines them into the exact 128-bit S, applies REDC and writes the tiles, then its
-// two halves run the column NTT of the pair's two targets side by side and store them.
+// take the items in turn. A group's two halves of 128 threads own two targets each: a
+// thread reads its eight points (N1/8 rows apart) of both targets from TMEM, reduces them,
+// and runs each target's column NTT in radix-8 register rounds, the first straight on
+// the points it reduced, with an exchange through the half's tile between rounds and the
+// last round's results stored from registers.
 // Full / empty mbarriers and a read counter hand the buffers over between the roles.
 #include <algorithm>
 
+#include "ks_core.cuh"
 #include "ks_internal.h"
 #include "ks_kern.cuh"
 
@@ -111,24 +116,21 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// The exact S = sum_s v_s 2^(8s) from the fp32 bits r[s] = 0x4B000000 + v_s
-// (v_s < 2^23): pairs P_k = v_2k + v_2k+1 2^8 (< 2^32, weight 2^16k; the 0x4B
-// exponent byte of the shifted word falls off the top), quads Q_m = P_2m + P_2m+1 2^16
-// (weight 2^32m), then S = Q_0 + Q_1 2^32 + Q_2 2^64 + Q_3 2^96. S < 2^128 keeps
-// Q_3 2^32 inside the high word.
-__device__ __forceinline__ U128 tc_sum(const uint32_t (&r)[16]) {
-  constexpr uint32_t E = 0x4B000000u;
-  uint32_t P[8];
-#pragma unroll
-  for (int k = 0; k < 7; ++k) P[k] = r[2 * k] + (r[2 * k + 1] << 8) - E;
-  P[7] = r[14] - E;
-  u64 Q[4];
-#pragma unroll
-  for (int m = 0; m < 4; ++m) Q[m] = (u64)P[2 * m] + ((u64)P[2 * m + 1] << 16);
-  U128 s;
-  s.lo = Q[0] + (Q[1] << 32);
-  s.hi = (Q[1] >> 32) + Q[2] + (Q[3] << 32) + (s.lo < Q[0] ? 1ull : 0ull);
-  return s;
+// S 2^-32 mod m in (0, 1.01 m] from the fp32 bits r[b] = 0x4B000000 + v_b of S = sum_b v_b
+// 2^(8b), S < 2^15 m. Pairs P_k = v_2k + v_2k+1 2^8 keep one 0x4B000000 each (below 2^32
+// with it; the shifted word's falls off the top), Q_0 = P_0 + P_1 2^16 and Q_1 = P_2 +
+// P_3 2^16 (weight 2^32) then hold kTcBias too much; mc = m - kTcBias takes Q_1's back and
+// adds the m that keeps the result positive. One Montgomery step: u = S m^-1 mod 2^32
+// (inv = m^-1), S - u m is a multiple of 2^32.
+constexpr u64 kTcBias = 0x4B000000ull * 65537ull;
+__device__ __forceinline__ u64 tc_reduce(const uint32_t *r, u64 m, uint32_t inv, u64 mc) {
+  const uint32_t p0 = r[0] + (r[1] << 8), p1 = r[2] + (r[3] << 8);
+  const uint32_t p2 = r[4] + (r[5] << 8), p3 = r[6] + (r[7] << 8);
+  const u64 q0 = (u64)p0 + ((u64)p1 << 16) - kTcBias;
+  const u64 q1 = (u64)p2 + ((u64)p3 << 16) + mc;
+  const uint32_t u = (uint32_t)q0 * inv;
+  const u64 e = (mul_wide(u, (uint32_t)m) >> 32) + mul_wide(u, (uint32_t)(m >> 32));
+  return q1 + (q0 >> 32) - e;
 }
 
 // A progress counter in shared memory, written by one thread and polled by another:
@@ -154,37 +156,37 @@ __device__ __forceinline__ bool rd_wait(volatile int *c, int want) {
 }
 
 // Column tiles of TP = 2^kTcTpLog points (N1 rows x GC columns; the inverse column
-// passes write the source bytes in blocks of this size), kTcTargets = 2 targets per
+// passes write the source bytes in blocks of this size), kTcTargets = 4 targets per
 // work item (ks_internal.h).
 // Consumer groups per CTA.
 constexpr int kTcGroups = 2;
 
 // Geometry. Consumers: GRP groups of 256 threads taking items round-robin (so that one
 // group's waits and barriers overlap the other's arithmetic); a group is two halves of
-// 128 threads, one per target of the pair, 8 points per thread (radix-8 NTT rounds).
-// Per group: a TMEM accumulator (8 M blocks x 32 columns), a double constant buffer and
-// two NTT tiles. The column twiddles are read from the table (L1).
+// 128 threads with two targets and one exchange tile each, 8 points of a target per
+// thread. Per group: a TMEM accumulator (8 M blocks x 32 columns) and a double constant
+// buffer. The column twiddles are read from the table (L1).
 template <int LOGN, int GRP>
 struct TcGeo {
   static constexpr int LOGA = geo_loga(LOGN), LOGB = LOGN - LOGA;
   static constexpr int N1 = 1 << LOGA;
   static constexpr int TPLOG = kTcTpLog, TP = 1 << TPLOG;
-  static constexpr int LOGGC = TPLOG - LOGA, GC = 1 << LOGGC, PC = GC + 1;
+  static constexpr int LOGGC = TPLOG - LOGA, GC = 1 << LOGGC;
   static constexpr int MB = TP / 128;  // M blocks of 128 points
-  static constexpr int PTS = 8, RM = 3;  // points per consumer thread, NTT stages per round
-  static constexpr int HT = TP / PTS;    // consumer threads per target
+  static constexpr int RL = 3, PTS = 8;  // points of a target per consumer thread
+  static constexpr int HT = TP / PTS;    // threads of a half
   static constexpr int GT = 2 * HT;      // threads per group
   static constexpr int NT = GRP * GT;    // consumer threads (+ issuer and loader warps)
   static constexpr int TILES = (1 << LOGN) / TP;
-  static constexpr int DCOLS = MB * 32;  // TMEM columns per group
+  static constexpr int DCOLS = MB * 8 * kTcTargets;  // TMEM columns per group
   static constexpr int COLS = GRP * DCOLS <= 256 ? 256 : 512;
-  static constexpr int TILE_W = N1 * PC;  // words of one target's NTT tile
+  static constexpr int TILE_W = core::col_words<LOGA, GC, RL>();  // words of a half's tile
   static constexpr int APMAX = 10;        // K slots (alpha <= 9)
   __host__ __device__ static constexpr int smem(int ap) {
-    return ap * TP * 16 + GRP * 1024 * ap + GRP * 2 * TILE_W * 8;
+    return ap * TP * 16 + GRP * 2 * kTcTargets * 128 * ap + GRP * 2 * TILE_W * 8;
   }
-  static_assert(kTcTargets == 2 && LOGGC >= 1 && MB % 4 == 0 && (HT / 32) % 4 == 0 &&
-                    GRP * DCOLS <= 512 && smem(APMAX) <= 227 * 1024 - 256 && NT + 64 <= 1024,
+  static_assert(kTcTargets == 4 && MB == PTS && HT == 128 && GRP * DCOLS <= 512 &&
+                    smem(APMAX) <= 227 * 1024 - 512 && NT + 64 <= 1024,
                 "tile shape");
 };
 
@@ -221,17 +223,17 @@ __global__ void __launch_bounds__(TcGeo<LOGN, GRP>::NT + 64, 1)
   __shared__ u64 bar_a, bar_b[GRP][2], bar_m[GRP], bar_tm[GRP];
   __shared__ uint32_t tm_slot;
   __shared__ volatile int rd[GRP];
-  // per group and slot, written by the loader before it arms bar_b: the pair's decoded
-  // work items, how many are real, the tile, whether both moduli take the fast
-  // butterflies, and the source set
-  __shared__ uint32_t info_w[GRP][2][2];
-  __shared__ int info_cnt[GRP][2], info_tile[GRP][2], info_fast[GRP][2], info_set[GRP][2];
+  // per group and slot, written by the loader before it arms bar_b: the targets' decoded
+  // work items, how many are real, the tile and the source set
+  __shared__ uint32_t info_w[GRP][2][kTcTargets];
+  __shared__ int info_cnt[GRP][2], info_tile[GRP][2], info_set[GRP][2];
   const JobPtr &jp = js.j[blockIdx.z];
   const int AP = a.tc_ap;
   const int it0 = blockIdx.x * ti.per_cta, it1 = min(ti.items, it0 + ti.per_cta);
   unsigned char *sA = raw;
-  unsigned char *sB = raw + (size_t)AP * G::TP * 16;  // [GRP][buffer 2][target 2][256 ap]
-  u64 *sT = reinterpret_cast<u64 *>(sB + (size_t)GRP * 1024 * AP);  // [GRP][2][TILE_W]
+  constexpr int TB = 128;  // constant bytes of a target per K slot
+  unsigned char *sB = raw + (size_t)AP * G::TP * 16;  // [GRP][buffer 2][target 4][128 ap]
+  u64 *sT = reinterpret_cast<u64 *>(sB + (size_t)GRP * 2 * kTcTargets * TB * AP);  // [GRP][2][TILE_W]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int CW = G::NT / 32;  // consumer warps; warp CW issues, warp CW + 1 loads
 
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(TcGeo<LOGN, GRP>::NT + 64, 1)
   // zero), with bf16 1.0 in the first K element of slot alpha (the 2^23 row); B: zero.
   for (int k = threadIdx.x; k < AP * G::TP; k += blockDim.x)
     reinterpret_cast<uint4 *>(sA)[k] = make_uint4(k / G::TP == a.alpha ? 0x3F80u : 0u, 0, 0, 0);
-  for (int k = threadIdx.x; k < GRP * 64 * AP; k += blockDim.x)
+  for (int k = threadIdx.x; k < GRP * 2 * kTcTargets * TB / 16 * AP; k += blockDim.x)
     reinterpret_cast<uint4 *>(sB)[k] = make_uint4(0, 0, 0, 0);
   proxy_fence();
   tc_fence_before();
@@ -262,8 +264,8 @@ __global__ void __launch_bounds__(TcGeo<LOGN, GRP>::NT + 64, 1)
   auto target = [&](const TcItem &x, int u) { return decode(a, tk, x.y0 + min(u, x.cnt - 1)); };
   if (warp == CW + 1) {
     // Loader warp: each item's decoded targets (the info its group and the issuer read)
-    // and the pair's constants, into the group's buffer of the item's index mod 2; lane
-    // u < 2 decodes and copies target u.
+    // and their constants, into the group's buffer of the item's index mod 2; lane
+    // u < kTcTargets decodes and copies target u.
     for (int it = it0; it < it1; ++it) {
       const int g = (it - it0) % GRP, k = (it - it0) / GRP, b = k & 1;
       // buffer b and info slot b were last used by the group's item k - 2: wait until
@@ -276,29 +278,26 @@ __global__ void __launch_bounds__(TcGeo<LOGN, GRP>::NT + 64, 1)
       }
       const TcItem x = tc_item(ti, it);
       uint32_t w = 0;
-      int f = 1;
-      if (lane < 2) {
+      if (lane < kTcTargets) {
         w = target(x, lane);
         info_w[g][b][lane] = w;
-        f = a.tab.mod[task_limb(w)].m < kFastModulus;
       }
-      f = __all_sync(0xffffffffu, f);
       if (lane == 0) {
         info_cnt[g][b] = x.cnt;
         info_tile[g][b] = x.tile;
         info_set[g][b] = x.set;
-        info_fast[g][b] = f;
       }
       __threadfence_block();
       __syncwarp();
-      if (lane == 0) mbar_expect_tx(&bar_b[g][b], 2u * 256 * AP);  // releases the info
+      if (lane == 0) mbar_expect_tx(&bar_b[g][b], kTcTargets * TB * AP);  // releases the info
       __syncwarp();
-      if (lane < 2) {
+      if (lane < kTcTargets) {
         const int t = task_limb(w);
         const u64 *src = PRO == PRO_UP
-                             ? a.tab.bup + ((size_t)task_dig(w) * a.qp + t) * 32 * AP
-                             : a.tab.bdown + (size_t)t * 32 * AP;
-        bulk_g2s(sB + (size_t)((g * 2 + b) * 2 + lane) * 256 * AP, src, 256 * AP, &bar_b[g][b]);
+                             ? a.tab.bup + ((size_t)task_dig(w) * a.qp + t) * (TB / 8) * AP
+                             : a.tab.bdown + (size_t)t * (TB / 8) * AP;
+        bulk_g2s(sB + (size_t)((g * 2 + b) * kTcTargets + lane) * TB * AP, src, TB * AP,
+                 &bar_b[g][b]);
       }
     }
   } else if (warp == CW) {
@@ -342,79 +341,84 @@ __global__ void __launch_bounds__(TcGeo<LOGN, GRP>::NT + 64, 1)
           cur_set = xset;
         }
         tc_fence_after();
-        const u64 bd0 = smem_desc(smem_u32(sB + (size_t)(g * 2 + b) * 512 * AP), 128, AP * 128);
+        const u64 bd0 =
+            smem_desc(smem_u32(sB + (size_t)(g * 2 + b) * kTcTargets * TB * AP), 128, AP * TB);
         const uint32_t d0 = tmem + g * G::DCOLS;
         // descriptors advance by (byte offset >> 4) in their start-address field; the
         // K steps outside, so consecutive MMAs accumulate into different M blocks
         for (int s = 0; s < AP / 2; ++s)
 #pragma unroll
           for (int mb = 0; mb < G::MB; ++mb)
-            tc_mma(d0 + mb * 32, ad0 + (u64)(2 * s * G::TP + mb * 128), bd0 + (u64)(16 * s),
-                   tc_idesc(32), s > 0);
+            tc_mma(d0 + mb * 8 * kTcTargets, ad0 + (u64)(2 * s * G::TP + mb * 128),
+                   bd0 + (u64)(16 * s), tc_idesc(8 * kTcTargets), s > 0);
         tc_commit(&bar_m[g]);
       }
     }
   } else {
-    // Consumers: recombine the sums of each item, then the two targets' column NTTs.
-    const int group = threadIdx.x / G::GT, bar_id = 1 + group;
-    const int half = (threadIdx.x % G::GT) / G::HT;  // the target of the pair
+    // Consumers: reduce the sums of each item, then the half's two column NTTs.
+    const int group = threadIdx.x / G::GT;
+    const int half = (threadIdx.x % G::GT) / G::HT;  // targets 2 half, 2 half + 1 of the item
     const int q = warp & 3;  // TMEM lane quadrant of the warp (its 32 points of each M block)
+    // the thread's points of a target: row (N1/8) mb + ct, column cg, mb = 0..7
+    const int lt = 32 * q + lane, ct = lt >> G::LOGGC, cg = lt & (G::GC - 1);
     u64 *dst = jp.ws + (PRO == PRO_UP ? wo.tmp : wo.tmp2);
     u64 *tile = sT + (group * 2 + half) * G::TILE_W;
+    auto sync = [&] { round_sync<G::HT>(1 + group * 2 + half); };
     for (int it = it0 + group, k = 0; it < it1; it += GRP, ++k) {
-      // the pair's decoded items (the loader's info, released with its constants)
+      // the targets' decoded items (the loader's info, released with their constants)
       const int b = k & 1;
       if (!mbar_wait(&bar_b[group][b], (k >> 1) & 1)) atomicExch(a.tab.err, 1);
-      const uint32_t w = info_w[group][b][half];
+      uint32_t w[2];
+      u64 mm[2];
+      uint32_t inv[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        w[i] = info_w[group][b][2 * half + i];
+        const ModInfo &mi = a.tab.mod[task_limb(w[i])];
+        mm[i] = mi.m;
+        inv[i] = 0u - (uint32_t)mi.minv;
+      }
       const int cnt = info_cnt[group][b], xtile = info_tile[group][b];
-      const bool fast = info_fast[group][b] != 0;
-      const ModInfo mi = a.tab.mod[task_limb(w)];
       if (!mbar_wait(&bar_m[group], k & 1)) atomicExch(a.tab.err, 1);
       tc_fence_after();
+      u64 z[2][G::PTS];
 #pragma unroll
-      for (int b0 = 0; b0 < G::MB; b0 += 4) {
-        uint32_t v[4][16];
+      for (int b0 = 0; b0 < G::MB; b0 += 2) {
+        uint32_t v[2][16];
 #pragma unroll
-        for (int bb = 0; bb < 4; ++bb)
-          tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + group * G::DCOLS + (b0 + bb) * 32 +
-                        half * 16,
+        for (int bb = 0; bb < 2; ++bb)
+          tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + group * G::DCOLS +
+                        (b0 + bb) * 8 * kTcTargets + half * 16,
                     v[bb]);
         tmem_wait_ld();
-        if (b0 + 4 == G::MB) {  // the warp's last reads of the accumulator
+        if (b0 + 2 == G::MB) {  // the warp's last reads of the accumulator
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&bar_tm[group]);
         }
 #pragma unroll
-        for (int bb = 0; bb < 4; ++bb) {
-          const u64 z = redc(tc_sum(v[bb]), mi.m, mi.minv);
-          const int p = (b0 + bb) * 128 + 32 * q + lane;
-          tile[(p >> G::LOGGC) * G::PC + (p & (G::GC - 1))] = z;
-        }
-      }
-      round_sync<G::GT>(bar_id);
-      // both halves take the same butterflies (their rounds share the barrier): the fast
-      // ones only when both moduli allow them; twiddles from the column table
-      const ulonglong2 *tw = a.tab.twc_f + ((size_t)task_limb(w) << G::LOGA);
-      if (fast)
-        tile_fwd_t<G::LOGA, G::LOGGC, G::PC, G::HT, false, G::RM, true, 0, true, G::GT>(
-            tile, tw, mi.m, bar_id);
-      else
-        tile_fwd_t<G::LOGA, G::LOGGC, G::PC, G::HT, false, G::RM, false, 0, true, G::GT>(
-            tile, tw, mi.m, bar_id);
-      if (half < cnt) {
-        u64 *d = dst + (size_t)task_slot(w) * a.N;
-        const int c0 = xtile * G::GC, lt = threadIdx.x & (G::HT - 1);
+        for (int bb = 0; bb < 2; ++bb)
 #pragma unroll
-        for (int r = 0; r < G::TP / 2 / G::HT; ++r) {
-          const int e = 2 * (lt + r * G::HT), y = e >> G::LOGGC, c = e & (G::GC - 1);
-          ulonglong2 val;
-          val.x = tile[y * G::PC + c];
-          val.y = tile[y * G::PC + c + 1];
-          *reinterpret_cast<ulonglong2 *>(d + ((size_t)y << G::LOGB) + c0 + c) = val;
-        }
+          for (int i = 0; i < 2; ++i)
+            z[i][b0 + bb] = tc_reduce(v[bb] + 8 * i, mm[i], inv[i], mm[i] - kTcBias);
       }
-      round_sync<G::GT>(bar_id);  // the group's tiles are free for its next item
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (2 * half + i >= cnt) break;
+        const int t = task_limb(w[i]), cls = mod_class(mm[i]);
+        const ulonglong2 *tw = a.tab.twc_f + ((size_t)t << G::LOGA);
+        if (cls == CLS_FAST)
+          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_FAST, 0>(z[i], tile, tw, mm[i], ct, cg, sync);
+        else if (cls == CLS_MID)
+          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_MID, 0>(z[i], tile, tw, mm[i], ct, cg, sync);
+        else
+          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_EXACT, 0>(z[i], tile, tw, mm[i], ct, cg, sync);
+        using CL = core::ColRound<G::LOGA, G::RL, core::col_rounds<G::LOGA, G::RL>() - 1>;
+        u64 *d = dst + ((size_t)task_slot(w[i]) << LOGN) + xtile * G::GC + cg;
+#pragma unroll
+        for (int r = 0; r < G::PTS; ++r) d[(size_t)CL::point(ct, r) << G::LOGB] = z[i][r];
+        sync();  // the tile is free for the next target
+      }
     }
   }
   tc_fence_before();
