@@ -59,7 +59,7 @@ extern "C" {
 #define KS_UNFUSED 0x100
 /* OR-ed into the variant: register rounds of radix 4 (4 points per thread, twice the
  * threads per tile) instead of radix 8. The radix, the schedule and the column tiles below
- * tell kernels apart at N <= 2^12 (the column tiles nowhere); the larger sizes have one set
+ * tell kernels apart at N <= 2^11 (the column tiles nowhere); the larger sizes have one set
  * of kernels, and accept these flags without effect. */
 #define KS_RADIX4 0x200
 /* OR-ed into the variant: register rounds of radix 16 (16 points per thread, half the
@@ -203,7 +203,7 @@ int ks_workspace_size(const ks_context *ctx, int variant, int chunks, size_t *by
  *           workspace (allocated on first use and grown as needed; calls that use it
  *           must then be ordered, e.g. issued on one stream).
  * Asynchronous on `stream`. The kernels are chained by programmatic dependent launch
- * (consecutive calls on a stream overlap their boundaries); for N <= 2^12 repeated
+ * (consecutive calls on a stream overlap their boundaries); for N <= 2^11 repeated
  * calls with the same plan, buffers and stream replay a cached CUDA graph. */
 int ks_switch(ks_context *ctx, const uint64_t *d_dev, const uint64_t *evk_dev,
               uint64_t *out_dev, int variant, int chunks, void *workspace_dev,
@@ -260,7 +260,7 @@ int ks_switch_host(ks_context *ctx, const uint64_t *d_host, const uint64_t *evk_
  * the last one writes out_host; the result is there once `stream` has passed this call
  * (an event or a synchronize), and d_host must stay unmodified until then. Calls on one context share its staging
  * buffer and workspace, so they must be ordered (issued on one stream); consecutive
- * calls are chained like ks_switch's (N <= 2^12: cached graph replay). */
+ * calls are chained like ks_switch's (N <= 2^11: cached graph replay). */
 int ks_switch_host_async(ks_context *ctx, const uint64_t *d_host, const uint64_t *evk_dev,
                          uint64_t *out_host, int variant, int chunks, void *stream);
 
@@ -354,7 +354,7 @@ int ks_switch_batch(const ks_job *jobs, int njobs, int flags, void *stream);
  * launched by this process: KS_OK, or KS_ETIMEOUT if a bounded wait gave up. */
 int ks_batch_status(void *stream);
 
-/* Autotuner: times the dataflows {DPOB, DSOB, DPOC c=2, DPOC c=4, DSOC c=2} (N <= 2^12:
+/* Autotuner: times the dataflows {DPOB, DSOB, DPOC c=2, DPOC c=4, DSOC c=2} (N <= 2^11:
  * each with radix 8, radix 4 and radix 16) on this job (replicated `batch` times, 1..16, in
  * one launch set); then, for N >= 2^13, tries the tensor-core basis conversions
  * (KS_BCONV_TC, else KS_BCONV_TC_DOWN) and, for DPOB, the split ModDown (KS_SPLIT_DOWN) on

@@ -59,6 +59,17 @@ int tc_rule(const ks_context *c) {
 // integer plans) with the tensor-core rule.
 int selected_plan(const ks_context *c) { return c->sel_variant | tc_rule(c); }
 
+// The cluster kernels (ks_fused.cuh) serve the plain fused DPOB plan when they have the
+// size's limbs, the digits fit a CTA's shared memory, and their widest launch, eight CTAs
+// per target limb of every job, gives each CTA its own SM: they are latency-bound, and
+// lose to the general kernels once a launch takes a second wave. Measured (cluster /
+// general kernels): (2, 2^12, 3) 27.9 / 32.1 us, (2, 2^12, 11) 33.0 / 34.1, (2, 2^13, 7)
+// 31.9 / 33.2, (2, 2^13, 11) 36.0 / 37.3; beyond: (4, 2^13, 15) 44.7 / 39.7,
+// (6, 2^13, 44) 119 / 87; (7, 2^14, 30) 154 / 130, (2, 2^15, 10) 88 / 64.
+bool fused_rule(const ks_context *c, int jobs) {
+  return c->fu && c->fu->fits(c->beta) && 8 * c->qp * jobs <= 152;
+}
+
 int make_plan(const ks_context *c, int variant, int chunks, Plan *pl) {
   if (variant & ~(0xff | KS_UNFUSED | KS_RADIX4 | KS_RADIX16 | kSchedMask | KS_COLTILE_ALT |
                   KS_SPLIT_DOWN | KS_BCONV_TC | KS_BCONV_TC_DOWN))
@@ -215,6 +226,14 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
   const bool dp = pl.base == KS_DPOB || pl.base == KS_DPOC;
   const bool oc = pl.base == KS_DSOC || pl.base == KS_DPOC;
   auto dsize = [&](int j) { return std::min(c->nq, (j + 1) * c->alpha) - j * c->alpha; };
+
+  // Small sizes: the four steps as one cluster kernel each. (While the profiler is on, the
+  // stages run as their own launches, which it times.)
+  if (pl.base == KS_DPOB && !pl.unfused && !pl.tc_down && !split && !g_prof.on &&
+      fused_rule(c, js.n)) {
+    KS_TRY(c->fu->run(c, js, wo, s));
+    return KS_OK;
+  }
 
   // Input iNTT, fused with the per-limb factor N^-1 * Qhat_{j,i}^-1 of the ModUp BConv.
   {
@@ -500,7 +519,6 @@ int create_context(int dnum, int logn, int L, const u64 *q, const u64 *p, int al
   c->N = 1 << logn;
   c->loga = ks::geo_loga(logn);
   c->logb = logn - c->loga;
-  c->loggr = ks::geo_loggr(logn);
   for (int r = 0; r < 3; ++r) {
     const LaunchTable *t = ks::launch_table(logn, r + 2);
     if (!t || t->prepare() != cudaSuccess) {
@@ -511,6 +529,11 @@ int create_context(int dnum, int logn, int L, const u64 *q, const u64 *p, int al
     c->ltab[r] = t;
   }
   c->lt = c->ltab[1];
+  c->fu = ks::fused_table(logn);
+  if (c->fu && c->fu->prepare() != cudaSuccess) {
+    cudaGetLastError();
+    c->fu = nullptr;
+  }
   if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
@@ -528,7 +551,7 @@ int create_context(int dnum, int logn, int L, const u64 *q, const u64 *p, int al
   // fp32 sums of byte products stay exact below 2^23 up to 16 sources; the source bytes
   // of a 1024-point tile fill the shared memory at 9), one REDC per sum, at most
   // kTcMaxSets digits.
-  if (c->loga > 0 && logn <= 17 && alpha >= 2 && alpha <= 9 && beta <= ks::kTcMaxSets &&
+  if (logn >= 13 && logn <= 17 && alpha >= 2 && alpha <= 9 && beta <= ks::kTcMaxSets &&
       c->run_up >= alpha && c->run_down >= alpha) {
     c->tc_ap = (alpha + 2) & ~1;  // alpha + 1 slots (the last adds 2^23), rounded to even
     c->tc_tplog = ks::kTcTpLog;   // column tiles of the tensor-core items
@@ -621,7 +644,7 @@ void drop_graph_cache(ks_context *c) {
 // operations on a stream when they are launched directly but not across graph
 // launches. Directly launched, (2, 2^15, 10) runs at 76.7 us per KeySwitch against
 // 83.0 us replayed from graphs. Graphs are used where launches cost more than they
-// overlap: single-pass sizes (N <= 2^12, a few microseconds of GPU work per kernel)
+// overlap: single-pass sizes (N <= 2^11, a few microseconds of GPU work per kernel)
 // and the synchronous host-buffer entry point (one launch per call).
 bool use_graphs(const ks_context *c) { return c->loga == 0; }
 template <class F>
@@ -1450,7 +1473,7 @@ int ks_tune(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *out
     }
     return ms_min;
   };
-  // 1) dataflow, and the radix where it names different kernels (N <= 2^12)
+  // 1) dataflow, and the radix where it names different kernels (N <= 2^11)
   float best = 1e30f;
   int best_v = KS_DPOB, best_c = 0;
   for (auto &b : bases)

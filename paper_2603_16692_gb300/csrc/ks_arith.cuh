@@ -205,17 +205,22 @@ __device__ __forceinline__ uint4 bf16_bytes(u64 x) {
 }
 
 // Programmatic dependent launch. Every KeySwitch kernel lets the next kernel of its
-// stream launch once all its CTAs reach their end (pdl_trigger), and waits for the
-// previous kernel to complete, with its memory visible, before it reads or writes any
-// buffer that kernels share (pdl_wait); what comes before the wait reads only the
-// context's constant tables and writes only shared memory. Without the launch
-// attribute both are no-ops. (Measured on GB300: triggering at the end rather than at
-// the start took (2, 2^13, 7) from 61 to 52 us per KeySwitch; triggering at the start
-// slowed (2, 2^15, 10) by 16%, the dependent CTAs being placed while the previous
-// kernel still ran.)
+// stream launch (pdl_trigger), and waits for the previous kernel to complete, with its
+// memory visible, before it reads or writes any buffer that kernels share (pdl_wait); what
+// comes before the wait reads only the context's constant tables and the keys (into L2)
+// and writes only shared memory. Without the launch attribute both are no-ops.
+// When the next kernel may launch: a launch of more than one wave (early) triggers right
+// after its wait, so that the next kernel's CTAs start their prologues in the slots that
+// its last wave leaves free: (4, 2^16, 35) 363 -> 344 us, (10, 2^17, 60) 1,646 -> 1,634,
+// (7, 2^14, 30) 130 -> 123. A smaller launch triggers at its end: its CTAs all start at
+// once, and dependents placed at that moment crowd the SMs it left empty ((2, 2^15, 10) 64
+// -> 74 us with every launch early, (2, 2^12, 3) 32 -> 36).
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait(int early = 0) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (early) pdl_trigger();
+}
 
 __device__ __forceinline__ u64 addmod(u64 a, u64 b, u64 m) { return csub(a + b, m); }

@@ -159,6 +159,7 @@ template <class SB, int CLS>
 __device__ __forceinline__ void row_fwd(u64 *v, u64 *s, const ulonglong2 *tw, u64 m, int t) {
   constexpr int RL = SB::RL, R2 = SB::R2, S = SB::S, E = SB::E;
   auto exchange = [&] {
+    __syncwarp();  // the row's earlier reads are done
 #pragma unroll
     for (int u = 0; u < E; ++u) s[row_pos((u << SB::LOGT) + t)] = v[u];
     __syncwarp();

@@ -38,9 +38,9 @@ const LaunchTable &launch_table_10_4_0();
 const LaunchTable &launch_table_11_3_0();
 const LaunchTable &launch_table_11_2_0();
 const LaunchTable &launch_table_11_4_0();
-const LaunchTable &launch_table_12_3_0();
-const LaunchTable &launch_table_12_2_0();
-const LaunchTable &launch_table_12_4_0();
+const FusedTable &fused_table_12();
+const FusedTable &fused_table_13();
+const LaunchTable &launch_table_12();
 const LaunchTable &launch_table_13();
 const LaunchTable &launch_table_14();
 const LaunchTable &launch_table_15();
@@ -48,7 +48,7 @@ const LaunchTable &launch_table_16();
 const LaunchTable &launch_table_17();
 
 namespace {
-// [log N][radix log 2..4]: the single-pass sizes (N <= 2^12) have kernels per register-round
+// [log N][radix log 2..4]: the single-pass sizes (N <= 2^11) have kernels per register-round
 // radix; the two-pass sizes have one set, which every radix and column tile names.
 using TableFn = const LaunchTable &(*)();
 struct TableSet {
@@ -60,8 +60,8 @@ struct TableSet {
   fn[N][4] = &launch_table_##N##_4_0;
 #define KS_T1(N) fn[N][2] = fn[N][3] = fn[N][4] = &launch_table_##N;
     KS_T0(1) KS_T0(2) KS_T0(3) KS_T0(4) KS_T0(5) KS_T0(6) KS_T0(7) KS_T0(8) KS_T0(9)
-    KS_T0(10) KS_T0(11) KS_T0(12)
-    KS_T1(13) KS_T1(14) KS_T1(15) KS_T1(16) KS_T1(17)
+    KS_T0(10) KS_T0(11)
+    KS_T1(12) KS_T1(13) KS_T1(14) KS_T1(15) KS_T1(16) KS_T1(17)
 #undef KS_T0
 #undef KS_T1
   }
@@ -73,6 +73,14 @@ const LaunchTable *launch_table(int logn, int rl) {
   if (logn < 1 || logn > 17 || rl < 2 || rl > 4) return nullptr;
   const TableFn f = t.fn[logn][rl];
   return f ? &f() : nullptr;
+}
+
+const FusedTable *fused_table(int logn) {
+  switch (logn) {
+    case 12: return &fused_table_12();
+    case 13: return &fused_table_13();
+    default: return nullptr;
+  }
 }
 
 namespace kern {

@@ -1,4 +1,4 @@
-// Kernel instantiations for N = 2^LOGN, LOGN in { 11 12 }, radix 8, 4 and 16.
+// Kernel instantiations for N = 2^LOGN, LOGN in { 11 }, radix 8, 4 and 16.
 #include "ks_rows.cuh"
 
 namespace ks {
@@ -7,8 +7,5 @@ namespace ks {
 KS_INST(11, 3, 0)
 KS_INST(11, 2, 0)
 KS_INST(11, 4, 0)
-KS_INST(12, 3, 0)
-KS_INST(12, 2, 0)
-KS_INST(12, 4, 0)
 #undef KS_INST
 }  // namespace ks

@@ -14,6 +14,8 @@ typedef unsigned long long u64;
 
 namespace ks {
 
+struct FusedTable;
+
 constexpr int kMaxLimbs = 256;   // QP limit (L+1 <= 128, alpha <= 128)
 
 // Per-modulus constants (device).
@@ -134,11 +136,14 @@ struct ks_context {
   int eqp = 0, epb = 0;
   int top_L = -1;  // level of the context whose keys this one uses (-1: itself)
   int N;
-  int loga, logb, loggr;  // two-pass split N = 2^loga * 2^logb; rows per row tile 2^loggr
+  int loga, logb;  // two-pass split N = 2^loga * 2^logb (loga = 0: one pass)
   // Launchers by register-round radix (index log2 radix - 2; the two-pass sizes have one
   // set); lt = radix 8.
   const ks::LaunchTable *ltab[3] = {};
   const ks::LaunchTable *lt = nullptr;
+  // cluster kernels for the plain fused DPOB plan (null for sizes without them; fused_rule
+  // in ks_api.cu says when they run)
+  const ks::FusedTable *fu = nullptr;
   int run_up = 1, run_down = 1;  // max terms per exact 128-bit BConv sum
   // Tensor-core basis conversions: K slots per source set (alpha + 1 rounded up to
   // even; 0 = not available for this context) and log2 of the points per column tile.
@@ -215,7 +220,7 @@ struct LaunchTable {
   int (*count)(const ks_context *, const Tasks &);
   // iNTT of the L+1 input limbs (which = 0: d -> v, scaled by N^-1 Qhat^-1) or of the
   // alpha P-limbs of both accumulators (which = 1: acc -> vp, scaled by N^-1 Phat^-1).
-  // Row pass (src -> dst), then the column pass in place (none when N <= 4096).
+  // Row pass (src -> dst), then the column pass in place (none when N <= 2048).
   cudaError_t (*intt_row)(const ks_context *, const JobSet &, const WsOff &, int which,
                           cudaStream_t);
   cudaError_t (*intt_col)(const ks_context *, const JobSet &, const WsOff &, int which,
@@ -244,6 +249,15 @@ struct LaunchTable {
   cudaError_t (*ntt_row)(const ks_context *, const JobSet &, const WsOff &, const Tasks &,
                          int buf, cudaStream_t);
 };
+// The cluster kernels of a small N (ks_fused.cuh): a whole fused DPOB KeySwitch in four
+// launches. fits: the digits of a target fit a CTA's shared memory.
+struct FusedTable {
+  cudaError_t (*prepare)();
+  bool (*fits)(int beta);
+  cudaError_t (*run)(const ks_context *, const JobSet &, const WsOff &, cudaStream_t);
+};
+const FusedTable *fused_table(int logn);  // null for sizes without them
+
 // ks_switch on the caller's workspace `ws` (ws_bytes >= ks_workspace_size) that only
 // launches kernels, all on `stream` (a KS_SPLIT_DOWN plan runs unsplit): no graph
 // cache, no arena (ks_api.cu).
@@ -253,7 +267,7 @@ int switch_launch_only(ks_context *c, const uint64_t *d, const uint64_t *evk, ui
 bool selected_current(const ks_context *c);
 
 // rl = log2 of the radix of the register rounds (3: 8 points per thread, 2: 4, 4: 16); it
-// tells kernels apart at N <= 2^12 only.
+// tells kernels apart at N <= 2^11 only.
 const LaunchTable *launch_table(int logn, int rl);
 
 // Tensor-core basis conversion + first forward NTT pass (ks_tc.cu), in place of the

@@ -26,6 +26,7 @@ struct KArgs {
   int run_up, run_down;
   int eqp, epb;  // key layout (see ks_context)
   int tc_ap, tc_tplog;  // tensor-core basis conversion (see ks_context)
+  int early;            // let the next kernel launch at this one's start (early_rule)
 };
 
 // Word offset of evk[j][c][limb t] (t in the context's Q u P numbering).
@@ -55,6 +56,7 @@ inline KArgs make_args(const ks_context *c) {
   a.epb = c->epb;
   a.tc_ap = c->tc_ap;
   a.tc_tplog = c->tc_tplog;
+  a.early = 0;
   return a;
 }
 
@@ -1094,6 +1096,21 @@ inline cudaError_t smem_attr(K kernel, int bytes) {
 }
 
 inline KArgs args_of(const ks_context *c) { return make_args(c); }
+
+// Whether a launch of `threads` threads lets its dependent launch as soon as its own CTAs
+// have all started (see pdl_trigger): when it is more than a wave at the kernels' 768
+// threads per SM. (Half of that: (4, 2^16, 35) in four chunks 672 -> 716 us, whose launches
+// are about a wave; twice: (4, 2^16, 35) 344 -> 349 us.)
+inline int early_rule(size_t threads) { return threads > (size_t)152 * 768 ? 1 : 0; }
+
+// launch_pdl of a kernel whose first argument is its KArgs, with the early rule applied.
+template <class... KT, class... AT>
+inline cudaError_t launch_rule(void (*kernel)(KArgs, KT...), dim3 grid, dim3 block, size_t smem,
+                               cudaStream_t s, const ks_context *c, AT &&...args) {
+  KArgs a = args_of(c);
+  a.early = early_rule((size_t)grid.x * grid.y * grid.z * block.x);
+  return launch_pdl(kernel, grid, block, smem, s, a, static_cast<AT &&>(args)...);
+}
 
 }  // namespace kern
 }  // namespace ks

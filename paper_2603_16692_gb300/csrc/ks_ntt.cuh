@@ -15,7 +15,7 @@
 // N = N1 * N2. The column pass runs stages 0..log N1-1 on the N2 columns (each an
 // N1-point transform with twiddle index 2^ls + c for local stage ls, block c);
 // the row pass runs the remaining stages on the N1 rows of N2 contiguous points
-// (twiddle index (N1 + row) 2^ls + c). For N <= 4096 one row pass does all.
+// (twiddle index (N1 + row) 2^ls + c). For N <= 2048 one row pass does all.
 //
 // A tile holds G = 2^LOGG sub-transforms of M = 2^LOGM points; point x of
 // sub-transform g lives at s[x*P + g] (P = G+1 for G > 1: an odd pitch keeps
@@ -33,7 +33,7 @@ namespace ks {
 
 // Compile-time geometry of the two passes for N = 2^LOGN (also used on the host
 // to lay out the row-pass twiddle table by row tile).
-__host__ __device__ constexpr int geo_loga(int logn) { return logn <= 12 ? 0 : logn / 2; }
+__host__ __device__ constexpr int geo_loga(int logn) { return logn <= 11 ? 0 : logn / 2; }
 // Tiles (measured on GB300). Column pass: 2^10 points up to N = 2^15, 2^11 above (at
 // 2^15 the smaller tiles double the CTAs of the one-wave launches, 94.8 -> 85.8 us per
 // KeySwitch at (2, 2^15, 10); at 2^16 the column passes are slower with 2^10 points).
@@ -41,14 +41,14 @@ __host__ __device__ constexpr int geo_loga(int logn) { return logn <= 12 ? 0 : l
 // (2, 2^13, 7), 81.5 -> 77.8 us at (2, 2^14, 20), 13.4 k -> 14.0 k KeySwitch/s at
 // (2, 2^15, 10); at (4, 2^16, 35) 2^9 is 2% slower).
 __host__ __device__ constexpr int geo_tile_log_col(int logn) {
-  return logn <= 12 ? logn : (logn >= 16 ? 11 : 10);
+  return logn <= 11 ? logn : (logn >= 16 ? 11 : 10);
 }
 // The alternative column tile the tuner may pick (CA = 1): the other of 2^10 / 2^11.
 __host__ __device__ constexpr int geo_tile_log_col_alt(int logn) {
-  return logn <= 12 ? logn : (logn >= 16 ? 10 : 11);
+  return logn <= 11 ? logn : (logn >= 16 ? 10 : 11);
 }
 __host__ __device__ constexpr int geo_tile_log_row(int logn) {
-  return logn <= 12 ? logn : (logn <= 15 ? 9 : 10);
+  return logn <= 11 ? logn : (logn <= 15 ? 9 : 10);
 }
 __host__ __device__ constexpr int geo_loggr(int logn) {
   return geo_tile_log_row(logn) - (logn - geo_loga(logn));

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(128, 6)
   // (see inv_row_body: an input in host memory is read without waiting for the
   // predecessor, which is waited for at the end)
   const bool host_in = which == 0 && jp.dsrc;
-  if (!host_in) pdl_wait();
+  if (!host_in) pdl_wait(a.early);
   const size_t off = ((size_t)(r0 + w0) << RG::LOGB);
   const u64 *src = host_in ? jp.dsrc + (size_t)ii * N + off
                            : is.src + ((size_t)o * is.src_outer + ii) * N + off;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(128, 6)
   u64 *d = is.dst + ((size_t)o * is.dst_outer + ii) * N + ((size_t)(r0 + row) << RG::LOGB);
 #pragma unroll
   for (int u = 0; u < SB::E; ++u) d[(u << SB::LOGT) + t] = reduce_full(v[u], m, mu);
-  if (host_in) pdl_wait();
+  if (host_in) pdl_wait(a.early);
   pdl_trigger();
 }
 
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(2 * ColGeo<LOGN>::GP, 768 / (2 * ColGeo<LOGN>:
     mbar_expect_tx(&twbar, CG::TW_BYTES);
     bulk_g2s(tws, a.tab.twc_i + ((size_t)prime << CG::LOGA), CG::TW_BYTES, &twbar);
   }
-  pdl_wait();
+  pdl_wait(a.early);
   u64 *d = is.dst + ((size_t)o * is.dst_outer + ii) * ((size_t)1 << LOGN);
   u64 v[CG::E];
 #pragma unroll
@@ -260,11 +260,79 @@ struct FwdColGeo {
   static constexpr int GRID = N2 / GC, SMEM = TW_BYTES + TILEW * 8;
 };
 
+// Fast basis conversion of a thread's eight points of a column (points C0::point(t, .) of the
+// first forward round; src: the sources' limb 0 at the column) onto limb tgt: REDC(sum_i
+// x_i c_i), canonical. PRO_UP: from digit dig's limbs of v; PRO_DOWN: from polynomial dig's
+// P-limbs of vp. The sums are exact (Mac3), four points at a time.
+template <int PRO, int LOGN>
+__device__ __forceinline__ void bconv_points(u64 *v, const KArgs &a, int tgt, int dig,
+                                             const u64 *src, int t, int cls) {
+  constexpr int LOGA = geo_loga(LOGN), LOGB = LOGN - LOGA;
+  using C0 = core::ColRound<LOGA, 3, 0>;
+  const ModInfo &mi = a.tab.mod[tgt];
+  const u64 m = mi.m;
+  const int i0 = dig * (PRO == PRO_UP ? a.alpha : a.np);
+  const int ns = PRO == PRO_UP ? min(a.nq, i0 + a.alpha) - i0 : a.np;
+  const u64 *cst = PRO == PRO_UP ? a.tab.cup + ((size_t)dig * a.qp + tgt) * a.alpha
+                                 : a.tab.cdown + (size_t)tgt * a.alpha;
+  // run: terms of one reduction (their sum below m 2^64); fl: terms whose middle products
+  // stay below 2^63 (source + m + 2^33 each), or 2^64 where the reduction folds them first
+  const int run = PRO == PRO_UP ? a.run_up : a.run_down;
+  const int fl = min(run, cls == CLS_FAST && run >= (1 << 13) ? 1 << 10 : run >= 16 ? 3 : 1);
+  const int rcls = run < 16 ? CLS_EXACT : cls;  // a modulus or a source above 2^60
+  const uint32_t inv = 0u - (uint32_t)mi.minv;
+  src += (size_t)i0 << LOGN;
+  constexpr int H = 4;  // points per batch (bounds the live registers)
+#pragma unroll
+  for (int h = 0; h < 8; h += H) {
+    Mac3 s[H] = {};
+    u64 x[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) x[k] = src[(size_t)C0::point(t, h + k) << LOGB];
+    u64 c = __ldg(cst);
+    bool one = true;  // no reduction yet
+    int left = run, fold = fl;
+#pragma unroll 1
+    for (int i = 0; i < ns; ++i) {
+      u64 xn[H], cn = 0;
+      if (i + 1 < ns) {  // the next limb's loads before this one's products (two limbs
+                         // ahead measured the same)
+        const u64 *sn = src + ((size_t)(i + 1) << LOGN);
+#pragma unroll
+        for (int k = 0; k < H; ++k) xn[k] = sn[(size_t)C0::point(t, h + k) << LOGB];
+        cn = __ldg(cst + i + 1);
+      }
+#pragma unroll
+      for (int k = 0; k < H; ++k) s[k].add(x[k], c);
+      --left;
+      if (--fold == 0 || left == 0 || i == ns - 1) {
+        fold = fl;
+        if (left == 0 || i == ns - 1) {
+          left = run;
+#pragma unroll
+          for (int k = 0; k < H; ++k) {
+            const u64 z = mac_reduce(s[k], mi, m, inv, rcls);
+            v[h + k] = one ? z : csub(v[h + k] + z, m);
+            s[k] = Mac3{};
+          }
+          one = false;
+        } else {
+#pragma unroll
+          for (int k = 0; k < H; ++k) s[k].fold();
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < H; ++k) x[k] = xn[k];
+      c = cn;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Forward column pass: the integer basis conversion of a task (PRO_UP, PRO_DOWN) or a plain
 // load (PRO_LOAD, in place), then the first forward NTT pass on the thread's eight points.
-// The conversion's sums are exact (Mac3), four points at a time, and reduced in registers;
-// the tile in shared memory is only the NTT's exchange. Bound by the integer pipe.
+// The conversion ends in registers; the tile in shared memory is only the NTT's exchange.
+// Bound by the integer pipe.
 template <int LOGN, int PRO>
 __global__ void __launch_bounds__(FwdColGeo<LOGN>::GP, 768 / FwdColGeo<LOGN>::GP)
     k_fwd_col2(KArgs a, JobSet js, WsOff wo, Tasks tk, int buf) {
@@ -292,66 +360,12 @@ __global__ void __launch_bounds__(FwdColGeo<LOGN>::GP, 768 / FwdColGeo<LOGN>::GP
   dst += ((size_t)task_slot(w) << LOGN) + c0 + g;
   u64 v[CG::E];
   if constexpr (PRO == PRO_LOAD) {
-    pdl_wait();
+    pdl_wait(a.early);
 #pragma unroll
     for (int r = 0; r < CG::E; ++r) v[r] = dst[(size_t)C0::point(t, r) << CG::LOGB];
   } else {
-    // sources: digit dig's limbs of v, or polynomial dig's P-limbs of vp
-    const int i0 = dig * (PRO == PRO_UP ? a.alpha : a.np);
-    const int ns = PRO == PRO_UP ? min(a.nq, i0 + a.alpha) - i0 : a.np;
-    const u64 *cst = PRO == PRO_UP ? a.tab.cup + ((size_t)dig * a.qp + tgt) * a.alpha
-                                   : a.tab.cdown + (size_t)tgt * a.alpha;
-    // run: terms of one reduction (their sum below m 2^64); fl: terms whose middle products
-    // stay below 2^63: source + m + 2^33 each
-    const int run = PRO == PRO_UP ? a.run_up : a.run_down;
-    const int fl = min(run, cls == CLS_FAST && run >= (1 << 13) ? 1 << 10 : run >= 16 ? 3 : 1);
-    const bool exact = cls == CLS_EXACT || run < 16;  // a modulus or source above 2^60
-    const uint32_t inv = 0u - (uint32_t)mi.minv;
-    src += ((size_t)i0 << LOGN) + c0 + g;
-    pdl_wait();
-    constexpr int H = 4;  // points per batch (bounds the live registers)
-#pragma unroll
-    for (int h = 0; h < CG::E; h += H) {
-      Mac3 s[H] = {};
-      u64 x[H];
-#pragma unroll
-      for (int k = 0; k < H; ++k) x[k] = src[(size_t)C0::point(t, h + k) << CG::LOGB];
-      u64 c = __ldg(cst);
-      bool one = true;  // no reduction yet
-      int left = run, fold = fl;
-#pragma unroll 1
-      for (int i = 0; i < ns; ++i) {
-        u64 xn[H], cn = 0;
-        if (i + 1 < ns) {  // the next limb's loads before this one's products
-          const u64 *sn = src + ((size_t)(i + 1) << LOGN);
-#pragma unroll
-          for (int k = 0; k < H; ++k) xn[k] = sn[(size_t)C0::point(t, h + k) << CG::LOGB];
-          cn = __ldg(cst + i + 1);
-        }
-#pragma unroll
-        for (int k = 0; k < H; ++k) s[k].add(x[k], c);
-        --left;
-        if (--fold == 0 || left == 0 || i == ns - 1) {
-          fold = fl;
-          if (left == 0 || i == ns - 1) {
-            left = run;
-#pragma unroll
-            for (int k = 0; k < H; ++k) {
-              const u64 z = mac_reduce(s[k], mi, m, inv, exact ? CLS_EXACT : cls);
-              v[h + k] = one ? z : csub(v[h + k] + z, m);
-              s[k] = Mac3{};
-            }
-            one = false;
-          } else {
-#pragma unroll
-            for (int k = 0; k < H; ++k) s[k].fold();
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < H; ++k) x[k] = xn[k];
-        c = cn;
-      }
-    }
+    pdl_wait(a.early);
+    bconv_points<PRO, LOGN>(v, a, tgt, dig, src + c0 + g, t, cls);
   }
   __syncthreads();  // the barrier's initialisation
   tw_ready<true>(&twbar, a.tab.err);
@@ -387,7 +401,7 @@ __global__ void __launch_bounds__(64)
   const ModInfo &mi = a.tab.mod[p];
   const u64 m = mi.m, mu = mi.mu;
   stage_row_tw<RG>(tws, a.tab.twr_f, p, blk, &twbar);
-  pdl_wait();
+  pdl_wait(a.early);
   u64 *b = dst + ((size_t)task_slot(w) << LOGN);
   u64 v[SB::E];
 #pragma unroll
@@ -424,6 +438,101 @@ __global__ void __launch_bounds__(64)
 constexpr int kKmDigits = 10;   // most digits of a tile held in shared memory
 constexpr int kKmGroups = 4;    // most groups of threads (one tile each)
 
+// The multiply phase of a key multiply: for every point e of a tile (`words` points),
+//   acc_c[e] (+)= sum_j ext_j[e] * key_jc[e],  c = 0, 1, over n digits.
+// ext: digit tiles in shared memory, `tilew` words apart, rows of 2^LOGB points at a pitch
+// of RP; kp: the tile's key words of digit 0, polynomial 0, polynomials cst words apart
+// (digits 2 cst); o: accumulators, polynomials oc1 words apart; first: write, else add.
+// One loop of (pair of points, digit) steps. The next step's key words (and at a new pair
+// the old accumulators) are loaded before a step's products, the first ones before
+// ready(), the barrier after which ext may be read.
+template <int LOGB, int RP, class READY>
+__device__ __forceinline__ void mac_tile(const KArgs &a, const ModInfo &mi, const u64 *ext,
+                                         int tilew, int n, int words, const u64 *kp, size_t cst,
+                                         u64 *o, size_t oc1, bool first, int cls, READY ready) {
+  const u64 m = mi.m, pol = l2_stream();
+  const uint32_t inv = 0u - (uint32_t)mi.minv;
+  const int bd = blockDim.x, fl = mac_terms(cls);
+  kp += 2 * threadIdx.x;
+  o += 2 * threadIdx.x;
+  ulonglong2 na = {}, nb = {}, no0 = {}, no1 = {}, old0 = {}, old1 = {};
+  if (2 * threadIdx.x < words) {
+    na = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp), pol);
+    nb = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp + cst), pol);
+    if (!first) {
+      no0 = *reinterpret_cast<const ulonglong2 *>(o);
+      no1 = *reinterpret_cast<const ulonglong2 *>(o + oc1);
+    }
+  }
+  ready();
+  Mac3 s[4] = {};
+  int jj = 0, fold = fl;
+  for (int e = 2 * threadIdx.x; e < words;) {
+    const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(
+        ext + jj * tilew + (e >> LOGB) * RP + core::row_pos(e & ((1 << LOGB) - 1)));
+    const ulonglong2 ka = na, kb = nb;
+    if (jj == 0) old0 = no0, old1 = no1;
+    const bool last = jj == n - 1;
+    kp += last ? (long long)(2 * bd) - (long long)((n - 1) * 2 * cst) : (long long)(2 * cst);
+    if (!last || e + 2 * bd < words) {
+      na = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp), pol);
+      nb = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp + cst), pol);
+      if (last && !first) {
+        no0 = *reinterpret_cast<const ulonglong2 *>(o + 2 * bd);
+        no1 = *reinterpret_cast<const ulonglong2 *>(o + 2 * bd + oc1);
+      }
+    }
+    s[0].add(y.x, ka.x);
+    s[1].add(y.y, ka.y);
+    s[2].add(y.x, kb.x);
+    s[3].add(y.y, kb.y);
+    if (last) {
+      u64 r[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        r[i] = mac_reduce(s[i], mi, m, inv, cls);
+        s[i] = Mac3{};
+      }
+      if (!first) {
+        r[0] = addmod(r[0], old0.x, m);
+        r[1] = addmod(r[1], old0.y, m);
+        r[2] = addmod(r[2], old1.x, m);
+        r[3] = addmod(r[3], old1.y, m);
+      }
+      *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(r[0], r[1]);
+      *reinterpret_cast<ulonglong2 *>(o + oc1) = make_ulonglong2(r[2], r[3]);
+      o += 2 * bd;
+      e += 2 * bd;
+      jj = 0;
+      fold = fl;
+    } else {
+      ++jj;
+      if (--fold == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[i].fold();
+        fold = fl;
+      }
+    }
+  }
+}
+
+// Own digit's tile: the warp's rows of the input in Montgomery form, into their shared rows.
+template <class RG>
+__device__ __forceinline__ void own_rows(u64 *ws, const u64 *dt, const ModInfo &mi, bool lazy) {
+  const u64 m = mi.m, r1 = mi.r1, r1s = mi.r1s;
+  warp_rows<RG>([&](int e, int p) {
+    ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(dt + e);
+    if (lazy) {
+      x.x = shoup4(x.x, r1, r1s, m);  // [0, 4m)
+      x.y = shoup4(x.y, r1, r1s, m);
+    } else {
+      x.x = csub(shoup(x.x, r1, r1s, m), m);
+      x.y = csub(shoup(x.y, r1, r1s, m), m);
+    }
+    *reinterpret_cast<ulonglong2 *>(ws + p) = x;
+  });
+}
+
 // A warp per digit's tile of two 256-point rows (one of 512) at N >= 2^16, two warps per
 // tile of 512 points below: small CTAs, so that several of them mix their transform and
 // multiply phases on an SM. (Several tiles per CTA at one or two digits: 21 -> 23 us per
@@ -447,7 +556,6 @@ __global__ void __launch_bounds__(km_gp(LOGN) * kKmGroups, 768 / (km_gp(LOGN) * 
   const int tgt = tk.t0 + (gridDim.y - 1 - blockIdx.y);
   const ModInfo &mi = a.tab.mod[tgt];
   const u64 m = mi.m;
-  const uint32_t inv = 0u - (uint32_t)mi.minv;  // m^-1 mod 2^32
   const int blk = blockIdx.x, off0 = blk * RG::TILE;
   const int od = tgt < a.nq ? tgt / a.alpha : -1;  // the target's own digit
   const int nd = tk.j1 - tk.j0;
@@ -456,10 +564,10 @@ __global__ void __launch_bounds__(km_gp(LOGN) * kKmGroups, 768 / (km_gp(LOGN) * 
   for (int k = threadIdx.x; k < 2 * nd; k += blockDim.x)
     prefetch_l2(evk + ((size_t)((2 * tk.j0 + k) * a.eqp) << LOGN), RG::TILE * 8);
   stage_row_tw<RG>(tws, a.tab.twr_f, tgt, blk, &twbar);
-  const int cls = mod_class(m), fl = mac_terms(cls);
+  const int cls = mod_class(m);
   // ext stays lazy when the exact digit sum of its products fits one reduction
   const bool lazy = cls == CLS_FAST && __umul64hi(kFwdLazy * min(nd, ds), m) == 0;
-  pdl_wait();
+  pdl_wait(a.early);
   __syncthreads();  // the twiddle barrier's initialisation
   for (int c0 = tk.j0; c0 < tk.j1; c0 += ds) {
     const int n = min(ds, tk.j1 - c0);
@@ -471,19 +579,7 @@ __global__ void __launch_bounds__(km_gp(LOGN) * kKmGroups, 768 / (km_gp(LOGN) * 
       u64 *ex = ext + jx * RG::TILEW;
       if (has && jx == oc) {
         const u64 *dt = jp.d + ((size_t)tgt << LOGN) + off0 + (w0 << RG::LOGB);
-        u64 *ws = ex + w0 * RG::RP;
-        const u64 r1 = mi.r1, r1s = mi.r1s;
-        warp_rows<RG>([&](int e, int p) {
-          ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(dt + e);
-          if (lazy) {
-            x.x = shoup4(x.x, r1, r1s, m);  // [0, 4m)
-            x.y = shoup4(x.y, r1, r1s, m);
-          } else {
-            x.x = csub(shoup(x.x, r1, r1s, m), m);
-            x.y = csub(shoup(x.y, r1, r1s, m), m);
-          }
-          *reinterpret_cast<ulonglong2 *>(ws + p) = x;
-        });
+        own_rows<RG>(ex + w0 * RG::RP, dt, mi, lazy);
         continue;
       }
       const int j = c0 + jx;
@@ -504,74 +600,14 @@ __global__ void __launch_bounds__(km_gp(LOGN) * kKmGroups, 768 / (km_gp(LOGN) * 
       __syncwarp();
       core::put_row<SB>(s, v, t);
     }
-    // Multiply: this thread's pairs of points in turn, each over the turn's digits, as one
-    // loop of (pair, digit) steps. The next step's key words (and at a new pair the old
-    // accumulators) are loaded before a step's products, the first ones before the barrier.
-    const u64 pol = l2_stream();
-    const bool first = tk.first && c0 == tk.j0;
-    const size_t cst = (size_t)a.eqp << LOGN;  // words between a digit's two polynomials
-    const int bd = blockDim.x;
-    const u64 *kp = evk + c0 * 2 * cst + 2 * threadIdx.x;
-    u64 *o = jp.ws + wo.acc + ((size_t)tgt << LOGN) + off0 + 2 * threadIdx.x;
-    const size_t oc1 = (size_t)a.qp << LOGN;  // to polynomial 1's accumulators
-    ulonglong2 na = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp), pol);
-    ulonglong2 nb = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp + cst), pol);
-    ulonglong2 no0 = {}, no1 = {}, old0 = {}, old1 = {};
-    if (!first) {
-      no0 = *reinterpret_cast<const ulonglong2 *>(o);
-      no1 = *reinterpret_cast<const ulonglong2 *>(o + oc1);
-    }
-    __syncthreads();
-    tw_ready<true>(&twbar, a.tab.err);  // (a CTA with no digit to transform, too)
-    Mac3 s[4] = {};
-    int jj = 0, fold = fl;
-    for (int e = 2 * threadIdx.x; e < RG::TILE;) {
-      const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(
-          ext + jj * RG::TILEW + (e >> RG::LOGB) * RG::RP + core::row_pos(e & (RG::N2 - 1)));
-      const ulonglong2 ka = na, kb = nb;
-      if (jj == 0) old0 = no0, old1 = no1;
-      const bool last = jj == n - 1;
-      kp += last ? (long long)(2 * bd) - (long long)((n - 1) * 2 * cst) : (long long)(2 * cst);
-      if (!last || e + 2 * bd < RG::TILE) {
-        na = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp), pol);
-        nb = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp + cst), pol);
-        if (last && !first) {
-          no0 = *reinterpret_cast<const ulonglong2 *>(o + 2 * bd);
-          no1 = *reinterpret_cast<const ulonglong2 *>(o + 2 * bd + oc1);
-        }
-      }
-      s[0].add(y.x, ka.x);
-      s[1].add(y.y, ka.y);
-      s[2].add(y.x, kb.x);
-      s[3].add(y.y, kb.y);
-      if (last) {
-        u64 r[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          r[i] = mac_reduce(s[i], mi, m, inv, cls);
-          s[i] = Mac3{};
-        }
-        if (!first) {
-          r[0] = addmod(r[0], old0.x, m);
-          r[1] = addmod(r[1], old0.y, m);
-          r[2] = addmod(r[2], old1.x, m);
-          r[3] = addmod(r[3], old1.y, m);
-        }
-        *reinterpret_cast<ulonglong2 *>(o) = make_ulonglong2(r[0], r[1]);
-        *reinterpret_cast<ulonglong2 *>(o + oc1) = make_ulonglong2(r[2], r[3]);
-        o += 2 * bd;
-        e += 2 * bd;
-        jj = 0;
-        fold = fl;
-      } else {
-        ++jj;
-        if (--fold == 0) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) s[i].fold();
-          fold = fl;
-        }
-      }
-    }
+    mac_tile<RG::LOGB, RG::RP>(
+        a, mi, ext, RG::TILEW, n, RG::TILE, evk + (((size_t)(2 * c0) * a.eqp) << LOGN),
+        (size_t)a.eqp << LOGN, jp.ws + wo.acc + ((size_t)tgt << LOGN) + off0,
+        (size_t)a.qp << LOGN, tk.first && c0 == tk.j0, cls,
+        [&] {
+          __syncthreads();
+          tw_ready<true>(&twbar, a.tab.err);  // (a CTA with no digit to transform, too)
+        });
     if (c0 + ds < tk.j1) __syncthreads();  // ext is free for the next turn
   }
   pdl_trigger();
@@ -605,7 +641,7 @@ __global__ void __launch_bounds__(128, 6)
   const int cls = mod_class(m);
   const bool fast = cls == CLS_FAST;
   const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
-  pdl_wait();
+  pdl_wait(a.early);
   const size_t woff = (size_t)(r0 + w0) << RG::LOGB;  // the warp's rows
   const u64 *ac = jp.ws + wo.acc + ((size_t)c * a.qp + i) * N + woff;
   u64 v[SB::E];
@@ -671,15 +707,15 @@ struct RowFns {
                               cudaStream_t s) {
     const int inner = which == 0 ? c->nq : c->np, tiles = which + 1;
     if (inner == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_inv_row2<LOGN>, dim3(RG::GRID, inner, js.n), dim3(RG::GP * tiles),
-                      smem_row(tiles), s, args_of(c), js, wo, which);
+    return launch_rule(k_inv_row2<LOGN>, dim3(RG::GRID, inner, js.n), dim3(RG::GP * tiles),
+                      smem_row(tiles), s, c, js, wo, which);
   }
   static cudaError_t col(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
                          int pieces, cudaStream_t s) {
     const int inner = which == 0 ? c->nq : c->np, tiles = which + 1;
     if (inner == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_inv_col2<LOGN>, dim3(CG::GRID, inner, js.n), dim3(CG::GP * tiles),
-                      smem_col(tiles), s, args_of(c), js, wo, which, pieces);
+    return launch_rule(k_inv_col2<LOGN>, dim3(CG::GRID, inner, js.n), dim3(CG::GP * tiles),
+                      smem_col(tiles), s, c, js, wo, which, pieces);
   }
   static cudaError_t intt_col(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
                               cudaStream_t s) {
@@ -694,8 +730,8 @@ struct RowFns {
                              const Tasks &tk, int buf, cudaStream_t s) {
     const int n = count_tasks(c, tk);
     if (n == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_fwd_col2<LOGN, PRO>, dim3(FG::GRID, n, js.n), dim3(FG::GP), FG::SMEM, s,
-                      args_of(c), js, wo, tk, buf);
+    return launch_rule(k_fwd_col2<LOGN, PRO>, dim3(FG::GRID, n, js.n), dim3(FG::GP), FG::SMEM, s,
+                      c, js, wo, tk, buf);
   }
   static cudaError_t modup_col(const ks_context *c, const JobSet &js, const WsOff &wo,
                                const Tasks &tk, cudaStream_t s) {
@@ -714,23 +750,23 @@ struct RowFns {
     const int n = count_tasks(c, tk), nd = tk.j1 - tk.j0;
     if (n == 0 || js.n == 0 || nd < 1) return cudaSuccess;
     const int turns = (nd + kKmDigits - 1) / kKmDigits, ds = (nd + turns - 1) / turns;
-    return launch_pdl(k_keymult2<LOGN>, dim3(KG::GRID, n, js.n),
+    return launch_rule(k_keymult2<LOGN>, dim3(KG::GRID, n, js.n),
                       dim3(KG::GP * std::min(ds, kKmGroups)), smem_km(ds), s,
-                      args_of(c), js, wo, tk, ds);
+                      c, js, wo, tk, ds);
   }
   static cudaError_t moddown_row(const ks_context *c, const JobSet &js, const WsOff &wo,
                                  const Tasks &tk, cudaStream_t s) {
     const int n = count_tasks(c, tk);
     if (n == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_moddown2<LOGN>, dim3(RG::GRID, n, js.n), dim3(RG::GP * 2), smem_row(2), s,
-                      args_of(c), js, wo, tk);
+    return launch_rule(k_moddown2<LOGN>, dim3(RG::GRID, n, js.n), dim3(RG::GP * 2), smem_row(2), s,
+                      c, js, wo, tk);
   }
   static cudaError_t ntt_row(const ks_context *c, const JobSet &js, const WsOff &wo,
                              const Tasks &tk, int buf, cudaStream_t s) {
     const int n = count_tasks(c, tk);
     if (n == 0 || js.n == 0) return cudaSuccess;
-    return launch_pdl(k_row_store2<LOGN>, dim3(RG::GRID, n, js.n), dim3(RG::GP), smem_row(1), s,
-                      args_of(c), js, wo, tk, buf);
+    return launch_rule(k_row_store2<LOGN>, dim3(RG::GRID, n, js.n), dim3(RG::GP), smem_row(1), s,
+                      c, js, wo, tk, buf);
   }
   static const LaunchTable &table() {
     static const LaunchTable t = {&prepare,     &count_tasks, &intt_row,  &intt_col,
@@ -740,7 +776,7 @@ struct RowFns {
   }
 };
 
-// Launchers of a single-pass size (N <= 2^12): the shared-memory tile rounds of radix RL.
+// Launchers of a single-pass size (N <= 2^11): the shared-memory tile rounds of radix RL.
 template <int LOGN, int RL>
 struct LaunchOne {
   using GTR = GeoT<LOGN, RL, 1>;

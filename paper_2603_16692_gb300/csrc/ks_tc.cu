@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(TcGeo<LOGN, GRP>::NT + 64, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tm_slot;
-  pdl_wait();
+  pdl_wait(a.early);
 
   auto target = [&](const TcItem &x, int u) { return decode(a, tk, x.y0 + min(u, x.cnt - 1)); };
   if (warp == CW + 1) {
@@ -442,11 +442,14 @@ cudaError_t launch_one(const ks_context *c, const JobSet &js, const WsOff &wo, c
   constexpr int GRP = kTcGroups;
   using G = TcGeo<LOGN, GRP>;
   const int smem = G::smem(c->tc_ap);
+  KArgs a = args_of(c);
+  // one CTA per SM; the dependent row pass has about this launch's points
+  a.early = early_rule((size_t)ti.items * js.n * (kTcTargets * G::TP / 8));
   if (up)
     return launch_pdl(k_bconv_tc<LOGN, PRO_UP, GRP>, dim3(grid, 1, js.n), dim3(G::NT + 64), smem,
-                      s, args_of(c), js, wo, tk, ti);
+                      s, a, js, wo, tk, ti);
   return launch_pdl(k_bconv_tc<LOGN, PRO_DOWN, GRP>, dim3(grid, 1, js.n), dim3(G::NT + 64), smem,
-                    s, args_of(c), js, wo, tk, ti);
+                    s, a, js, wo, tk, ti);
 }
 
 }  // namespace kern
