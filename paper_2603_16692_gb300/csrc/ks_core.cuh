@@ -22,10 +22,13 @@
 namespace ks {
 namespace core {
 
-// log2 of the points per thread of the row pass (rows of 128 points at N = 2^13 and 2^14,
-// 256 at 2^15 and 2^16, 512 at 2^17): 8 up to 2^15, where a launch is a wave or two and
-// twice the threads shorten each one's serial work ...
-__host__ __device__ constexpr int row_rl(int logn) { return logn >= 16 ? 4 : 3; }
+// log2 of the points per thread of the row pass (rows of 64 points at N = 2^12, 128 at 2^13
+// and 2^14, 256 at 2^15 and 2^16, 512 at 2^17). 16 points halve the exchange traffic and the
+// instructions around it, but half the threads with 80 registers instead of 64 wait longer
+// on memory: at N = 2^16 8 points took (4, 2^16, 35) in four chunks from 674 to 604 us and
+// (4, 2^16, 13 limbs up) from 167 to 160, (4, 2^16, 35) 346 -> 348; rows of 512 points do
+// not fit a warp at 8.
+__host__ __device__ constexpr int row_rl(int logn) { return logn >= 17 ? 4 : 3; }
 // ... and of the column pass (columns of 64, 128, 128, 256, 256 points).
 __host__ __device__ constexpr int col_rl(int logn) { return geo_loga(logn) == 8 ? 4 : 3; }
 
@@ -380,6 +383,7 @@ __device__ __forceinline__ void col_fwd(u64 *v, u64 *s, const ulonglong2 *tw, u6
     col_fwd<LOGM, RL, GC, CLS, K + 1>(v, s, tw, m, t, g, sync);
   }
 }
+
 // Words of a column tile's exchange buffer.
 template <int LOGM, int GC, int RL>
 __host__ __device__ constexpr int col_words() {

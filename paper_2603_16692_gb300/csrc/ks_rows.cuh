@@ -27,6 +27,10 @@ struct RowGeo {
   static_assert(SB::T <= 32, "a row inside a warp");
 };
 
+// CTAs of 128 threads per SM that the row kernels' registers leave room for: 64 registers
+// at 8 points per thread, 80 at 16 (which spills at 64).
+__host__ __device__ constexpr int row_blocks(int logn) { return core::row_rl(logn) == 3 ? 8 : 6; }
+
 // The twiddle slab of (prime, row tile) by one bulk copy (see stage_tw); tw_ready waits.
 template <class RG>
 __device__ __forceinline__ void stage_row_tw(ulonglong2 *tws, const ulonglong2 *tab, int prime,
@@ -79,7 +83,7 @@ __device__ __forceinline__ void warp_rows(F f) {
 // output for the column pass. Bound by the integer pipe and the twiddle slab's traffic
 // (16 bytes per point against 8 in and 8 out).
 template <int LOGN>
-__global__ void __launch_bounds__(128, 6)
+__global__ void __launch_bounds__(128, row_blocks(LOGN))
     k_inv_row2(KArgs a, JobSet js, WsOff wo, int which) {
   using RG = RowGeo<LOGN>;
   using SB = typename RG::SB;
@@ -533,16 +537,15 @@ __device__ __forceinline__ void own_rows(u64 *ws, const u64 *dt, const ModInfo &
   });
 }
 
-// A warp per digit's tile of two 256-point rows (one of 512) at N >= 2^16, two warps per
-// tile of 512 points below: small CTAs, so that several of them mix their transform and
-// multiply phases on an SM. (Several tiles per CTA at one or two digits: 21 -> 23 us per
-// digit launch of (4, 2^16, 35) in four chunks, not kept.)
-__host__ __device__ constexpr int km_gp(int logn) { return logn >= 16 ? 32 : 64; }
+// A tile is one warp's rows (one row of 256 or 512 points, two of 128): small CTAs, so that
+// several of them mix their transform and multiply phases on an SM (tiles of two warps:
+// (4, 2^16, 35) 346 -> 341 us, (8, 2^16, 15) 239 -> 234).
+constexpr int kKmGp = 32;
 
 template <int LOGN>
-__global__ void __launch_bounds__(km_gp(LOGN) * kKmGroups, 768 / (km_gp(LOGN) * kKmGroups))
+__global__ void __launch_bounds__(kKmGp * kKmGroups, 768 / (kKmGp * kKmGroups))
     k_keymult2(KArgs a, JobSet js, WsOff wo, Tasks tk, int ds) {
-  using RG = RowGeo<LOGN, km_gp(LOGN)>;
+  using RG = RowGeo<LOGN, kKmGp>;
   using SB = typename RG::SB;
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ u64 twbar;
@@ -619,7 +622,7 @@ __global__ void __launch_bounds__(km_gp(LOGN) * kKmGroups, 768 / (km_gp(LOGN) * 
 // the two polynomials of limb i side by side in two groups of 64 threads that share the
 // twiddle slab; each warp finishes its own rows (no block barrier after the start).
 template <int LOGN>
-__global__ void __launch_bounds__(128, 6)
+__global__ void __launch_bounds__(128, row_blocks(LOGN))
     k_moddown2(KArgs a, JobSet js, WsOff wo, Tasks tk) {
   using RG = RowGeo<LOGN>;
   using SB = typename RG::SB;
@@ -685,7 +688,7 @@ __global__ void __launch_bounds__(128, 6)
 template <int LOGN>
 struct RowFns {
   using RG = RowGeo<LOGN>;
-  using KG = RowGeo<LOGN, km_gp(LOGN)>;  // the key multiply's tile
+  using KG = RowGeo<LOGN, kKmGp>;  // the key multiply's tile
   using CG = ColGeo<LOGN>;
   using FG = FwdColGeo<LOGN>;
   static constexpr int smem_row(int tiles) { return RG::TW_BYTES + tiles * RG::TILEW * 8; }
@@ -751,8 +754,7 @@ struct RowFns {
     if (n == 0 || js.n == 0 || nd < 1) return cudaSuccess;
     const int turns = (nd + kKmDigits - 1) / kKmDigits, ds = (nd + turns - 1) / turns;
     return launch_rule(k_keymult2<LOGN>, dim3(KG::GRID, n, js.n),
-                      dim3(KG::GP * std::min(ds, kKmGroups)), smem_km(ds), s,
-                      c, js, wo, tk, ds);
+                       dim3(KG::GP * std::min(ds, kKmGroups)), smem_km(ds), s, c, js, wo, tk, ds);
   }
   static cudaError_t moddown_row(const ks_context *c, const JobSet &js, const WsOff &wo,
                                  const Tasks &tk, cudaStream_t s) {

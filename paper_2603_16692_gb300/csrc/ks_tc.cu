@@ -100,17 +100,14 @@ __device__ __forceinline__ void tc_commit(u64 *bar) {
           smem_u32(bar))
       : "memory");
 }
-// 16 consecutive 32-bit columns of the warp's lane (TMEM lane = warp quadrant * 32 +
-// lane); complete after tmem_wait_ld.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
+// 8 consecutive 32-bit columns of the warp's lane (TMEM lane = warp quadrant * 32 + lane);
+// complete after tmem_wait_ld.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -381,42 +378,44 @@ __global__ void __launch_bounds__(TcGeo<LOGN, GRP>::NT + 64, 1)
       const int cnt = info_cnt[group][b], xtile = info_tile[group][b];
       if (!mbar_wait(&bar_m[group], k & 1)) atomicExch(a.tab.err, 1);
       tc_fence_after();
-      u64 z[2][G::PTS];
+      // One target after the other, over one copy of the code (both at once, with the
+      // second's points held in registers meanwhile, is twice the instructions of a loop
+      // that has to stay in the instruction cache).
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i) {
+        const u64 m = i ? mm[1] : mm[0], mc = m - kTcBias;
+        const uint32_t wi = i ? w[1] : w[0], iv = i ? inv[1] : inv[0];
+        u64 v[G::PTS];
 #pragma unroll
-      for (int b0 = 0; b0 < G::MB; b0 += 2) {
-        uint32_t v[2][16];
+        for (int b0 = 0; b0 < G::MB; b0 += 4) {
+          uint32_t r[4][8];
 #pragma unroll
-        for (int bb = 0; bb < 2; ++bb)
-          tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + group * G::DCOLS +
-                        (b0 + bb) * 8 * kTcTargets + half * 16,
-                    v[bb]);
-        tmem_wait_ld();
-        if (b0 + 2 == G::MB) {  // the warp's last reads of the accumulator
+          for (int bb = 0; bb < 4; ++bb)
+            tmem_ld8(tmem + ((uint32_t)(32 * q) << 16) + group * G::DCOLS +
+                         (b0 + bb) * 8 * kTcTargets + half * 16 + i * 8,
+                     r[bb]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int bb = 0; bb < 4; ++bb) v[b0 + bb] = tc_reduce(r[bb], m, iv, mc);
+        }
+        if (i == 1) {  // the warp's last reads of the accumulator
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&bar_tm[group]);
         }
-#pragma unroll
-        for (int bb = 0; bb < 2; ++bb)
-#pragma unroll
-          for (int i = 0; i < 2; ++i)
-            z[i][b0 + bb] = tc_reduce(v[bb] + 8 * i, mm[i], inv[i], mm[i] - kTcBias);
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        if (2 * half + i >= cnt) break;
-        const int t = task_limb(w[i]), cls = mod_class(mm[i]);
+        if (2 * half + i >= cnt) continue;
+        const int t = task_limb(wi), cls = mod_class(m);
         const ulonglong2 *tw = a.tab.twc_f + ((size_t)t << G::LOGA);
         if (cls == CLS_FAST)
-          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_FAST, 0>(z[i], tile, tw, mm[i], ct, cg, sync);
+          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_FAST, 0>(v, tile, tw, m, ct, cg, sync);
         else if (cls == CLS_MID)
-          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_MID, 0>(z[i], tile, tw, mm[i], ct, cg, sync);
+          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_MID, 0>(v, tile, tw, m, ct, cg, sync);
         else
-          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_EXACT, 0>(z[i], tile, tw, mm[i], ct, cg, sync);
+          core::col_fwd<G::LOGA, G::RL, G::GC, CLS_EXACT, 0>(v, tile, tw, m, ct, cg, sync);
         using CL = core::ColRound<G::LOGA, G::RL, core::col_rounds<G::LOGA, G::RL>() - 1>;
-        u64 *d = dst + ((size_t)task_slot(w[i]) << LOGN) + xtile * G::GC + cg;
+        u64 *d = dst + ((size_t)task_slot(wi) << LOGN) + xtile * G::GC + cg;
 #pragma unroll
-        for (int r = 0; r < G::PTS; ++r) d[(size_t)CL::point(ct, r) << G::LOGB] = z[i][r];
+        for (int r = 0; r < G::PTS; ++r) d[(size_t)CL::point(ct, r) << G::LOGB] = v[r];
         sync();  // the tile is free for the next target
       }
     }
