@@ -324,7 +324,9 @@ __host__ __device__ constexpr int col_rounds() {
 }
 
 // Inverse column transform of column g of a tile of GC columns (tw: the column table, entry
-// 2^ls + c). In: v[r] = point ColRound<last>::point(t, r). Out: v[u] = point u T + t.
+// 2^ls + c). In: v[r] = point ColRound<last>::point(t, r), below 4m (fast; so the biases are
+// four times a canonical start's, and the outputs below 2^(LOGM + 3) m), 8m (mid) or 2m
+// (exact). Out: v[u] = point u T + t.
 // sync(): barrier of the tile's threads.
 template <int LOGM, int RL, int GC, int CLS, int K, class SYNC>
 __device__ __forceinline__ void col_inv(u64 *v, u64 *s, const ulonglong2 *tw, u64 m, int t, int g,
@@ -340,7 +342,7 @@ __device__ __forceinline__ void col_inv(u64 *v, u64 *s, const ulonglong2 *tw, u6
   };
   if constexpr (LOGM == 2 * RL) {  // both rounds as one loop (see row_fwd)
     int h = (1 << RL) + C::hi(t, 0);  // entry of (stage q of the round, sub): (h << q) + sub
-    u64 mb = m;
+    u64 mb = 4 * m;
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
       round_inv<RL, 0, RL, 0, CLS, false>(
@@ -348,7 +350,7 @@ __device__ __forceinline__ void col_inv(u64 *v, u64 *s, const ulonglong2 *tw, u6
       if (k == 0) {
         exchange();
         h = 1;
-        mb = m << RL;
+        mb = m << (RL + 2);
       }
     }
   } else {
@@ -357,7 +359,7 @@ __device__ __forceinline__ void col_inv(u64 *v, u64 *s, const ulonglong2 *tw, u6
         [&](int q, int ex, int sub) {
           return tw[(1 << (C::LS0 + q)) + (C::hi(t, ex) << q) + sub];
         },
-        m);
+        4 * m);
     if constexpr (K > 0) {
       exchange();  // (the next one writes where this thread just read)
       col_inv<LOGM, RL, GC, CLS, K - 1>(v, s, tw, m, t, g, sync);

@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
   for (int u = 0; u < 8; ++u) {
     const int x = (u << FG::SB::LOGT) + t2;
     cluster_st(cluster_map(colbuf, x / FG::CC) + 8 * (core::col_pos<3>(y) * FG::CC + x % FG::CC),
-               reduce_full(v[u], m, mu));
+               inv_between(v[u], m, mu, cls));
   }
   cluster_arrive();
   cluster_wait();
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) k_fu_up(KArgs a, JobSet js, WsO
   for (int j = grp; j < a.beta; j += ngrp)
     if (j != od) fu_row<FG>(ext + j * FG::ROWW + row * FG::RP, twr + row * FG::N2, mi, m, cls, t2,
                             !lazy);
-  mac_tile<FG::LOGB, FG::RP>(a, mi, ext, FG::ROWW, a.beta, FG::PTS, evk, (size_t)a.eqp << LOGN,
+  mac_tile<FG::LOGB, FG::RP, true>(mi, ext, FG::ROWW, a.beta, FG::PTS, evk, (size_t)a.eqp << LOGN,
                              jp.ws + wo.acc + ((size_t)tgt << LOGN) + off0,
                              (size_t)a.qp << LOGN, true, cls, [] { __syncthreads(); });
   pdl_trigger();

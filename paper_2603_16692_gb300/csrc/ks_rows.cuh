@@ -77,6 +77,17 @@ __device__ __forceinline__ void warp_rows(F f) {
   }
 }
 
+// A value between the two inverse passes: the column pass starts from values below 4m
+// (fast; the row pass leaves them below 2^10 m), or takes the row pass's bounds as they are
+// (mid: 8m, exact: 2m). q = floor(x_hi floor(2^64 / m) / 2^32) is at most 3 below x / m when
+// m > 2^32; smaller fast moduli take the full reduction. One 32x32 product for the quotient
+// instead of a 64x64 one: six instructions a point against eighteen.
+__device__ __forceinline__ u64 inv_between(u64 x, u64 m, u64 mu, int cls) {
+  if (cls != CLS_FAST) return x;
+  if (mu >> 32) return reduce_full(x, m, mu);
+  return x - (u64)__umulhi((uint32_t)(x >> 32), (uint32_t)mu) * m;
+}
+
 // ---------------------------------------------------------------------------
 // Inverse row pass: d -> v (which 0, one polynomial) or the P-limbs of acc -> vp (which 1,
 // both polynomials, one group of 64 threads each, sharing the twiddle slab). Canonical
@@ -125,10 +136,11 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   u64 v[SB::E];
   u64 *s = tile + row * RG::RP;
   core::get_row<SB>(v, s, t);
-  row_inv_cls<RG>(v, s, tws + (size_t)(RG::GR - 1 - row) * RG::N2, m, t, mod_class(m));
+  const int cls = mod_class(m);
+  row_inv_cls<RG>(v, s, tws + (size_t)(RG::GR - 1 - row) * RG::N2, m, t, cls);
   u64 *d = is.dst + ((size_t)o * is.dst_outer + ii) * N + ((size_t)(r0 + row) << RG::LOGB);
 #pragma unroll
-  for (int u = 0; u < SB::E; ++u) d[(u << SB::LOGT) + t] = reduce_full(v[u], m, mu);
+  for (int u = 0; u < SB::E; ++u) d[(u << SB::LOGT) + t] = inv_between(v[u], m, mu, cls);
   if (host_in) pdl_wait(a.early);
   pdl_trigger();
 }
@@ -286,7 +298,7 @@ __device__ __forceinline__ void bconv_points(u64 *v, const KArgs &a, int tgt, in
   const int rcls = run < 16 ? CLS_EXACT : cls;  // a modulus or a source above 2^60
   const uint32_t inv = 0u - (uint32_t)mi.minv;
   src += (size_t)i0 << LOGN;
-  constexpr int H = 4;  // points per batch (bounds the live registers)
+  constexpr int H = 4;  // points per batch (eight spill: (2, 2^15, 10) 63 -> 72 us)
 #pragma unroll
   for (int h = 0; h < 8; h += H) {
     Mac3 s[H] = {};
@@ -446,14 +458,16 @@ constexpr int kKmGroups = 4;    // most groups of threads (one tile each)
 //   acc_c[e] (+)= sum_j ext_j[e] * key_jc[e],  c = 0, 1, over n digits.
 // ext: digit tiles in shared memory, `tilew` words apart, rows of 2^LOGB points at a pitch
 // of RP; kp: the tile's key words of digit 0, polynomial 0, polynomials cst words apart
-// (digits 2 cst); o: accumulators, polynomials oc1 words apart; first: write, else add.
+// (digits 2 cst); o: accumulators, polynomials oc1 words apart; first: write, else add (FIRST: always write,
+// without the old accumulators' registers).
 // One loop of (pair of points, digit) steps. The next step's key words (and at a new pair
 // the old accumulators) are loaded before a step's products, the first ones before
 // ready(), the barrier after which ext may be read.
-template <int LOGB, int RP, class READY>
-__device__ __forceinline__ void mac_tile(const KArgs &a, const ModInfo &mi, const u64 *ext,
-                                         int tilew, int n, int words, const u64 *kp, size_t cst,
-                                         u64 *o, size_t oc1, bool first, int cls, READY ready) {
+template <int LOGB, int RP, bool FIRST, class READY>
+__device__ __forceinline__ void mac_tile(const ModInfo &mi, const u64 *ext, int tilew, int n,
+                                         int words, const u64 *kp, size_t cst, u64 *o, size_t oc1,
+                                         bool first, int cls, READY ready) {
+  first = first || FIRST;
   const u64 m = mi.m, pol = l2_stream();
   const uint32_t inv = 0u - (uint32_t)mi.minv;
   const int bd = blockDim.x, fl = mac_terms(cls);
@@ -471,13 +485,16 @@ __device__ __forceinline__ void mac_tile(const KArgs &a, const ModInfo &mi, cons
   ready();
   Mac3 s[4] = {};
   int jj = 0, fold = fl;
+  auto pos = [&](int e) { return ext + (e >> LOGB) * RP + core::row_pos(e & ((1 << LOGB) - 1)); };
+  const u64 *yp = pos(2 * threadIdx.x);
   for (int e = 2 * threadIdx.x; e < words;) {
-    const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(
-        ext + jj * tilew + (e >> LOGB) * RP + core::row_pos(e & ((1 << LOGB) - 1)));
+    const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(yp);
+    yp += tilew;
     const ulonglong2 ka = na, kb = nb;
     if (jj == 0) old0 = no0, old1 = no1;
     const bool last = jj == n - 1;
-    kp += last ? (long long)(2 * bd) - (long long)((n - 1) * 2 * cst) : (long long)(2 * cst);
+    kp += 2 * cst;
+    if (last) kp += 2 * bd - 2 * cst * n;
     if (!last || e + 2 * bd < words) {
       na = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp), pol);
       nb = ldg_pol(reinterpret_cast<const ulonglong2 *>(kp + cst), pol);
@@ -507,6 +524,7 @@ __device__ __forceinline__ void mac_tile(const KArgs &a, const ModInfo &mi, cons
       *reinterpret_cast<ulonglong2 *>(o + oc1) = make_ulonglong2(r[2], r[3]);
       o += 2 * bd;
       e += 2 * bd;
+      yp = pos(e);
       jj = 0;
       fold = fl;
     } else {
@@ -542,7 +560,7 @@ __device__ __forceinline__ void own_rows(u64 *ws, const u64 *dt, const ModInfo &
 // (4, 2^16, 35) 346 -> 341 us, (8, 2^16, 15) 239 -> 234).
 constexpr int kKmGp = 32;
 
-template <int LOGN>
+template <int LOGN, bool FIRST>
 __global__ void __launch_bounds__(kKmGp * kKmGroups, 768 / (kKmGp * kKmGroups))
     k_keymult2(KArgs a, JobSet js, WsOff wo, Tasks tk, int ds) {
   using RG = RowGeo<LOGN, kKmGp>;
@@ -603,8 +621,8 @@ __global__ void __launch_bounds__(kKmGp * kKmGroups, 768 / (kKmGp * kKmGroups))
       __syncwarp();
       core::put_row<SB>(s, v, t);
     }
-    mac_tile<RG::LOGB, RG::RP>(
-        a, mi, ext, RG::TILEW, n, RG::TILE, evk + (((size_t)(2 * c0) * a.eqp) << LOGN),
+    mac_tile<RG::LOGB, RG::RP, FIRST>(
+        mi, ext, RG::TILEW, n, RG::TILE, evk + (((size_t)(2 * c0) * a.eqp) << LOGN),
         (size_t)a.eqp << LOGN, jp.ws + wo.acc + ((size_t)tgt << LOGN) + off0,
         (size_t)a.qp << LOGN, tk.first && c0 == tk.j0, cls,
         [&] {
@@ -703,7 +721,8 @@ struct RowFns {
     if ((e = smem_attr(k_fwd_col2<LOGN, PRO_UP>, FG::SMEM))) return e;
     if ((e = smem_attr(k_fwd_col2<LOGN, PRO_DOWN>, FG::SMEM))) return e;
     if ((e = smem_attr(k_row_store2<LOGN>, smem_row(1)))) return e;
-    if ((e = smem_attr(k_keymult2<LOGN>, smem_km(kKmDigits)))) return e;
+    if ((e = smem_attr(k_keymult2<LOGN, true>, smem_km(kKmDigits)))) return e;
+    if ((e = smem_attr(k_keymult2<LOGN, false>, smem_km(kKmDigits)))) return e;
     return smem_attr(k_moddown2<LOGN>, smem_row(2));
   }
   static cudaError_t intt_row(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
@@ -717,8 +736,12 @@ struct RowFns {
                          int pieces, cudaStream_t s) {
     const int inner = which == 0 ? c->nq : c->np, tiles = which + 1;
     if (inner == 0 || js.n == 0) return cudaSuccess;
-    return launch_rule(k_inv_col2<LOGN>, dim3(CG::GRID, inner, js.n), dim3(CG::GP * tiles),
-                      smem_col(tiles), s, c, js, wo, which, pieces);
+    KArgs a = args_of(c);
+    const dim3 grid(CG::GRID, inner, js.n), block(CG::GP * tiles);
+    // writing bytes, the tensor-core kernel follows: one CTA per SM, which cannot crowd the
+    // SMs that this launch leaves empty ((4, 2^16, 35) 324 -> 317 us)
+    a.early = pieces || early_rule((size_t)grid.x * grid.y * grid.z * block.x);
+    return launch_pdl(k_inv_col2<LOGN>, grid, block, smem_col(tiles), s, a, js, wo, which, pieces);
   }
   static cudaError_t intt_col(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
                               cudaStream_t s) {
@@ -753,8 +776,10 @@ struct RowFns {
     const int n = count_tasks(c, tk), nd = tk.j1 - tk.j0;
     if (n == 0 || js.n == 0 || nd < 1) return cudaSuccess;
     const int turns = (nd + kKmDigits - 1) / kKmDigits, ds = (nd + turns - 1) / turns;
-    return launch_rule(k_keymult2<LOGN>, dim3(KG::GRID, n, js.n),
-                       dim3(KG::GP * std::min(ds, kKmGroups)), smem_km(ds), s, c, js, wo, tk, ds);
+    const dim3 grid(KG::GRID, n, js.n), block(KG::GP * std::min(ds, kKmGroups));
+    if (tk.first && turns == 1)
+      return launch_rule(k_keymult2<LOGN, true>, grid, block, smem_km(ds), s, c, js, wo, tk, ds);
+    return launch_rule(k_keymult2<LOGN, false>, grid, block, smem_km(ds), s, c, js, wo, tk, ds);
   }
   static cudaError_t moddown_row(const ks_context *c, const JobSet &js, const WsOff &wo,
                                  const Tasks &tk, cudaStream_t s) {
