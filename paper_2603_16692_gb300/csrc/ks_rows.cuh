@@ -217,47 +217,6 @@ __global__ void __launch_bounds__(2 * ColGeo<LOGN>::GP, 768 / (2 * ColGeo<LOGN>:
   pdl_trigger();
 }
 
-// Exact sum of 64 x 64-bit products: value lo + 2^32 mid + 2^64 hi. The middle products
-// are summed on their own, so a term takes four 32x32->64 products and three 64-bit adds
-// (19 cycles a warp against 28.7 for a carry chain over the whole 128 bits). mid must stay
-// below 2^63: at most `fl` terms between two folds (mac_terms).
-struct Mac3 {
-  u64 lo, hi, mid;
-  __device__ __forceinline__ void add(u64 y, u64 k) {
-    const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
-    const uint32_t kl = (uint32_t)k, kh = (uint32_t)(k >> 32);
-    const u64 l = mul_wide(yl, kl), h = mul_wide(yh, kh);
-    mid += mul_wide(yl, kh) + mul_wide(yh, kl);
-    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(lo), "+l"(hi) : "l"(l), "l"(h));
-  }
-  __device__ __forceinline__ void fold() {
-    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;"
-        : "+l"(lo), "+l"(hi)
-        : "l"(mid << 32), "l"(mid >> 32));
-    mid = 0;
-  }
-  // value * 2^-64 mod m, canonical, for a value below m 2^64 and mid below 2^63: two 32-bit
-  // Montgomery steps (inv = m^-1 mod 2^32), each taking off u m with u the low word times
-  // inv; six products against nine and about half the instructions of fold() and a 64-bit
-  // step.
-  __device__ __forceinline__ u64 reduce(u64 m, uint32_t inv) const {
-    const uint32_t ml = (uint32_t)m, mh = (uint32_t)(m >> 32);
-    const uint32_t u0 = (uint32_t)lo * inv;
-    const long long t = (long long)(mid + (lo >> 32) - (mul_wide(u0, ml) >> 32)) -
-                        (long long)mul_wide(u0, mh);
-    const uint32_t u1 = (uint32_t)t * inv;
-    const u64 r = hi + (u64)(t >> 32) - (mul_wide(u1, ml) >> 32) - mul_wide(u1, mh) + m;
-    return csub(r, m);
-  }
-};
-// The canonical residue of a sum; exact moduli, whose mid may pass 2^63, by fold() and the
-// 64-bit step.
-__device__ __forceinline__ u64 mac_reduce(Mac3 &s, const ModInfo &mi, u64 m, uint32_t inv,
-                                          int cls) {
-  if (cls != CLS_EXACT) return s.reduce(m, inv);
-  s.fold();
-  return csub(redc(U128{s.lo, s.hi}, m, mi.minv), m);
-}
 // Terms whose middle products stay below 2^63 - 2^33 in the key multiply: 71 m + 2^33 each
 // with lazy ext (below 70 m, m < 2^51), 2 m + 2^33 otherwise (m < 2^60); exact moduli fold
 // every term.
@@ -305,41 +264,55 @@ __device__ __forceinline__ void bconv_points(u64 *v, const KArgs &a, int tgt, in
     u64 x[H];
 #pragma unroll
     for (int k = 0; k < H; ++k) x[k] = src[(size_t)C0::point(t, h + k) << LOGB];
-    u64 c = __ldg(cst);
-    bool one = true;  // no reduction yet
-    int left = run, fold = fl;
-#pragma unroll 1
-    for (int i = 0; i < ns; ++i) {
-      u64 xn[H], cn = 0;
-      if (i + 1 < ns) {  // the next limb's loads before this one's products (two limbs
-                         // ahead measured the same)
-        const u64 *sn = src + ((size_t)(i + 1) << LOGN);
+    if (ns <= fl) {  // the usual case: one sum, no fold on the way
+#pragma unroll 2
+      for (int i = 0; i < ns; ++i) {
+        const u64 c = __ldg(cst + i);
+        u64 xn[H];
+        if (i + 1 < ns) {  // the next limb's loads before this one's products
+          const u64 *sn = src + ((size_t)(i + 1) << LOGN);
 #pragma unroll
-        for (int k = 0; k < H; ++k) xn[k] = sn[(size_t)C0::point(t, h + k) << LOGB];
-        cn = __ldg(cst + i + 1);
+          for (int k = 0; k < H; ++k) xn[k] = sn[(size_t)C0::point(t, h + k) << LOGB];
+        }
+#pragma unroll
+        for (int k = 0; k < H; ++k) s[k].add(x[k], c);
+#pragma unroll
+        for (int k = 0; k < H; ++k) x[k] = xn[k];
       }
 #pragma unroll
-      for (int k = 0; k < H; ++k) s[k].add(x[k], c);
-      --left;
-      if (--fold == 0 || left == 0 || i == ns - 1) {
-        fold = fl;
+      for (int k = 0; k < H; ++k) v[h + k] = mac_reduce(s[k], mi, m, inv, rcls);
+    } else {
+#pragma unroll
+      for (int k = 0; k < H; ++k) v[h + k] = 0;
+      int left = run, fold = fl;
+#pragma unroll 1
+      for (int i = 0; i < ns; ++i) {
+        const u64 c = __ldg(cst + i);
+        u64 xn[H];
+        if (i + 1 < ns) {
+          const u64 *sn = src + ((size_t)(i + 1) << LOGN);
+#pragma unroll
+          for (int k = 0; k < H; ++k) xn[k] = sn[(size_t)C0::point(t, h + k) << LOGB];
+        }
+#pragma unroll
+        for (int k = 0; k < H; ++k) s[k].add(x[k], c);
+        --left;
         if (left == 0 || i == ns - 1) {
           left = run;
+          fold = fl;
 #pragma unroll
           for (int k = 0; k < H; ++k) {
-            const u64 z = mac_reduce(s[k], mi, m, inv, rcls);
-            v[h + k] = one ? z : csub(v[h + k] + z, m);
+            v[h + k] = csub(v[h + k] + mac_reduce(s[k], mi, m, inv, rcls), m);
             s[k] = Mac3{};
           }
-          one = false;
-        } else {
+        } else if (--fold == 0) {
+          fold = fl;
 #pragma unroll
           for (int k = 0; k < H; ++k) s[k].fold();
         }
-      }
 #pragma unroll
-      for (int k = 0; k < H; ++k) x[k] = xn[k];
-      c = cn;
+        for (int k = 0; k < H; ++k) x[k] = xn[k];
+      }
     }
   }
 }
