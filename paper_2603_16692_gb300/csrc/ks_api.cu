@@ -236,7 +236,11 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
   }
 
   // Input iNTT, fused with the per-limb factor N^-1 * Qhat_{j,i}^-1 of the ModUp BConv.
-  {
+  // one cluster kernel where the size has it (its stages on their own while profiling)
+  const bool fuinv = c->fu && !g_prof.on;
+  if (fuinv && !pl.tc_up) {
+    KS_TRY(c->fu->inv(c, js, wo, 0, s));
+  } else {
     const double nl = c->nq;
     KS_TRY(timed("intt_row(d)", 2 * nl * W, nl * (BF_B + (single ? NJ : 0)), 0, s,
                  [&] { return L.intt_row(c, js, wo, 0, s); }));
@@ -335,7 +339,9 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
   }
 
   // iNTT of the P-limbs of both accumulators, fused with N^-1 * Phat_k^-1.
-  {
+  if (fuinv && !pl.tc_down) {
+    KS_TRY(c->fu->inv(c, js, wo, 1, s));
+  } else {
     const double nl = 2.0 * c->np;
     KS_TRY(timed("intt_row(accP)", 2 * nl * W, nl * (BF_B + (single ? NJ : 0)), 0, s,
                  [&] { return L.intt_row(c, js, wo, 1, s); }));

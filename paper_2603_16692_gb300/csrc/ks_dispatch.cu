@@ -40,6 +40,7 @@ const LaunchTable &launch_table_11_2_0();
 const LaunchTable &launch_table_11_4_0();
 const FusedTable &fused_table_12();
 const FusedTable &fused_table_13();
+const FusedTable &fused_table_14();
 const LaunchTable &launch_table_12();
 const LaunchTable &launch_table_13();
 const LaunchTable &launch_table_14();
@@ -79,6 +80,7 @@ const FusedTable *fused_table(int logn) {
   switch (logn) {
     case 12: return &fused_table_12();
     case 13: return &fused_table_13();
+    case 14: return &fused_table_14();
     default: return nullptr;
   }
 }

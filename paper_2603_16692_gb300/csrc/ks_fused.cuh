@@ -1,11 +1,15 @@
-// The four steps of a KeySwitch as one kernel each for small N (2^12, 2^13): a cluster of
+// The steps of a KeySwitch as one kernel each for small N (2^12, 2^13; the inverse
+// transform alone at 2^14): a cluster of
 // eight CTAs holds a whole limb, a CTA an eighth of its columns in the column pass and an
 // eighth of its rows in the row pass, and the points change hands through distributed
 // shared memory between the two. Against the two kernels per step of the general path this
 // takes out four launches with their fill and drain (more than the arithmetic of a pass at
 // these sizes) and the ModUp and ModDown intermediates' trip through L2. Bound by latency:
 // one or two warps per scheduler. (2, 2^12, 3): 27.9 us against 32.1 on the general kernels
-// and 67.5 on one CTA per limb; where the line lies: fused_rule in ks_api.cu.
+// and 67.5 on one CTA per limb; where the line lies: fused_rule in ks_api.cu. The inverse
+// transform is the faster form at every limb count up to 2^14, in front of the general
+// kernels too ((7, 2^14, 30) 119.9 -> 113.6 us, (6, 2^13, 44) 85.3 -> 83.6), and the slower
+// one at 2^15 ((10, 2^15, 33) 256 -> 276 us; clusters of 16: 271).
 //   k_fu_inv    rows, columns and scale of one limb's iNTT (input limbs, or one polynomial's
 //               P-limb of the accumulators)
 //   k_fu_up     one target limb: per digit basis conversion, columns, rows; then the key
@@ -324,9 +328,15 @@ struct FusedFns {
   // groups of threads that take the digits in turn
   static int groups(int beta) { return std::max(1, std::min(beta, kFuThreads / FG::NT)); }
   static bool fits(int beta) { return FG::smem_up(beta, groups(beta)) <= kSmemMax; }
+  static cudaError_t prepare_inv() { return smem_attr(k_fu_inv<LOGN>, FG::smem_inv()); }
+  static cudaError_t inv(const ks_context *c, const JobSet &js, const WsOff &wo, int which,
+                         cudaStream_t s) {
+    return launch_cluster(k_fu_inv<LOGN>, dim3(kFuC, which == 0 ? c->nq : 2 * c->np, js.n),
+                          FG::NT, FG::smem_inv(), s, args_of(c), js, wo, which);
+  }
   static cudaError_t prepare() {
     cudaError_t e;
-    if ((e = smem_attr(k_fu_inv<LOGN>, FG::smem_inv()))) return e;
+    if ((e = prepare_inv())) return e;
     if ((e = smem_attr(k_fu_down<LOGN>, FG::smem_inv()))) return e;
     return smem_attr(k_fu_up<LOGN>, kSmemMax);
   }
@@ -335,20 +345,22 @@ struct FusedFns {
     const KArgs a = args_of(c);
     const int G = groups(c->beta);
     cudaError_t e;
-    if ((e = launch_cluster(k_fu_inv<LOGN>, dim3(kFuC, c->nq, js.n), FG::NT, FG::smem_inv(), s, a,
-                            js, wo, 0)))
-      return e;
+    if ((e = inv(c, js, wo, 0, s))) return e;
     if ((e = launch_cluster(k_fu_up<LOGN>, dim3(kFuC, c->qp, js.n), G * FG::NT,
                             FG::smem_up(c->beta, G), s, a, js, wo)))
       return e;
-    if ((e = launch_cluster(k_fu_inv<LOGN>, dim3(kFuC, 2 * c->np, js.n), FG::NT, FG::smem_inv(),
-                            s, a, js, wo, 1)))
-      return e;
+    if ((e = inv(c, js, wo, 1, s))) return e;
     return launch_cluster(k_fu_down<LOGN>, dim3(kFuC, 2 * c->nq, js.n), FG::NT, FG::smem_inv(), s,
                           a, js, wo);
   }
   static const FusedTable &table() {
-    static const FusedTable t = {&prepare, &fits, &run};
+    static const FusedTable t = {&prepare, &fits, &run, &inv};
+    return t;
+  }
+  // only the inverse transform
+  static bool no_fit(int) { return false; }
+  static const FusedTable &table_inv() {
+    static const FusedTable t = {&prepare_inv, &no_fit, nullptr, &inv};
     return t;
   }
 };

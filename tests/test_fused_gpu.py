@@ -1,4 +1,4 @@
-"""The cluster kernels of N = 2^12 and 2^13 == oracle, bit for bit, on both sides of their
+"""The cluster kernels of N = 2^12 .. 2^14 == oracle, bit for bit, on both sides of their
 dispatch rule (eight CTAs per target limb within the 152 SMs; digits within a CTA's shared
 memory), with every epilogue that they share with the general kernels.
 
@@ -19,7 +19,8 @@ from tests.gpu_util import dev, first_mismatch, host, oracle_case
 pytestmark = pytest.mark.gpu
 
 CFGS = [(1, 12, 0), (1, 12, 8), (2, 12, 3), (2, 12, 4), (6, 12, 5), (9, 12, 16), (15, 12, 14),
-        (4, 12, 15), (1, 13, 5), (2, 13, 7), (5, 13, 6), (8, 13, 15), (4, 13, 14), (4, 13, 15)]
+        (4, 12, 15), (1, 13, 5), (2, 13, 7), (5, 13, 6), (8, 13, 15), (4, 13, 14), (4, 13, 15),
+        (1, 14, 0), (3, 14, 7)]
 
 
 @pytest.mark.parametrize("cfg", CFGS, ids=str)
