@@ -194,8 +194,11 @@ int ks_workspace_size(const ks_context *ctx, int variant, int chunks, size_t *by
  *   variant KS_DSOB..KS_DPOC (| KS_UNFUSED | KS_RADIX4 | KS_RADIX16 | a radix schedule
  *           KS_STAGE_RADIX(..) | KS_COLALT_* | KS_SPLIT_DOWN | KS_BCONV_TC |
  *           KS_BCONV_TC_DOWN), or KS_AUTO (the plan ks_tune chose for this context,
- *           else the one ks_select chose, else DPOB fused radix 8; the last two with
- *           KS_BCONV_TC added where ks_info.tc = 1, N >= 2^16 and L+1 > alpha)
+ *           else the one ks_select chose, else DPOB fused; the last two with
+ *           KS_BCONV_TC added where ks_info.tc = 1 and (beta QP + L+1) alpha N is at least
+ *           7 * 2^20 per conversion launch: 2 for DPOB, beta + 1 for DSOB, chunks times as
+ *           many for DPOC and DSOC. KS_AUTO leaves that addition out when the scratch at
+ *           hand, or the device, holds the plan only without it)
  *   chunks  1..64 output groups for the OC variants (0 = 2; the paper searches 2..10);
  *           ignored for OB
  *   workspace_dev / workspace_bytes: caller scratch of at least
@@ -288,7 +291,8 @@ int ks_switch_host_async_ws(ks_context *ctx, const uint64_t *d_host, const uint6
  *   Scratch: a static device array of ks_noalloc_scratch_bytes() bytes (128 MiB) in
  *   this library; every GPU that loads it holds it until the process exits. The
  *   caller still passes the inputs and the output.
- *   Limit: if ks_workspace_size(ctx, variant, chunks) exceeds that size, returns
+ *   Limit: if ks_workspace_size(ctx, variant, chunks) exceeds that size (and KS_AUTO has
+ *   no tensor-core conversions of its own to leave out), returns
  *   KS_EINVAL and launches nothing (e.g. (4,2^16,35) fits with KS_DSOC and
  *   chunks >= 4, not with KS_DPOB).
  *   Device: the current device must be the context's (else KS_EINVAL).
@@ -423,8 +427,7 @@ int ks_selector_load(const ks_selector *sel);
  * uses it when ks_tune has not chosen one, and ks_switch_batch with KS_BATCH_SELECT
  * uses it for jobs naming KS_AUTO. Writes the plan to *variant / *chunks when not
  * null (ks_info.selected_variant reports the same pick). The selected plan runs with
- * KS_BCONV_TC added where the context has the tensor-core path (ks_info.tc), N >= 2^16
- * and the input spans more than one digit (L+1 > alpha). KS_EINVAL when no selector is
+ * KS_BCONV_TC added by the rule that ks_switch's KS_AUTO states. KS_EINVAL when no selector is
  * installed on the current device. */
 int ks_select(ks_context *ctx, int *variant, int *chunks, void *stream);
 

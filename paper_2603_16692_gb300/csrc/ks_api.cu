@@ -35,6 +35,7 @@ struct Plan {
   int srl[ST_COUNT];  // per stage (the plan's unless the variant's schedule sets one)
   int code;      // every variant bit that changes the launches (graph-cache key)
   bool split;    // KS_SPLIT_DOWN in effect (fused DPOB, two-pass N)
+  bool ruled;    // tc_up by tc_rule alone (KS_AUTO)
   bool tc_up;    // KS_BCONV_TC in effect (fused, context with a tensor-core path)
   bool tc_down;  // KS_BCONV_TC or KS_BCONV_TC_DOWN in effect
   int chunks;    // phase-1 and phase-2 group counts (1 for OB)
@@ -48,16 +49,25 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 
 constexpr int kSchedMask = 0x3ff << KS_STAGE_SHIFT;
 
-// The tensor-core basis conversions where they measured faster than the integer ones:
-// contexts that have them, N >= 2^16 and an input of more than one digit (at
-// (4, 2^16, 35) the tuned per-level plans use them at every level with two or more
-// digits and at none with one). Added to the plans KS_AUTO takes without a tuned one.
-int tc_rule(const ks_context *c) {
-  return c->tc_ap > 0 && c->logn >= 16 && c->nq > c->alpha ? KS_BCONV_TC : 0;
+// The tensor-core basis conversions where they are the faster ones, for the plans KS_AUTO
+// takes without a tuned one: per conversion launch (ModUp and ModDown, per digit and group
+// where the dataflow splits them), the products of a source and a target residue that leave
+// the integer pipes have to outweigh the launch's start-up and the wider intermediate.
+// Measured (integer / tensor-core, us; products per launch in 2^20):
+//   DPOB (2,2^15,10) 4.2 64.1 / 72.6, (3,2^14,18) 5.3 63.7 / 66.7, (4,2^16,35) level 7 7.0
+//   109.3 / 111.1, level 8 7.6 112.6 / 108.7, (4,2^15,19) 9.4 117.5 / 112.8, (7,2^14,30)
+//   11 112.9 / 107.1, (9,2^14,52) 27 216.6 / 184.1, (8,2^16,60) 153 905 / 693
+//   DSOB (2,2^15,17) 6.8 108.7 / 116.3, (3,2^15,26) 9.5 177 / 167.5
+//   DPOC (7,2^14,30) 5.5 125.3 / 135.0, (10,2^13,60) 9.2 147.9 / 143.4
+//   DSOC (3,2^15,26) 4.7 199 / 233, (2,2^16,17) 6.8 233.8 / 227.7
+constexpr double kTcWork = 7 << 20;
+int tc_rule(const ks_context *c, int base, int chunks) {
+  const bool dp = base == KS_DPOB || base == KS_DPOC, oc = base == KS_DSOC || base == KS_DPOC;
+  const int groups = oc ? (chunks ? chunks : 2) : 1;
+  const double targets = (double)c->beta * c->qp + c->nq;  // each digit's others, ModDown's
+  const double launches = (double)groups * ((dp ? 1 : c->beta) + 1);
+  return c->tc_ap > 0 && targets * c->alpha * c->N >= kTcWork * launches ? KS_BCONV_TC : 0;
 }
-// The plan a selected context runs: the network's pick (a dataflow and radix among
-// integer plans) with the tensor-core rule.
-int selected_plan(const ks_context *c) { return c->sel_variant | tc_rule(c); }
 
 // The cluster kernels (ks_fused.cuh) serve the plain fused DPOB plan when they have the
 // size's limbs, the digits fit a CTA's shared memory, and their widest launch, eight CTAs
@@ -70,22 +80,31 @@ bool fused_rule(const ks_context *c, int jobs) {
   return c->fu && c->fu->fits(c->beta) && 8 * c->qp * jobs <= 152;
 }
 
-int make_plan(const ks_context *c, int variant, int chunks, Plan *pl) {
+// room: words of scratch there are. A KS_AUTO plan whose tensor-core conversions tc_rule
+// added goes without them where they do not fit.
+int make_plan(const ks_context *c, int variant, int chunks, Plan *pl,
+              size_t room = ~(size_t)0) {
   if (variant & ~(0xff | KS_UNFUSED | KS_RADIX4 | KS_RADIX16 | kSchedMask | KS_COLTILE_ALT |
                   KS_SPLIT_DOWN | KS_BCONV_TC | KS_BCONV_TC_DOWN))
     return KS_EINVAL;
   if ((variant & KS_RADIX4) && (variant & KS_RADIX16)) return KS_EINVAL;
+  pl->ruled = false;
   if ((variant & 0xff) == KS_AUTO) {
-    // the tuned choice for single KeySwitches, else the selector's, else DPOB radix 8
-    // (the last two with the tensor-core rule)
+    // the tuned choice for single KeySwitches, else the selector's, else DPOB (the last two
+    // with tc_rule)
+    const int flags = variant & ~0xff;
     if (c->tuned_variant > 0) {
-      variant = c->tuned_variant | (variant & ~0xff);
+      variant = c->tuned_variant | flags;
       if (chunks == 0) chunks = c->tuned_chunks;
-    } else if (c->sel_variant > 0) {
-      variant = selected_plan(c) | (variant & ~0xff);
-      if (chunks == 0) chunks = c->sel_chunks;
     } else {
-      variant = KS_DPOB | tc_rule(c) | (variant & ~0xff);
+      variant = KS_DPOB | flags;
+      if (c->sel_variant > 0) {
+        variant = c->sel_variant | flags;
+        if (chunks == 0) chunks = c->sel_chunks;
+      }
+      const int tc = tc_rule(c, variant & 0xff, chunks);
+      pl->ruled = tc & ~variant;
+      variant |= tc;
     }
   }
   const int base = variant & 0xff;
@@ -137,7 +156,14 @@ int make_plan(const ks_context *c, int variant, int chunks, Plan *pl) {
   pl->off_pv = pl->tc_up ? take((size_t)2 * c->nq * N) : 0;
   pl->off_ppv = pl->tc_down ? take((size_t)4 * c->np * N) : 0;
   pl->total = off;
+  if (pl->ruled && off > room) return make_plan(c, variant & ~KS_BCONV_TC, chunks, pl);
   return KS_OK;
+}
+// The words that a caller's workspace holds (the context's own: as many as needed) beside
+// `extra` words for other buffers.
+size_t room_of(const void *ws, size_t ws_bytes, size_t extra) {
+  if (!ws) return ~(size_t)0;
+  return ws_bytes / 8 > extra ? ws_bytes / 8 - extra : 0;
 }
 
 thread_local cudaError_t g_last_cuda = cudaSuccess;
@@ -736,6 +762,17 @@ int with_workspace(ks_context *c, void *ws, size_t ws_bytes, size_t need, F fn) 
   return fn((u64 *)c->ws);
 }
 
+// with_workspace for plan pl (made from variant, chunks) and `extra` words; when the arena
+// cannot grow to it, pl again without the tensor-core conversions that tc_rule added.
+template <class F>
+int with_plan(ks_context *c, int variant, int chunks, Plan &pl, void *ws, size_t ws_bytes,
+              size_t extra, F fn) {
+  int rc = with_workspace(c, ws, ws_bytes, (pl.total + extra) * 8, fn);
+  if (rc != KS_ENOMEM || !pl.ruled) return rc;
+  rc = make_plan(c, variant, chunks, &pl, 0);
+  return rc ? rc : with_workspace(c, ws, ws_bytes, (pl.total + extra) * 8, fn);
+}
+
 // Device-time budget of one wait of the persistent batch kernel.
 constexpr unsigned long long kPersistWaitNs = 2000000000ull;
 
@@ -972,10 +1009,10 @@ int ks_switch(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *o
   if (!aligned16(d) || !aligned16(evk) || !aligned16(out) || (ws && !aligned16(ws)))
     return KS_EALIGN;
   Plan pl;
-  int rc = make_plan(c, variant, chunks, &pl);
+  int rc = make_plan(c, variant, chunks, &pl, room_of(ws, ws_bytes, 0));
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  return with_workspace(c, ws, ws_bytes, pl.total * 8, [&](u64 *base) {
+  return with_plan(c, variant, chunks, pl, ws, ws_bytes, 0, [&](u64 *base) {
     JobSet js = {};
     js.n = 1;
     js.j[0].d = (const u64 *)d;
@@ -994,6 +1031,12 @@ int ks_switch(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *o
 
 namespace ks {
 
+int plan_fits(const ks_context *c, int variant, int chunks, size_t bytes) {
+  Plan pl;
+  int rc = make_plan(c, variant, chunks, &pl, bytes / 8);
+  return rc ? rc : pl.total * 8 <= bytes ? KS_OK : KS_EINVAL;
+}
+
 // ks_switch on a caller workspace with every kernel launched directly on `stream`: no
 // graph cache (no capture, instantiation or stream creation) and no context arena.
 int switch_launch_only(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *out,
@@ -1001,7 +1044,7 @@ int switch_launch_only(ks_context *c, const uint64_t *d, const uint64_t *evk, ui
   if (!c || !d || !evk || !out || !ws) return KS_EINVAL;
   if (!aligned16(d) || !aligned16(evk) || !aligned16(out) || !aligned16(ws)) return KS_EALIGN;
   Plan pl;
-  int rc = make_plan(c, variant, chunks, &pl);
+  int rc = make_plan(c, variant, chunks, &pl, room_of(ws, ws_bytes, 0));
   if (rc) return rc;
   if (ws_bytes < pl.total * 8) return KS_EINVAL;
   JobSet js = {};
@@ -1027,10 +1070,10 @@ int switch_host_ws(ks_context *c, const uint64_t *d_host, const uint64_t *evk, u
                    int variant, int chunks, void *ws, size_t ws_bytes, cudaStream_t s) {
   if (!c || !d_host || !evk || !out_host || !ws) return KS_EINVAL;
   if (!aligned16(evk) || !aligned16(ws)) return KS_EALIGN;
-  Plan pl;
-  int rc = make_plan(c, variant, chunks, &pl);
-  if (rc) return rc;
   const size_t in_w = (size_t)c->nq * c->N;
+  Plan pl;
+  int rc = make_plan(c, variant, chunks, &pl, room_of(ws, ws_bytes, 3 * in_w));
+  if (rc) return rc;
   if (ws_bytes < (pl.total + 3 * in_w) * 8) return KS_EINVAL;
   // pinned host memory only: pageable copies would not be asynchronous
   if (!host_mapped(d_host) || !host_mapped(out_host)) return KS_EINVAL;
@@ -1087,7 +1130,7 @@ int switch_host(ks_context *c, const uint64_t *d_host, const uint64_t *evk, uint
   if (async && !mapped) return KS_EINVAL;
   // the kernels access mapped host buffers with 16-byte vector loads and stores
   if (mapped && (!aligned16(d_map) || !aligned16(out_map))) return KS_EALIGN;
-  rc = with_workspace(c, nullptr, 0, pl.total * 8, [&](u64 *base) {
+  rc = with_plan(c, variant, chunks, pl, nullptr, 0, 0, [&](u64 *base) {
     JobSet js = {};
     js.n = 1;
     js.j[0].d = (const u64 *)din;
@@ -1177,12 +1220,12 @@ int ks_hmul(ks_context *c, const uint64_t *ct1, const uint64_t *ct2, const uint6
   if (!aligned16(ct1) || !aligned16(ct2) || !aligned16(rlk) || !aligned16(out) ||
       (ws && !aligned16(ws)))
     return KS_EALIGN;
-  Plan pl;
-  int rc = make_plan(c, variant, chunks, &pl);
-  if (rc) return rc;
   const size_t extra = (size_t)c->nq * c->N;
+  Plan pl;
+  int rc = make_plan(c, variant, chunks, &pl, room_of(ws, ws_bytes, extra));
+  if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  return with_workspace(c, ws, ws_bytes, (pl.total + extra) * 8, [&](u64 *base) {
+  return with_plan(c, variant, chunks, pl, ws, ws_bytes, extra, [&](u64 *base) {
     u64 *d2 = base + pl.total;
     JobSet js = {};
     js.n = 1;
@@ -1208,12 +1251,12 @@ int ks_hrot(ks_context *c, const uint64_t *ct, uint32_t galois_elt, const uint64
   if (!c || !ct || !rtk || !out || !galois_ok(c, galois_elt)) return KS_EINVAL;
   if (!aligned16(ct) || !aligned16(rtk) || !aligned16(out) || (ws && !aligned16(ws)))
     return KS_EALIGN;
-  Plan pl;
-  int rc = make_plan(c, variant, chunks, &pl);
-  if (rc) return rc;
   const size_t extra = (size_t)2 * c->nq * c->N;
+  Plan pl;
+  int rc = make_plan(c, variant, chunks, &pl, room_of(ws, ws_bytes, extra));
+  if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  return with_workspace(c, ws, ws_bytes, (pl.total + extra) * 8, [&](u64 *base) {
+  return with_plan(c, variant, chunks, pl, ws, ws_bytes, extra, [&](u64 *base) {
     u64 *y0 = base + pl.total, *y1 = y0 + (size_t)c->nq * c->N;
     JobSet js = {};
     js.n = 1;
@@ -1281,6 +1324,7 @@ int ks_switch_batch(const ks_job *jobs, int njobs, int flags, void *stream) {
       if (rc) return rc;
     }
   }
+  std::vector<char> gruled(ctxs.size());  // tensor-core conversions, if any, by tc_rule alone
   if (flags & KS_BATCH_SELECT) {
     for (size_t g = 0; g < ctxs.size(); ++g) {
       ks_context *c = ctxs[g];
@@ -1289,17 +1333,27 @@ int ks_switch_batch(const ks_job *jobs, int njobs, int flags, void *stream) {
         int rc = ks_select(c, nullptr, nullptr, stream);
         if (rc) return rc;
       }
-      gplan[g] = {selected_plan(c) | (gplan[g].first & ~0xff),
-                  gplan[g].second ? gplan[g].second : c->sel_chunks};
+      const int v = c->sel_variant | (gplan[g].first & ~0xff);
+      const int ch = gplan[g].second ? gplan[g].second : c->sel_chunks;
+      const int tc = tc_rule(c, v & 0xff, ch);
+      gruled[g] = (tc & ~v) != 0;
+      gplan[g] = {v | tc, ch};
     }
   }
   std::vector<Plan> plans(ctxs.size());
   size_t total = 0;
-  for (size_t g = 0; g < ctxs.size(); ++g) {
-    int rc = make_plan(ctxs[g], gplan[g].first, gplan[g].second, &plans[g]);
-    if (rc) return rc;
-    total += plans[g].total * 8 * members[g].size();
-  }
+  auto plan_groups = [&](size_t room) {
+    total = 0;
+    for (size_t g = 0; g < ctxs.size(); ++g) {
+      if (room == 0 && gruled[g]) gplan[g].first &= ~KS_BCONV_TC;
+      int rc = make_plan(ctxs[g], gplan[g].first, gplan[g].second, &plans[g], room);
+      if (rc) return rc;
+      total += plans[g].total * 8 * members[g].size();
+    }
+    return (int)KS_OK;
+  };
+  int prc = plan_groups(~(size_t)0);
+  if (prc) return prc;
   std::lock_guard<std::mutex> lk(g_batch.mu);
   if (g_batch.arena_bytes < total) {
     if (g_batch.arena) {
@@ -1311,7 +1365,15 @@ int ks_switch_batch(const ks_job *jobs, int njobs, int flags, void *stream) {
     g_batch.arena_bytes = 0;
     if (cudaMalloc(&g_batch.arena, total) != cudaSuccess) {
       cudaGetLastError();
-      return KS_ENOMEM;
+      g_batch.arena = nullptr;
+      // as in with_plan: without the conversions that tc_rule added
+      const size_t full = total;
+      if ((prc = plan_groups(0))) return prc;
+      if (total == full || cudaMalloc(&g_batch.arena, total) != cudaSuccess) {
+        cudaGetLastError();
+        g_batch.arena = nullptr;
+        return KS_ENOMEM;
+      }
     }
     g_batch.arena_bytes = total;
   }

@@ -266,6 +266,9 @@ const FusedTable *fused_table(int logn);  // null for sizes without them
 // cache, no arena (ks_api.cu).
 int switch_launch_only(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *out,
                        int variant, int chunks, void *ws, size_t ws_bytes, void *stream);
+// KS_OK when the plan fits `bytes` of scratch (a KS_AUTO plan: with or without the
+// tensor-core conversions that its rule adds), else KS_EINVAL.
+int plan_fits(const ks_context *c, int variant, int chunks, size_t bytes);
 // True when ctx's selected plan came from the selector installed now (ks_select.cu).
 bool selected_current(const ks_context *c);
 

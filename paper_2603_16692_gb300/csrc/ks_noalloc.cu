@@ -55,10 +55,8 @@ size_t ks_noalloc_scratch_bytes(void) { return kScratchBytes; }
 int ks_switch_noalloc(ks_context *ctx, const uint64_t *d_dev, const uint64_t *evk_dev,
                       uint64_t *out_dev, int variant, int chunks, void *stream) {
   if (!ctx || !d_dev || !evk_dev || !out_dev) return KS_EINVAL;
-  size_t need = 0;
-  int rc = ks_workspace_size(ctx, variant, chunks, &need);
+  int rc = ks::plan_fits(ctx, variant, chunks, kScratchBytes);
   if (rc) return rc;
-  if (need > kScratchBytes) return KS_EINVAL;  // does not fit the static scratch
   // The scratch address belongs to the current device: it must be the context's.
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) {

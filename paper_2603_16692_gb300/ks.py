@@ -304,12 +304,16 @@ def ks_switch_noalloc(ctx: int, d, evk, out, variant: int = KS_AUTO, chunks: int
     CUDA-graph capture, under a fixed memory budget). Raises ValueError when the
     workload's scratch exceeds ks_noalloc_scratch_bytes()."""
     need = ks_workspace_size(ctx, variant, chunks)
-    if need > ks_noalloc_scratch_bytes():
+    fits = need <= ks_noalloc_scratch_bytes()
+    rc = KS_EINVAL
+    if fits or variant & 0xff == KS_AUTO:  # KS_AUTO may leave out its tensor-core conversions
+        rc = load().ks_switch_noalloc(ctx, _ptr(d), _ptr(evk), _ptr(out), variant, chunks,
+                                      _stream(stream))
+    if not fits and rc == KS_EINVAL:
         raise ValueError(f"ks_switch_noalloc: needs {need} bytes of scratch, the static scratch "
                          f"holds {ks_noalloc_scratch_bytes()}; use an OutputChunked variant or "
                          f"ks_switch with a workspace")
-    _check(load().ks_switch_noalloc(ctx, _ptr(d), _ptr(evk), _ptr(out), variant, chunks,
-                                    _stream(stream)), "ks_switch_noalloc")
+    _check(rc, "ks_switch_noalloc")
 
 
 def _host_ptr(x) -> int:
