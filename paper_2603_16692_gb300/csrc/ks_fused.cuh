@@ -144,17 +144,12 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
                             : is.src + ((size_t)(o * is.src_outer + ii) << LOGN)) +
                    off;
   u64 *ws = tile + w0 * FG::RP;
+  WarpPairs<FG> in;
+  in.load(src);
+  warp_rows<FG>([&](int k, int, int p) { *reinterpret_cast<ulonglong2 *>(ws + p) = in.x[k]; });
   if (host_in) {
     u64 *copy = const_cast<u64 *>(jp.d) + ((size_t)ii << LOGN) + off;
-    warp_rows<FG>([&](int e, int p) {
-      const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(src + e);
-      *reinterpret_cast<ulonglong2 *>(copy + e) = x;
-      *reinterpret_cast<ulonglong2 *>(ws + p) = x;
-    });
-  } else {
-    warp_rows<FG>([&](int e, int p) {
-      *reinterpret_cast<ulonglong2 *>(ws + p) = *reinterpret_cast<const ulonglong2 *>(src + e);
-    });
+    warp_rows<FG>([&](int k, int e, int) { *reinterpret_cast<ulonglong2 *>(copy + e) = in.x[k]; });
   }
   __syncthreads();  // the warp's rows, and the barrier's initialisation
   tw_ready<true>(&twbar, a.tab.err);
@@ -261,8 +256,6 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
   const u64 m = a.tab.mod[i].m;
   const ulonglong2 pv = a.tab.pinv[i];
   const int cls = mod_class(m);
-  const bool fast = cls == CLS_FAST;
-  const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
   const int g = threadIdx.x % FG::CC, t = threadIdx.x / FG::CC;
   const int row = threadIdx.x / FG::T2, t2 = threadIdx.x % FG::T2, w0 = row / FG::WR * FG::WR;
   const size_t woff = (size_t)(rank * FG::RC + w0) << FG::LOGB;  // the warp's rows
@@ -278,25 +271,12 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
   fu_columns<FG>(v, colbuf, twc, m, cls, t, g, rank, ext, sync);
   cluster_arrive();
   cluster_wait();
+  WarpPairs<FG> acc;
+  acc.load(ac);
   fu_row<FG>(ext + row * FG::RP, twr + row * FG::N2, a.tab.mod[i], m, cls, t2, false);
   __syncwarp();
   const u64 *ws = ext + w0 * FG::RP;
-  const size_t ob = ((size_t)(c * a.nq + i) << LOGN) + woff;
-  const bool add = (jp.addmask >> c) & 1;
-  warp_rows<FG>([&](int e, int q) {  // as in k_moddown2
-    const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(ws + q);
-    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(ac + e);
-    const u64 z0 = fast ? z.x : csub(z.x, zs), z1 = fast ? z.y : csub(z.y, zs);
-    ulonglong2 r;
-    r.x = csub(shoup(x.x + zb - z0, pv.x, pv.y, m), m);
-    r.y = csub(shoup(x.y + zb - z1, pv.x, pv.y, m), m);
-    if (add) {
-      const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(jp.add + ob + e);
-      r.x = addmod(r.x, y.x, m);
-      r.y = addmod(r.y, y.y, m);
-    }
-    *reinterpret_cast<ulonglong2 *>(jp.out + ob + e) = r;
-  });
+  scale_rows<FG>(jp, c, ws, acc, ((size_t)(c * a.nq + i) << LOGN) + woff, pv, m, cls);
   pdl_trigger();
 }
 

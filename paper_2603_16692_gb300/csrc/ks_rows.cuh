@@ -65,17 +65,31 @@ __device__ __forceinline__ void row_inv_cls(u64 *v, u64 *s, const ulonglong2 *tw
 }
 
 // Lane-linear 16-byte walk over a warp's own rows: pair k of lane l covers words
-// 2 (l + 32 k) of the warp's WR rows (contiguous in global memory); calls f(word offset in
-// the warp's rows, position in its shared rows).
+// 2 (l + 32 k) of the warp's WR rows (contiguous in global memory); calls f(k, word offset
+// in the warp's rows, position in its shared rows).
 template <class RG, class F>
 __device__ __forceinline__ void warp_rows(F f) {
-  constexpr int W = RG::WR * RG::N2;  // words of the warp's rows
 #pragma unroll
-  for (int k = 0; k < W / 64; ++k) {
+  for (int k = 0; k < RG::WR * RG::N2 / 64; ++k) {
     const int e = 2 * ((threadIdx.x & 31) + 32 * k);
-    f(e, (e >> RG::LOGB) * RG::RP + core::row_pos(e & (RG::N2 - 1)));
+    f(k, e, (e >> RG::LOGB) * RG::RP + core::row_pos(e & (RG::N2 - 1)));
   }
 }
+
+// A lane's pairs of the warp's rows at src, all in flight before the first is used. (A load
+// in the loop that also stores is not moved above the store of the pair before, which may
+// be its source: one round trip per pair. (2, 2^15, 10) 63.9 ->
+// 62.3 us, (4, 2^16, 35) on tensor cores 316 -> 310. The accumulators' pairs loaded before
+// the transform instead of after it: 311.)
+template <class RG>
+struct WarpPairs {
+  ulonglong2 x[RG::WR * RG::N2 / 64];
+  __device__ __forceinline__ void load(const u64 *src) {
+    warp_rows<RG>([&](int k, int e, int) {
+      x[k] = *reinterpret_cast<const ulonglong2 *>(src + e);
+    });
+  }
+};
 
 // A value between the two inverse passes: the column pass starts from values below 4m
 // (fast; the row pass leaves them below 2^10 m), or takes the row pass's bounds as they are
@@ -119,17 +133,12 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   const u64 *src = host_in ? jp.dsrc + (size_t)ii * N + off
                            : is.src + ((size_t)o * is.src_outer + ii) * N + off;
   u64 *ws = tile + w0 * RG::RP;
+  WarpPairs<RG> in;
+  in.load(src);
+  warp_rows<RG>([&](int k, int, int p) { *reinterpret_cast<ulonglong2 *>(ws + p) = in.x[k]; });
   if (host_in) {
     u64 *copy = const_cast<u64 *>(jp.d) + (size_t)ii * N + off;
-    warp_rows<RG>([&](int e, int p) {
-      const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(src + e);
-      *reinterpret_cast<ulonglong2 *>(copy + e) = x;
-      *reinterpret_cast<ulonglong2 *>(ws + p) = x;
-    });
-  } else {
-    warp_rows<RG>([&](int e, int p) {
-      *reinterpret_cast<ulonglong2 *>(ws + p) = *reinterpret_cast<const ulonglong2 *>(src + e);
-    });
+    warp_rows<RG>([&](int k, int e, int) { *reinterpret_cast<ulonglong2 *>(copy + e) = in.x[k]; });
   }
   __syncthreads();  // the warp's rows, and the barrier's initialisation
   tw_ready<true>(&twbar, a.tab.err);
@@ -405,7 +414,7 @@ __global__ void __launch_bounds__(64)
   __syncwarp();
   const u64 *ws = tile + w0 * RG::RP;
   u64 *o = b + ((size_t)(r0 + w0) << RG::LOGB);
-  warp_rows<RG>([&](int e, int q) {
+  warp_rows<RG>([&](int, int e, int q) {
     ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(ws + q);
     x.x = reduce_full(x.x, m, mu);
     x.y = reduce_full(x.y, m, mu);
@@ -515,8 +524,10 @@ __device__ __forceinline__ void mac_tile(const ModInfo &mi, const u64 *ext, int 
 template <class RG>
 __device__ __forceinline__ void own_rows(u64 *ws, const u64 *dt, const ModInfo &mi, bool lazy) {
   const u64 m = mi.m, r1 = mi.r1, r1s = mi.r1s;
-  warp_rows<RG>([&](int e, int p) {
-    ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(dt + e);
+  WarpPairs<RG> in;
+  in.load(dt);
+  warp_rows<RG>([&](int k, int, int p) {
+    ulonglong2 x = in.x[k];
     if (lazy) {
       x.x = shoup4(x.x, r1, r1s, m);  // [0, 4m)
       x.y = shoup4(x.y, r1, r1s, m);
@@ -607,6 +618,38 @@ __global__ void __launch_bounds__(kKmGp * kKmGroups, 768 / (kKmGp * kKmGroups))
   pdl_trigger();
 }
 
+// The final scaling of a warp's rows: out = (acc - z) P^-1 (+ addend) at word offset ob of the
+// output, z the NTT's lazy values in ws: below kFwdLazy * m (fast butterflies) or, after one
+// conditional subtraction, below 8m (mid) or 2m (exact); acc + zb - z is then positive and
+// below (kFwdLazy + 1) m, 9m or 3m < 2^64, and the Shoup product by P^-1 takes any word.
+template <class RG>
+__device__ __forceinline__ void scale_rows(const JobPtr &jp, int c, const u64 *ws,
+                                           const WarpPairs<RG> &acc, size_t ob,
+                                           const ulonglong2 &pv, u64 m, int cls) {
+  const bool fast = cls == CLS_FAST;
+  const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
+  auto word = [&](u64 z, u64 x) {
+    return csub(shoup(x + zb - (fast ? z : csub(z, zs)), pv.x, pv.y, m), m);
+  };
+  if ((jp.addmask >> c) & 1) {
+    WarpPairs<RG> y;
+    y.load(jp.add + ob);
+    warp_rows<RG>([&](int k, int e, int q) {
+      const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(ws + q);
+      ulonglong2 r;
+      r.x = addmod(word(z.x, acc.x[k].x), y.x[k].x, m);
+      r.y = addmod(word(z.y, acc.x[k].y), y.x[k].y, m);
+      *reinterpret_cast<ulonglong2 *>(jp.out + ob + e) = r;
+    });
+  } else {
+    warp_rows<RG>([&](int k, int e, int q) {
+      const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(ws + q);
+      *reinterpret_cast<ulonglong2 *>(jp.out + ob + e) =
+          make_ulonglong2(word(z.x, acc.x[k].x), word(z.y, acc.x[k].y));
+    });
+  }
+}
+
 // ---------------------------------------------------------------------------
 // ModDown row pass with the final scaling (TASK_DOWN1):
 //   out_c[i] = (acc_c[i] - NTT(BConv_{P->Q}(c))[i]) * P^-1 mod q_i (+ addend),
@@ -633,8 +676,6 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   constexpr size_t N = (size_t)1 << LOGN;
   stage_row_tw<RG>(tws, a.tab.twr_f, i, blk, &twbar);
   const int cls = mod_class(m);
-  const bool fast = cls == CLS_FAST;
-  const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
   pdl_wait(a.early);
   const size_t woff = (size_t)(r0 + w0) << RG::LOGB;  // the warp's rows
   const u64 *ac = jp.ws + wo.acc + ((size_t)c * a.qp + i) * N + woff;
@@ -653,24 +694,10 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   __syncwarp();
   core::put_row<SB>(s, v, t);
   __syncwarp();
+  WarpPairs<RG> acc;
+  acc.load(ac);
   const u64 *ws = tile + w0 * RG::RP;
-  const size_t ob = ((size_t)c * a.nq + i) * N + woff;
-  const bool add = (jp.addmask >> c) & 1;
-  // the NTT output z enters lazy, as in moddown_body
-  warp_rows<RG>([&](int e, int q) {
-    const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(ws + q);
-    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(ac + e);
-    const u64 z0 = fast ? z.x : csub(z.x, zs), z1 = fast ? z.y : csub(z.y, zs);
-    ulonglong2 r;
-    r.x = csub(shoup(x.x + zb - z0, pv.x, pv.y, m), m);
-    r.y = csub(shoup(x.y + zb - z1, pv.x, pv.y, m), m);
-    if (add) {
-      const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(jp.add + ob + e);
-      r.x = addmod(r.x, y.x, m);
-      r.y = addmod(r.y, y.y, m);
-    }
-    *reinterpret_cast<ulonglong2 *>(jp.out + ob + e) = r;
-  });
+  scale_rows<RG>(jp, c, ws, acc, ((size_t)c * a.nq + i) * N + woff, pv, m, cls);
   pdl_trigger();
 }
 
