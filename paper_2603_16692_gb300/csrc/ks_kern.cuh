@@ -1,7 +1,9 @@
-// KeySwitch kernel templates for sm_103a, specialised per N = 2^LOGN (included by
-// the ks_inst_*.cu instantiation units).
+// KeySwitch kernel templates for sm_103a, specialised per N = 2^LOGN: what every unit shares
+// (arguments, task decoding, launches), the kernels of the single-pass sizes (N <= 2^11) and
+// the stage bodies of the persistent batch (ks_persist.cu). The two-pass sizes' own kernels
+// are in ks_rows.cuh, ks_tc.cu and ks_fused.cuh.
 //
-// Two-pass negacyclic NTT / iNTT (column pass, row pass) with the fast basis
+// Negacyclic NTT / iNTT (the two-pass sizes: column pass, row pass) with the fast basis
 // conversions fused into the first forward pass and the key multiply or the
 // ModDown scaling fused into the last one (Sec. II-A, Fig. 1). Twiddles of a tile
 // are staged into shared memory once per CTA and reused for every polynomial the
@@ -469,33 +471,11 @@ __global__ void __launch_bounds__(GeoT<LOGN, RL, 1>::NT)
   pdl_trigger();  // the next kernel may launch once every CTA is here
 }
 
-// The bf16 bytes of a scaled column tile, in the layout of the tensor-core basis
-// conversion (ks_tc.cu): the limb's columns in blocks of 2^tplog / N1 columns, block
-// after block; inside a block, point (y, g) at y * (columns per block) + g, 16 bytes
-// (eight bf16) per point.
-template <class GT>
-__device__ __forceinline__ void store_pieces(u64 *pb, const u64 *s, int c0, int tplog) {
-  constexpr int TILE = GT::N1 * GT::GC;
-  const int lgc = tplog - GT::LOGA;
-#pragma unroll
-  for (int k = 0; k < (TILE + GT::NT - 1) / GT::NT; ++k) {
-    const int e = threadIdx.x + k * GT::NT;
-    if (TILE % GT::NT != 0 && e >= TILE) break;
-    const int y = e >> GT::LOGGC, g = e & (GT::GC - 1), col = c0 + g;
-    const size_t p =
-        ((size_t)(col >> lgc) << tplog) + ((size_t)y << lgc) + (col & ((1 << lgc) - 1));
-    *reinterpret_cast<uint4 *>(pb + 2 * p) = bf16_bytes(s[y * GT::PC + g]);
-  }
-}
-
-// Inverse NTT, column pass (global stages logN1-1 .. 0), in place, then the
-// per-limb scale; `only_o` as in the row pass. pieces: write the bf16 bytes of the
-// result to pv / ppv (tensor-core basis conversion) instead of the result to v / vp.
-template <int LOGN, int RL, int CA, bool TMA = true>
+// Inverse NTT, column pass (global stages logN1-1 .. 0), in place, then the per-limb scale.
+template <int LOGN, int RL, bool TMA = true>
 __device__ __forceinline__ void inv_col_body(const KArgs &a, const JobPtr &jp, const WsOff &wo,
-                                             int which, int bx, int by, unsigned char *raw,
-                                             int only_o = -1, bool pieces = false) {
-  using GT = GeoT<LOGN, RL, 0, CA>;
+                                             int which, int bx, int by, unsigned char *raw) {
+  using GT = GeoT<LOGN, RL, 0>;
   ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
   u64 *sm = tile_ptr<GT, true>(raw);
   const InttSet is = intt_set(a, jp, wo, which);
@@ -506,8 +486,7 @@ __device__ __forceinline__ void inv_col_body(const KArgs &a, const JobPtr &jp, c
   stage_tw<GT, TMA>(tws, col_table<GT>(a.tab.twc_i, prime), GT::TWC, &twbar);
   pdl_wait();
   const ulonglong2 sc = is.scale[ii];
-  const int o0 = only_o < 0 ? 0 : only_o, o1 = only_o < 0 ? is.outer : only_o + 1;
-  for (int o = o0; o < o1; ++o) {
+  for (int o = 0; o < is.outer; ++o) {
     u64 *d = is.dst + ((size_t)o * is.dst_outer + ii) * (size_t)a.N;
     load_cols<GT>(sm, d, c0);
     __syncthreads();
@@ -522,14 +501,7 @@ __device__ __forceinline__ void inv_col_body(const KArgs &a, const JobPtr &jp, c
       sm[y * GT::PC + g] = csub(shoup(sm[y * GT::PC + g], sc.x, sc.y, m), m);
     }
     __syncthreads();
-    if (pieces) {
-      // limb ii of v, or P-limb ii of polynomial o of vp: 2N words of bytes per limb
-      const size_t limb = which == 0 ? (size_t)ii : (size_t)o * a.np + ii;
-      store_pieces<GT>(jp.ws + (which == 0 ? wo.pv : wo.ppv) + limb * 2 * a.N, sm, c0,
-                       a.tc_tplog);
-    } else {
-      store_cols<GT>(d, sm, c0);
-    }
+    store_cols<GT>(d, sm, c0);
     __syncthreads();
   }
 }
@@ -552,11 +524,11 @@ __device__ __forceinline__ void fwd_bufs(const JobPtr &jp, const WsOff &wo, int 
 
 // Forward NTT, column pass (global stages 0 .. logN1-1) with a tile producer; the
 // lazy result goes to the output buffer's slot.
-template <int LOGN, int RL, int PRO, int CA, bool TMA = true>
+template <int LOGN, int RL, int PRO, bool TMA = true>
 __device__ __forceinline__ void fwd_col_body(const KArgs &a, const JobPtr &jp, const WsOff &wo,
                                              const Tasks &tk, int buf, int bx, int by,
                                              unsigned char *raw, u64 *cst) {
-  using GT = GeoT<LOGN, RL, 0, CA>;
+  using GT = GeoT<LOGN, RL, 0>;
   ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(raw);
   u64 *sm = tile_ptr<GT, true>(raw);
   const u64 *src;
@@ -751,15 +723,7 @@ struct KmSmem {
   static constexpr int BYTES = TW + 2 * TILEW * 8 + 2 * KEYW * 8;
 };
 
-// Which row kernels (key multiply, ModDown) are pipelined: two-pass sizes with radix-4
-// rounds (twice the threads per tile). With radix 8 or 16 the double buffers cost more
-// occupancy than the overlap gains (measured on GB300 at (4, 2^16, 35): key multiply
-// radix 4 115 -> 109 us but radix 8 119 -> 140 us; ModDown radix 4 55 -> 49 us, radix 8
-// 53 -> 57 us).
-template <int LOGN, int RL>
-constexpr bool ROW_PIPE = geo_loga(LOGN) != 0 && RL == 2;
-
-// The key multiply of keymult_body for N >= 2^13, software-pipelined over the digits:
+// The key multiply of keymult_body for N >= 2^13 (persistent batch), software-pipelined over the digits:
 // while digit j's ext tile is transformed and multiplied, the copies of digit j+1's
 // tile (the ModUp intermediate, or d_t on the digit's own limbs: cp.async into the odd
 // pitch) and of its two key tiles (TMA bulk copies on a barrier) are in flight into the
@@ -993,7 +957,7 @@ struct MdSmem {
   static constexpr int BYTES = TW + 2 * TILEW * 8 + 2 * GT::TILE * 8;
 };
 
-// moddown_body for N >= 2^13 with both polynomials' input tiles (cp.async into the odd
+// moddown_body for N >= 2^13 (persistent batch) with both polynomials' input tiles (cp.async into the odd
 // pitch) and accumulator tiles (TMA bulk copies on a barrier) copied into shared memory
 // at the start: the copies of c = 1 and of the accumulators are in flight while c = 0
 // is transformed. Same arithmetic and result.

@@ -34,18 +34,11 @@ namespace ks {
 // Compile-time geometry of the two passes for N = 2^LOGN (also used on the host
 // to lay out the row-pass twiddle table by row tile).
 __host__ __device__ constexpr int geo_loga(int logn) { return logn <= 11 ? 0 : logn / 2; }
-// Tiles (measured on GB300). Column pass: 2^10 points up to N = 2^15, 2^11 above (at
-// 2^15 the smaller tiles double the CTAs of the one-wave launches, 94.8 -> 85.8 us per
-// KeySwitch at (2, 2^15, 10); at 2^16 the column passes are slower with 2^10 points).
-// Row pass: 2^9 points up to N = 2^15, 2^10 above (2^9 against 2^10: 36.9 -> 33.3 us at
-// (2, 2^13, 7), 81.5 -> 77.8 us at (2, 2^14, 20), 13.4 k -> 14.0 k KeySwitch/s at
-// (2, 2^15, 10); at (4, 2^16, 35) 2^9 is 2% slower).
+// Tiles of the shared-memory rounds (the persistent batch; one tile per limb at the
+// single-pass sizes). Column pass: 2^10 points up to N = 2^15, 2^11 above. Row pass: 2^9
+// points up to N = 2^15, 2^10 above.
 __host__ __device__ constexpr int geo_tile_log_col(int logn) {
   return logn <= 11 ? logn : (logn >= 16 ? 11 : 10);
-}
-// The alternative column tile the tuner may pick (CA = 1): the other of 2^10 / 2^11.
-__host__ __device__ constexpr int geo_tile_log_col_alt(int logn) {
-  return logn <= 11 ? logn : (logn >= 16 ? 10 : 11);
 }
 __host__ __device__ constexpr int geo_tile_log_row(int logn) {
   return logn <= 11 ? logn : (logn <= 15 ? 9 : 10);
@@ -71,14 +64,13 @@ __host__ __device__ constexpr int row_tw(int ls, int c) {
 
 // RL: log2 of the radix of the register rounds; a thread holds 2^RL points.
 // ROW: geometry of the row pass (1) or of the column pass (0); a kernel runs one pass
-// and uses only that pass's fields. CA: the column pass uses the alternative tile.
-template <int LOGN, int RL_, int ROW, int CA = 0>
+// and uses only that pass's fields.
+template <int LOGN, int RL_, int ROW>
 struct GeoT {
   static constexpr int RL = RL_;
   static constexpr int LOGA = geo_loga(LOGN);  // log N1
   static constexpr int LOGB = LOGN - LOGA;     // log N2
-  static constexpr int TILE_LOG =
-      ROW ? geo_tile_log_row(LOGN) : (CA ? geo_tile_log_col_alt(LOGN) : geo_tile_log_col(LOGN));
+  static constexpr int TILE_LOG = ROW ? geo_tile_log_row(LOGN) : geo_tile_log_col(LOGN);
   static constexpr int LOGGC = LOGA == 0 ? 0 : TILE_LOG - LOGA;  // columns per column tile
   static constexpr int LOGGR = TILE_LOG - LOGB;                  // rows per row tile
   static constexpr int TILE = 1 << TILE_LOG;
@@ -99,16 +91,16 @@ struct GeoT {
 //  fast  (m < 2^51): no reduction of the upper input, approximate Shoup product T in
 //        [0, 4m). Forward: each stage raises the bound by 4m, so a column pass (<= 8
 //        stages) starting below 2m (or 16m, see mid) ends below 48m and the row pass
-//        (<= 9 stages) below kFwdLazy m with a column start below 2m; 12 single-pass
-//        stages end below 50m. Inverse: canonical inputs; the k-th processed stage adds
+//        (<= 9 stages) below kFwdLazy m with a column start below 2m; 11 single-pass
+//        stages end below 46m. Inverse: canonical inputs; the k-th processed stage adds
 //        without reduction and biases the difference by m 2^(k+1) (>= the bound of both
 //        inputs), so after K stages all values are below m 2^(K+1) <= 2^13 m < 2^64.
 //  mid   (m < 2^60, the special primes): the same product; four bits of headroom, so the
 //        upper input is brought below 8m by one conditional subtraction on every other
 //        stage. Forward: even local stages take inputs below 16m (X < 8m after the
 //        subtraction, outputs below 12m), odd ones inputs below 12m (outputs below 16m).
-//        Inverse: values below 8m, one subtraction of 8m from the sum. Measured: 36 cycles per forward butterfly against
-//        43.8 for the exact form below.
+//        Inverse: values below 8m, one subtraction of 8m from the sum. Measured: 36 cycles
+//        per forward butterfly against 43.8 for the exact form below.
 //  exact (m < 2^62): Harvey's butterflies, forward values in [0, 4m), inverse in [0, 2m).
 enum { CLS_EXACT = 0, CLS_FAST = 1, CLS_MID = 2 };
 __device__ __forceinline__ int mod_class(u64 m) {

@@ -1,8 +1,7 @@
-// Row passes and the inverse column pass of the two-pass sizes on the register-tile core
-// (ks_core.cuh): the input and accumulator iNTTs, the key multiply, the ModDown row pass
-// and the plain forward row pass. One set of kernels per N serves every radix and column
-// tile a plan may name for these stages (a schedule's radix chooses the integer
-// basis-conversion column passes only; every schedule computes the same bits).
+// The kernels of the two-pass sizes on the register-tile core (ks_core.cuh): the input and
+// accumulator iNTTs, the basis conversions with the forward column pass, the key multiply,
+// the ModDown row pass and the plain forward passes. One set of kernels per N serves every
+// radix and column tile that a plan may name.
 #pragma once
 #include "ks_core.cuh"
 #include "ks_kern.cuh"
@@ -156,8 +155,9 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
 
 // ---------------------------------------------------------------------------
 // Inverse column pass, in place, with the per-limb scale; `pieces` writes the bf16 bytes
-// of the result for the tensor-core conversion instead (see store_pieces). Both
-// polynomials of which = 1 run side by side.
+// of the result for the tensor-core conversion (ks_tc.cu) instead: the limb's columns in
+// blocks of 2^tplog / N1, block after block; inside a block, point (y, g) at y * (columns per
+// block) + g, 16 bytes (eight bf16) per point. Both polynomials of which = 1 run side by side.
 template <int LOGN>
 struct ColGeo {
   static constexpr int LOGA = geo_loga(LOGN), LOGB = LOGN - LOGA;
