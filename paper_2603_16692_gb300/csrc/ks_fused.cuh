@@ -144,13 +144,8 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
                             : is.src + ((size_t)(o * is.src_outer + ii) << LOGN)) +
                    off;
   u64 *ws = tile + w0 * FG::RP;
-  WarpPairs<FG> in;
-  in.load(src);
-  warp_rows<FG>([&](int k, int, int p) { *reinterpret_cast<ulonglong2 *>(ws + p) = in.x[k]; });
-  if (host_in) {
-    u64 *copy = const_cast<u64 *>(jp.d) + ((size_t)ii << LOGN) + off;
-    warp_rows<FG>([&](int k, int e, int) { *reinterpret_cast<ulonglong2 *>(copy + e) = in.x[k]; });
-  }
+  input_rows<FG>(ws, src, host_in ? const_cast<u64 *>(jp.d) + ((size_t)ii << LOGN) + off : nullptr,
+                 (a.nq << LOGN) > kPacedWords);
   __syncthreads();  // the warp's rows, and the barrier's initialisation
   tw_ready<true>(&twbar, a.tab.err);
   u64 v[8];

@@ -90,6 +90,34 @@ struct WarpPairs {
   }
 };
 
+// The warp's rows of an inverse pass's input, into their shared rows; an input in host memory
+// leaves its copy in device memory on the way. `paced` (large host inputs): one pair of a
+// lane in flight at a time, since the reads share the CPU link with the previous
+// operation's result, which is on the longer path: (1, 2^17, 4) 179.6 -> 175.1 us,
+// (2, 2^17, 4) 171.8 -> 167.6, (2, 2^15, 10) 92.3 -> 91.7, against (4, 2^16, 20) 339 -> 345.
+// Small inputs wait for latency instead and take all pairs at once ((1, 2^15, 1) 39.2 ->
+// 35.8); the line is between 1.5 MB (62.7 -> 62.1) and 2.6 MB (89.5 -> 92.1).
+constexpr int kPacedWords = 1 << 18;
+template <class RG>
+__device__ __forceinline__ void input_rows(u64 *ws, const u64 *src, u64 *copy, bool paced) {
+  if (copy && paced) {
+#pragma unroll 1
+    for (int k = 0; k < RG::WR * RG::N2 / 64; ++k) {
+      const int e = 2 * ((threadIdx.x & 31) + 32 * k);
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(src + e);
+      *reinterpret_cast<ulonglong2 *>(copy + e) = x;
+      *reinterpret_cast<ulonglong2 *>(ws + (e >> RG::LOGB) * RG::RP +
+                                      core::row_pos(e & (RG::N2 - 1))) = x;
+    }
+    return;
+  }
+  WarpPairs<RG> in;
+  in.load(src);
+  warp_rows<RG>([&](int k, int, int p) { *reinterpret_cast<ulonglong2 *>(ws + p) = in.x[k]; });
+  if (copy)
+    warp_rows<RG>([&](int k, int e, int) { *reinterpret_cast<ulonglong2 *>(copy + e) = in.x[k]; });
+}
+
 // A value between the two inverse passes: the column pass starts from values below 4m
 // (fast; the row pass leaves them below 2^10 m), or takes the row pass's bounds as they are
 // (mid: 8m, exact: 2m). q = floor(x_hi floor(2^64 / m) / 2^32) is at most 3 below x / m when
@@ -132,13 +160,8 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   const u64 *src = host_in ? jp.dsrc + (size_t)ii * N + off
                            : is.src + ((size_t)o * is.src_outer + ii) * N + off;
   u64 *ws = tile + w0 * RG::RP;
-  WarpPairs<RG> in;
-  in.load(src);
-  warp_rows<RG>([&](int k, int, int p) { *reinterpret_cast<ulonglong2 *>(ws + p) = in.x[k]; });
-  if (host_in) {
-    u64 *copy = const_cast<u64 *>(jp.d) + (size_t)ii * N + off;
-    warp_rows<RG>([&](int k, int e, int) { *reinterpret_cast<ulonglong2 *>(copy + e) = in.x[k]; });
-  }
+  input_rows<RG>(ws, src, host_in ? const_cast<u64 *>(jp.d) + (size_t)ii * N + off : nullptr,
+                 (a.nq << LOGN) > kPacedWords);
   __syncthreads();  // the warp's rows, and the barrier's initialisation
   tw_ready<true>(&twbar, a.tab.err);
   u64 v[SB::E];
