@@ -83,8 +83,11 @@ struct GeoT {
   static constexpr int TWC = N1;                  // column-pass twiddles per tile
   // row-pass twiddles per tile: two-pass sizes hold N2 entries per row (the last unused)
   static constexpr int TWR = LOGA == 0 ? N2 - 1 : N2 * GR;
+  // ... in shared memory: a row's slab one entry longer, so that lanes on several rows of a
+  // tile read different banks
+  static constexpr int TWS = LOGA == 0 ? TWR : (N2 + 1) * GR;
   static constexpr int SMEM_COL = (N1 * PC) * 8 + TWC * 16;
-  static constexpr int SMEM_ROW = (N2 * PR) * 8 + TWR * 16;
+  static constexpr int SMEM_ROW = (N2 * PR) * 8 + TWS * 16;
 };
 
 // Butterflies by class of the modulus (mod_class):
@@ -209,8 +212,9 @@ __device__ __forceinline__ void ntt_round(u64 *s, const ulonglong2 *tw, u64 m) {
         const int half = 1 << (R - 1 - q);
         // twiddle index of local stage LS0+q, block (hi << q) + (u >> (R-q)); row tiles
         // with several rows (two-pass sizes) take the row-major slab
-        const ulonglong2 *twq = ROW ? (LOGG ? tw + (g << LOGM) : tw + (1 << (LS0 + q)) - 1 + (hi << q))
-                                    : tw + (1 << (LS0 + q)) + (hi << q);
+        const ulonglong2 *twq =
+            ROW ? (LOGG ? tw + g * ((1 << LOGM) + 1) : tw + (1 << (LS0 + q)) - 1 + (hi << q))
+                : tw + (1 << (LS0 + q)) + (hi << q);
 #pragma unroll
         for (int u = 0; u < (1 << R); ++u) {
           if (u & half) continue;
@@ -226,7 +230,7 @@ __device__ __forceinline__ void ntt_round(u64 *s, const ulonglong2 *tw, u64 m) {
         // row pass: the forward slab of the mirrored tile, row g' = G - 1 - g, block
         // c' = 2^ls - 1 - c (negated twiddles)
         const ulonglong2 *twq =
-            ROW ? (LOGG ? tw + (((1 << LOGG) - 1 - g) << LOGM)
+            ROW ? (LOGG ? tw + ((1 << LOGG) - 1 - g) * ((1 << LOGM) + 1)
                         : tw + (2 << (LS0 + q)) - 2 - (hi << q))
                 : tw + (1 << (LS0 + q)) + (hi << q);
         const u64 bias = m << (LOGM - (LS0 + q));
