@@ -41,40 +41,34 @@ UNIT = "KeySwitch/s"
 WORKLOADS = {"c1": W.C1, "c2": W.C2, "c3": W.C3}
 
 # Per-kernel DRAM bytes (read + write) per launch and pipe use, from the cold-cache ncu
-# launch list and the per-kernel --set full captures of one KeySwitch of the workload
-# (profile_case; summaries and commands in profiles/keyswitch_4_2e16_35_launches.md,
-# keyswitch_4_2e16_35_kernels_ncu.md and bconv_tc_4_2e16_35_ncu.md), one table per
-# captured plan, keyed by the kernel names of the library's profiler, so a change of the
-# dominant kernel still finds its row. In the split plan the key multiply's two launches
-# (P-limb and Q-limb targets) are averaged, as the profiler averages them. The integer
-# plan DPOB[km4,dnr4]-split and the tensor-core plan DPOB[km4]-tc (KS_BCONV_TC); pipe
-# use where a --set full capture exists.
+# launch list of one KeySwitch of the workload (profile_case; summary and commands in
+# profiles/keyswitch_4_2e16_35_launches.md), one table per captured plan, keyed by the kernel
+# names of the library's profiler, so a change of the dominant kernel still finds its row.
+# The integer plan DPOB and the tensor-core plan DPOB-tc (KS_BCONV_TC).
 NCU_PLANS = {
-    ("c3", "DPOB[km4,dnr4]-split"): {k: {"traffic": t, **pipes} for k, t, pipes in (
-        ("intt_row(d)", 57100000, {"issue_pct": 47.3, "fmaheavy_pct": 45.0, "alu_pct": 37.3}),
-        ("intt_col(d)", 19100000, {"issue_pct": 45.8, "fmaheavy_pct": 47.0, "alu_pct": 35.0}),
-        ("modup_col", 38400000, {"issue_pct": 59.8, "fmaheavy_pct": 69.0, "alu_pct": 48.3}),
-        ("modup_row_keymult", 176050000,
-         {"issue_pct": 54.1, "fmaheavy_pct": 55.0, "alu_pct": 37.2}),
-        ("intt_row(accP)", 18900000, {"issue_pct": 45.2, "fmaheavy_pct": 38.0, "alu_pct": 38.6}),
-        ("intt_col(accP)", 9500000, {"issue_pct": 45.0, "fmaheavy_pct": 41.0, "alu_pct": 37.1}),
-        ("moddown_col", 9600000, {"issue_pct": 58.2, "fmaheavy_pct": 66.0, "alu_pct": 46.0}),
-        ("moddown_row", 123700000, {"issue_pct": 51.7, "fmaheavy_pct": 52.0, "alu_pct": 44.7}))},
-    ("c3", "DPOB[km4]-tc"): {k: {"traffic": t, **pipes} for k, t, pipes in (
-        ("intt_row(d)", 57050000, {}),
-        ("intt_col(d)", 19080000, {}),
-        ("modup_col", 108350000,
-         {"issue_pct": 41.3, "tensor_pct": 8.9, "alu_pct": 29.1, "fma_pct": 27.9}),
-        ("modup_row_keymult", 361500000, {}),
-        ("intt_row(accP)", 18880000, {}),
-        ("intt_col(accP)", 9520000, {}),
-        ("moddown_col", 19190000,
-         {"issue_pct": 41.1, "tensor_pct": 9.1, "alu_pct": 28.5, "fma_pct": 27.5}),
-        ("moddown_row", 126320000, {}))},
+    ("c3", "DPOB"): {k: {"traffic": t, "issue_pct": i, "fmaheavy_pct": f, "alu_pct": a}
+                     for k, t, i, f, a in (
+        ("intt_row(d)", 57400000, 47, 46, 30), ("intt_col(d)", 19100000, 39, 50, 23),
+        ("modup_col", 42800000, 47, 65, 32), ("modup_row_keymult", 360400000, 55, 61, 41),
+        ("intt_row(accP)", 18900000, 44, 33, 30), ("intt_col(accP)", 9500000, 37, 36, 24),
+        ("moddown_col", 9800000, 54, 67, 34), ("moddown_row", 127900000, 58, 63, 45))},
+    ("c3", "DPOB-tc"): {k: {"traffic": t, "issue_pct": i, "fmaheavy_pct": f, "alu_pct": a,
+                            "tensor_pct": x} for k, t, i, f, a, x in (
+        ("intt_row(d)", 57300000, 46, 45, 30, 0), ("intt_col(d)", 19200000, 44, 42, 34, 0),
+        ("modup_col", 113500000, 45, 55, 29, 6),
+        ("modup_row_keymult", 360800000, 55, 61, 41, 0),
+        ("intt_row(accP)", 18900000, 45, 31, 28, 0), ("intt_col(accP)", 9500000, 42, 32, 33, 0),
+        ("moddown_col", 19300000, 40, 48, 25, 5), ("moddown_row", 127700000, 57, 63, 45, 0))},
 }
+# Plans with a radix schedule (tuned by earlier versions; the schedule names the same kernels
+# at this size); the split plan's key multiply is two launches, averaged as the profiler does.
+NCU_PLANS["c3", "DPOB[km4]-tc"] = NCU_PLANS["c3", "DPOB-tc"]
+NCU_PLANS["c3", "DPOB[km4,dnr4]-split"] = {
+    k: dict(r, traffic=r["traffic"] // 2) if k == "modup_row_keymult" else r
+    for k, r in NCU_PLANS["c3", "DPOB"].items()}
 # the column-pass kernels whose code depends on the tensor-core flags: a row for another
 # plan with the same flags stands for them (the other kernels' traffic depends on the
-# plan's split and schedule)
+# plan's split)
 TC_KERNELS = {"intt_col(d)": "up", "modup_col": "up", "intt_col(accP)": "down",
               "moddown_col": "down"}
 
@@ -724,7 +718,7 @@ def main():
                  "tuned_variant": ks.variant_name(variant, args.chunks),
                  "probe_ks_per_s_by_plan": {ks.variant_name(v, args.chunks): p_
                                             for v, p_ in probe_by_plan.items()},
-                 "chosen_by": "ks_tune (timed over dataflows x radices; with streams in "
+                 "chosen_by": "ks_tune (timed over dataflows and conversions; with streams in "
                                "flight, the tuned plan or the same without its split ModDown, "
                                "the faster on the probe)"
                  if args.variant.lower() == "tuned" else "--variant",
