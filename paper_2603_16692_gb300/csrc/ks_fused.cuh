@@ -266,12 +266,10 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
   fu_columns<FG>(v, colbuf, twc, m, cls, t, g, rank, ext, sync);
   cluster_arrive();
   cluster_wait();
-  WarpPairs<FG> acc;
-  acc.load(ac);
   fu_row<FG>(ext + row * FG::RP, twr + row * FG::N2, a.tab.mod[i], m, cls, t2, false);
   __syncwarp();
   const u64 *ws = ext + w0 * FG::RP;
-  scale_rows<FG>(jp, c, ws, acc, ((size_t)(c * a.nq + i) << LOGN) + woff, pv, m, cls);
+  scale_rows<FG>(jp, c, ws, ac, ((size_t)(c * a.nq + i) << LOGN) + woff, pv, m, cls, false);
   pdl_trigger();
 }
 

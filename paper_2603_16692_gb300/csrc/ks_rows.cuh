@@ -645,15 +645,32 @@ __global__ void __launch_bounds__(kKmGp * kKmGroups, 768 / (kKmGp * kKmGroups))
 // output, z the NTT's lazy values in ws: below kFwdLazy * m (fast butterflies) or, after one
 // conditional subtraction, below 8m (mid) or 2m (exact); acc + zb - z is then positive and
 // below (kFwdLazy + 1) m, 9m or 3m < 2^64, and the Shoup product by P^-1 takes any word.
+// paced (results to host memory, see input_rows): a pair at a time, so that the stores to the
+// CPU link spread over the kernel: (2, 2^15, 10) 91.7 -> 90.3 us, (2, 2^16, 4) 88.7 -> 87.0,
+// (2, 2^17, 4) the same, against (4, 2^16, 20) 345 -> 348.
 template <class RG>
 __device__ __forceinline__ void scale_rows(const JobPtr &jp, int c, const u64 *ws,
-                                           const WarpPairs<RG> &acc, size_t ob,
-                                           const ulonglong2 &pv, u64 m, int cls) {
+                                           const u64 *ac, size_t ob, const ulonglong2 &pv, u64 m,
+                                           int cls, bool paced) {
   const bool fast = cls == CLS_FAST;
   const u64 zs = cls == CLS_MID ? 8 * m : 2 * m, zb = fast ? kFwdLazy * m : zs;
   auto word = [&](u64 z, u64 x) {
     return csub(shoup(x + zb - (fast ? z : csub(z, zs)), pv.x, pv.y, m), m);
   };
+  if (paced) {  // (without addend)
+#pragma unroll 1
+    for (int k = 0; k < RG::WR * RG::N2 / 64; ++k) {
+      const int e = 2 * ((threadIdx.x & 31) + 32 * k);
+      const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(
+          ws + (e >> RG::LOGB) * RG::RP + core::row_pos(e & (RG::N2 - 1)));
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(ac + e);
+      *reinterpret_cast<ulonglong2 *>(jp.out + ob + e) =
+          make_ulonglong2(word(z.x, x.x), word(z.y, x.y));
+    }
+    return;
+  }
+  WarpPairs<RG> acc;
+  acc.load(ac);
   if ((jp.addmask >> c) & 1) {
     WarpPairs<RG> y;
     y.load(jp.add + ob);
@@ -717,10 +734,9 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   __syncwarp();
   core::put_row<SB>(s, v, t);
   __syncwarp();
-  WarpPairs<RG> acc;
-  acc.load(ac);
   const u64 *ws = tile + w0 * RG::RP;
-  scale_rows<RG>(jp, c, ws, acc, ((size_t)c * a.nq + i) * N + woff, pv, m, cls);
+  scale_rows<RG>(jp, c, ws, ac, ((size_t)c * a.nq + i) * N + woff, pv, m, cls,
+                 jp.dsrc && !jp.addmask && (a.nq << LOGN) > kPacedWords);
   pdl_trigger();
 }
 
