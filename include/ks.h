@@ -261,9 +261,13 @@ int ks_switch_host(ks_context *ctx, const uint64_t *d_host, const uint64_t *evk_
  * cudaHostRegister; anything else returns KS_EINVAL and launches nothing), 16-byte
  * aligned (else KS_EALIGN). The first kernel reads d_host over the CPU-GPU link and
  * the last one writes out_host; the result is there once `stream` has passed this call
- * (an event or a synchronize), and d_host must stay unmodified until then. Calls on one context share its staging
- * buffer and workspace, so they must be ordered (issued on one stream); consecutive
- * calls are chained like ks_switch's (N <= 2^11: cached graph replay). */
+ * (an event or a synchronize), and d_host must stay unmodified until then. d_host may be
+ * (part of) the result of an earlier call queued on `stream`; a kernel of the caller's own
+ * that writes it must not let its dependents launch early (programmatic dependent launch).
+ * Calls on one context share its staging buffer and workspace, so they must be ordered
+ * (issued on one stream); consecutive calls are chained like ks_switch's (N <= 2^11: cached
+ * graph replay), and read their input while the call before still writes its result where
+ * the two do not overlap. */
 int ks_switch_host_async(ks_context *ctx, const uint64_t *d_host, const uint64_t *evk_dev,
                          uint64_t *out_host, int variant, int chunks, void *stream);
 

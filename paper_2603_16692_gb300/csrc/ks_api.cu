@@ -422,6 +422,84 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
   return KS_OK;
 }
 
+// Which host-buffer operations may read their input before the operation queued ahead of them
+// on the stream is done. Their first kernel skips its wait for that operation's last kernel,
+// so that its host reads overlap that kernel's host writes ((2, 2^15, 10) from pinned buffers:
+// 94 us a call), which is sound only when the earlier operation does not write the words that
+// are read. The output of the last operation of each stream is kept here (a stream under
+// capture apart from the same stream outside it; operations before the last have completed
+// by then); an input that it overlaps, or a stream without an entry, is waited for.
+class InputOrder {
+  // A stream by its handle (the two names of the legacy stream as one, the per-thread stream
+  // by its thread too) and, under capture, the capture. (cudaStreamGetId would invalidate a
+  // capture. A handle that names a new stream finds the old one's entry, to no harm: what
+  // another stream has queued is waited for through events, which the launches keep.)
+  struct Key {
+    uintptr_t stream = 0, thread = 0;
+    unsigned long long capture = 0;
+    bool operator==(const Key &o) const {
+      return stream == o.stream && thread == o.thread && capture == o.capture;
+    }
+  };
+  struct Slot {
+    Key key;
+    unsigned long long used = 0;  // 0: free
+    uintptr_t lo = 0, hi = 0;
+  };
+  static constexpr int kSlots = 64;  // least recently used dropped
+  std::mutex mu_;
+  Slot slot_[kSlots];
+  unsigned long long clock_ = 0;
+
+  static bool key_of(cudaStream_t s, Key *k) {
+    static thread_local char tag;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamGetCaptureInfo(s, &st, &k->capture) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (st == cudaStreamCaptureStatusNone) k->capture = 0;
+    k->stream = s == cudaStreamLegacy ? 0 : (uintptr_t)s;
+    k->thread = s == cudaStreamPerThread ? (uintptr_t)&tag : 0;
+    return true;
+  }
+  Slot *find(const Key &k) {
+    for (Slot &x : slot_)
+      if (x.used && x.key == k) return &x;
+    return nullptr;
+  }
+
+ public:
+  // The operation just queued on s writes `bytes` bytes at p, and nothing else that the host
+  // may hand in as an input.
+  void wrote(cudaStream_t s, const void *p, size_t bytes) {
+    Key k;
+    if (!key_of(s, &k)) return;
+    std::lock_guard<std::mutex> lk(mu_);
+    Slot *x = find(k);
+    if (!x) {
+      x = slot_;
+      for (Slot &y : slot_)
+        if (y.used < x->used) x = &y;
+    }
+    x->key = k;
+    x->used = ++clock_;
+    x->lo = (uintptr_t)p;
+    x->hi = (uintptr_t)p + bytes;
+  }
+  // The operation queued on s writes several buffers: the next input is waited for.
+  void wrote_many(cudaStream_t s) { wrote(s, nullptr, ~(size_t)0); }
+  bool reads_ahead(cudaStream_t s, const void *p, size_t bytes) {
+    Key k;
+    if (!key_of(s, &k)) return false;
+    std::lock_guard<std::mutex> lk(mu_);
+    const Slot *x = find(k);
+    return x && ((uintptr_t)p + bytes <= x->lo || (uintptr_t)p >= x->hi);
+  }
+};
+
+InputOrder g_order;
+
 // Internal streams of ks_switch_batch.
 constexpr int kBatchStreams = 16;
 
@@ -1022,8 +1100,12 @@ int ks_switch(ks_context *c, const uint64_t *d, const uint64_t *evk, uint64_t *o
     const std::array<uintptr_t, 10> key = {
         0, (uintptr_t)plan_code(pl), (uintptr_t)pl.chunks, (uintptr_t)d, (uintptr_t)evk, 0,
         (uintptr_t)out, (uintptr_t)base, (uintptr_t)s, 0};
-    if (!use_graphs(c)) return run_plan(c, pl, js, s);
-    return cached_launch(c, key, s, [&](cudaStream_t q) { return run_plan(c, pl, js, q); });
+    const int r = use_graphs(c)
+                      ? cached_launch(c, key, s,
+                                      [&](cudaStream_t q) { return run_plan(c, pl, js, q); })
+                      : run_plan(c, pl, js, s);
+    g_order.wrote(s, out, 2 * (size_t)c->nq * c->N * 8);
+    return r;
   });
 }
 
@@ -1053,7 +1135,9 @@ int switch_launch_only(ks_context *c, const uint64_t *d, const uint64_t *evk, ui
   js.j[0].evk = (const u64 *)evk;
   js.j[0].out = (u64 *)out;
   js.j[0].ws = (u64 *)ws;
-  return run_plan(c, pl, js, (cudaStream_t)stream, false);
+  rc = run_plan(c, pl, js, (cudaStream_t)stream, false);
+  g_order.wrote((cudaStream_t)stream, out, 2 * (size_t)c->nq * c->N * 8);
+  return rc;
 }
 
 }  // namespace ks
@@ -1141,14 +1225,18 @@ int switch_host(ks_context *c, const uint64_t *d_host, const uint64_t *evk, uint
     const std::array<uintptr_t, 10> key = {
         3, (uintptr_t)plan_code(pl), (uintptr_t)pl.chunks, (uintptr_t)d_host, (uintptr_t)evk,
         (uintptr_t)din, (uintptr_t)out_host, (uintptr_t)base, (uintptr_t)s, 0};
-    if (async && !use_graphs(c)) return run_plan(c, pl, js, s);
-    return cached_launch(c, key, s, [&](cudaStream_t q) {
+    auto enqueue = [&](cudaStream_t q) {
+      // (a captured graph starts after all the work before it)
+      js.j[0].ahead = q == s && mapped && g_order.reads_ahead(s, d_map, in_b);
       if (!mapped) KS_TRY(cudaMemcpyAsync(din, d_host, in_b, cudaMemcpyHostToDevice, q));
       const int r = run_plan(c, pl, js, q);
       if (r) return r;
       if (!mapped) KS_TRY(cudaMemcpyAsync(out_host, dout, out_b, cudaMemcpyDeviceToHost, q));
       return (int)KS_OK;
-    });
+    };
+    const int r = async && !use_graphs(c) ? enqueue(s) : cached_launch(c, key, s, enqueue);
+    g_order.wrote(s, js.j[0].out, out_b);
+    return r;
   });
   if (rc || async) return rc;
   KS_TRY(cudaStreamSynchronize(s));
@@ -1242,7 +1330,9 @@ int ks_hmul(ks_context *c, const uint64_t *ct1, const uint64_t *ct2, const uint6
       KS_TRY(launch_tensor(c, (const u64 *)ct1, (const u64 *)ct2, (u64 *)out, d2, q));
       return run_plan(c, pl, js, q);
     };
-    return use_graphs(c) ? cached_launch(c, key, s, enqueue) : enqueue(s);
+    const int r = use_graphs(c) ? cached_launch(c, key, s, enqueue) : enqueue(s);
+    g_order.wrote(s, out, 2 * (size_t)c->nq * c->N * 8);
+    return r;
   });
 }
 
@@ -1273,7 +1363,9 @@ int ks_hrot(ks_context *c, const uint64_t *ct, uint32_t galois_elt, const uint64
       KS_TRY(launch_automorph(c, (const u64 *)ct, galois_elt, y0, y1, q));
       return run_plan(c, pl, js, q);
     };
-    return use_graphs(c) ? cached_launch(c, key, s, enqueue) : enqueue(s);
+    const int r = use_graphs(c) ? cached_launch(c, key, s, enqueue) : enqueue(s);
+    g_order.wrote(s, out, 2 * (size_t)c->nq * c->N * 8);
+    return r;
   });
 }
 
@@ -1292,6 +1384,7 @@ int ks_switch_batch(const ks_job *jobs, int njobs, int flags, void *stream) {
       return KS_EALIGN;
   }
   cudaStream_t s = (cudaStream_t)stream;
+  g_order.wrote_many(s);
   if (flags & KS_BATCH_PERSISTENT) return batch_persistent(jobs, njobs, flags, s);
   if (flags & KS_BATCH_TEST_STALL) return KS_EINVAL;
   // Groups of jobs sharing a context and a plan, in order of first appearance.

@@ -136,8 +136,8 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
   const int cls = mod_class(m);
   const ulonglong2 sc = is.scale[ii];
   // an input in host memory: see inv_row_body
-  const bool host_in = which == 0 && jp.dsrc;
-  if (!host_in) pdl_wait();
+  const bool host_in = which == 0 && jp.dsrc, ahead = host_in && jp.ahead;
+  if (!ahead) pdl_wait();
   const int row = threadIdx.x / FG::T2, t2 = threadIdx.x % FG::T2, w0 = row / FG::WR * FG::WR;
   const size_t off = (size_t)(rank * FG::RC + w0) << FG::LOGB;
   const u64 *src = (host_in ? jp.dsrc + ((size_t)ii << LOGN)
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(FuGeo<LOGN>::NT)
 #pragma unroll
   for (int u = 0; u < 8; ++u)
     d[(size_t)(u * FG::T1 + t) << FG::LOGB] = csub(shoup(v[u], sc.x, sc.y, m), m);
-  if (host_in) pdl_wait();
+  if (ahead) pdl_wait();
   pdl_trigger();
 }
 

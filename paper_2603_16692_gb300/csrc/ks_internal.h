@@ -72,6 +72,8 @@ struct JobPtr {
   u64 *ws;         // this job's workspace
   const u64 *add;  // optional addend [2][L+1][N] (may alias out): out_c += add_c when
   int addmask;     // bit c of addmask is set (HMUL / HROT epilogues); 0 = plain store
+  int ahead;       // dsrc may be read before the previous operation on the stream is done
+                   // (InputOrder in ks_api.cu)
   const u64 *dsrc; // optional: the input in (pinned, device-mapped) host memory; the
                    // input iNTT reads it and leaves a device copy in d
 };

@@ -437,10 +437,11 @@ __device__ __forceinline__ void inv_row_body(const KArgs &a, const JobPtr &jp, c
                           &twbar);
   // Reading the input from host memory (`dsrc`), this pass writes only v and the device
   // copy of d, which no kernel of the previous operation on the stream reads once its
-  // last kernel runs: it starts without waiting, so its host reads overlap that kernel's
-  // host writes, and waits for it at the end (keeping the chain's order for what follows).
-  const bool host_in = which == 0 && jp.dsrc;
-  if (!host_in) pdl_wait();
+  // last kernel runs. Where that operation does not write the input either (`ahead`), it
+  // starts without waiting, so its host reads overlap that kernel's host writes, and waits
+  // for it at the end (keeping the chain's order for what follows).
+  const bool ahead = which == 0 && jp.dsrc && jp.ahead;
+  if (!ahead) pdl_wait();
   const ulonglong2 sc = is.scale[ii];
   const int o0 = only_o < 0 ? 0 : only_o, o1 = only_o < 0 ? is.outer : only_o + 1;
   for (int o = o0; o < o1; ++o) {
@@ -465,7 +466,7 @@ __device__ __forceinline__ void inv_row_body(const KArgs &a, const JobPtr &jp, c
     }
     __syncthreads();
   }
-  if (host_in) pdl_wait();
+  if (ahead) pdl_wait();
 }
 
 // Grid row of an inverse-NTT launch: the limb, and with `split` the polynomial too

@@ -152,10 +152,10 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   const u64 m = mi.m, mu = mi.mu;
   constexpr size_t N = (size_t)1 << LOGN;
   stage_row_tw<RG>(tws, a.tab.twr_f, prime, RG::N1 / RG::GR - 1 - blk, &twbar);
-  // (see inv_row_body: an input in host memory is read without waiting for the
-  // predecessor, which is waited for at the end)
-  const bool host_in = which == 0 && jp.dsrc;
-  if (!host_in) pdl_wait(a.early);
+  // (see inv_row_body: an input in host memory that the predecessor does not write is read
+  // without waiting for it; it is waited for at the end)
+  const bool host_in = which == 0 && jp.dsrc, ahead = host_in && jp.ahead;
+  if (!ahead) pdl_wait(a.early);
   const size_t off = ((size_t)(r0 + w0) << RG::LOGB);
   const u64 *src = host_in ? jp.dsrc + (size_t)ii * N + off
                            : is.src + ((size_t)o * is.src_outer + ii) * N + off;
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(128, row_blocks(LOGN))
   u64 *d = is.dst + ((size_t)o * is.dst_outer + ii) * N + ((size_t)(r0 + row) << RG::LOGB);
 #pragma unroll
   for (int u = 0; u < SB::E; ++u) d[(u << SB::LOGT) + t] = inv_between(v[u], m, mu, cls);
-  if (host_in) pdl_wait(a.early);
+  if (ahead) pdl_wait(a.early);
   pdl_trigger();
 }
 
