@@ -253,19 +253,34 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
   const bool oc = pl.base == KS_DSOC || pl.base == KS_DPOC;
   auto dsize = [&](int j) { return std::min(c->nq, (j + 1) * c->alpha) - j * c->alpha; };
 
-  // Small sizes: the four steps as one cluster kernel each. (While the profiler is on, the
-  // stages run as their own launches, which it times.)
-  if (pl.base == KS_DPOB && !pl.unfused && !pl.tc_down && !split && !g_prof.on &&
-      fused_rule(c, js.n)) {
-    KS_TRY(c->fu->run(c, js, wo, s));
+  // An iNTT (which = 0: the input, 1: the P-limbs) as one cluster kernel.
+  auto fused_inv = [&](int which) {
+    const double nl = which == 0 ? c->nq : 2.0 * c->np;
+    return timed(which == 0 ? "fused_intt(d)" : "fused_intt(accP)", 2 * nl * W,
+                 nl * (BF_A + BF_B + NJ), 0, s, [&] { return c->fu->inv(c, js, wo, which, s); });
+  };
+
+  // Small sizes: the four steps as one cluster kernel each.
+  if (pl.base == KS_DPOB && !pl.unfused && !pl.tc_down && !split && fused_rule(c, js.n)) {
+    const double nq = c->nq, nkey = 2.0 * c->beta * c->qp, nconv = c->beta * c->qp - nq;
+    double up = 0;  // ModUp's terms, one reduction per output among them
+    for (int j = 0; j < c->beta; ++j) up += (double)(c->qp - dsize(j)) * (dsize(j) + 1);
+    const double km = nkey + nq, dn = 2 * nq * (c->np + 1.0);
+    KS_TRY(fused_inv(0));
+    KS_TRY(timed("fused_modup_keymult", (nkey + 2 * nq + 2 * c->qp) * W,
+                 (up + km) * NJ + nconv * (BF_A + BF_B), (up + km) * NJ, s,
+                 [&] { return c->fu->up(c, js, wo, s); }));
+    KS_TRY(fused_inv(1));
+    KS_TRY(timed("fused_moddown", (4 * nq + 2 * c->np) * W,
+                 dn * NJ + 2 * nq * (BF_A + BF_B + NJ), dn * NJ, s,
+                 [&] { return c->fu->down(c, js, wo, s); }));
     return KS_OK;
   }
 
-  // Input iNTT, fused with the per-limb factor N^-1 * Qhat_{j,i}^-1 of the ModUp BConv.
-  // one cluster kernel where the size has it (its stages on their own while profiling)
-  const bool fuinv = c->fu && !g_prof.on;
-  if (fuinv && !pl.tc_up) {
-    KS_TRY(c->fu->inv(c, js, wo, 0, s));
+  // Input iNTT, fused with the per-limb factor N^-1 * Qhat_{j,i}^-1 of the ModUp BConv; one
+  // cluster kernel where the size has it.
+  if (c->fu && !pl.tc_up) {
+    KS_TRY(fused_inv(0));
   } else {
     const double nl = c->nq;
     KS_TRY(timed("intt_row(d)", 2 * nl * W, nl * (BF_B + (single ? NJ : 0)), 0, s,
@@ -365,8 +380,8 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
   }
 
   // iNTT of the P-limbs of both accumulators, fused with N^-1 * Phat_k^-1.
-  if (fuinv && !pl.tc_down) {
-    KS_TRY(c->fu->inv(c, js, wo, 1, s));
+  if (c->fu && !pl.tc_down) {
+    KS_TRY(fused_inv(1));
   } else {
     const double nl = 2.0 * c->np;
     KS_TRY(timed("intt_row(accP)", 2 * nl * W, nl * (BF_B + (single ? NJ : 0)), 0, s,

@@ -313,27 +313,25 @@ struct FusedFns {
     if ((e = smem_attr(k_fu_down<LOGN>, FG::smem_inv()))) return e;
     return smem_attr(k_fu_up<LOGN>, kSmemMax);
   }
-  static cudaError_t run(const ks_context *c, const JobSet &js, const WsOff &wo,
-                         cudaStream_t s) {
-    const KArgs a = args_of(c);
+  static cudaError_t up(const ks_context *c, const JobSet &js, const WsOff &wo,
+                        cudaStream_t s) {
     const int G = groups(c->beta);
-    cudaError_t e;
-    if ((e = inv(c, js, wo, 0, s))) return e;
-    if ((e = launch_cluster(k_fu_up<LOGN>, dim3(kFuC, c->qp, js.n), G * FG::NT,
-                            FG::smem_up(c->beta, G), s, a, js, wo)))
-      return e;
-    if ((e = inv(c, js, wo, 1, s))) return e;
+    return launch_cluster(k_fu_up<LOGN>, dim3(kFuC, c->qp, js.n), G * FG::NT,
+                          FG::smem_up(c->beta, G), s, args_of(c), js, wo);
+  }
+  static cudaError_t down(const ks_context *c, const JobSet &js, const WsOff &wo,
+                          cudaStream_t s) {
     return launch_cluster(k_fu_down<LOGN>, dim3(kFuC, 2 * c->nq, js.n), FG::NT, FG::smem_inv(), s,
-                          a, js, wo);
+                          args_of(c), js, wo);
   }
   static const FusedTable &table() {
-    static const FusedTable t = {&prepare, &fits, &run, &inv};
+    static const FusedTable t = {&prepare, &fits, &up, &down, &inv};
     return t;
   }
   // only the inverse transform
   static bool no_fit(int) { return false; }
   static const FusedTable &table_inv() {
-    static const FusedTable t = {&prepare_inv, &no_fit, nullptr, &inv};
+    static const FusedTable t = {&prepare_inv, &no_fit, nullptr, nullptr, &inv};
     return t;
   }
 };

@@ -251,13 +251,15 @@ struct LaunchTable {
   cudaError_t (*ntt_row)(const ks_context *, const JobSet &, const WsOff &, const Tasks &,
                          int buf, cudaStream_t);
 };
-// The cluster kernels of a small N (ks_fused.cuh). run: a whole fused DPOB KeySwitch in four
-// launches, if fits (a target's digits in a CTA's shared memory; never at sizes that have
-// the inverse transform only).
+// The cluster kernels of a small N (ks_fused.cuh). inv, up, inv and down are a whole fused
+// DPOB KeySwitch, if fits (a target's digits in a CTA's shared memory; never at sizes that
+// have the inverse transform only).
 struct FusedTable {
   cudaError_t (*prepare)();
   bool (*fits)(int beta);
-  cudaError_t (*run)(const ks_context *, const JobSet &, const WsOff &, cudaStream_t);
+  // ModUp (conversion and NTT) and key multiply; ModDown's conversion, NTT and scaling
+  cudaError_t (*up)(const ks_context *, const JobSet &, const WsOff &, cudaStream_t);
+  cudaError_t (*down)(const ks_context *, const JobSet &, const WsOff &, cudaStream_t);
   // rows, columns and scale of one iNTT set (intt_row + intt_col)
   cudaError_t (*inv)(const ks_context *, const JobSet &, const WsOff &, int which, cudaStream_t);
 };
