@@ -195,7 +195,7 @@ int ks_workspace_size(const ks_context *ctx, int variant, int chunks, size_t *by
  *           KS_STAGE_RADIX(..) | KS_COLALT_* | KS_SPLIT_DOWN | KS_BCONV_TC |
  *           KS_BCONV_TC_DOWN), or KS_AUTO (the plan ks_tune chose for this context,
  *           else the one ks_select chose, else DPOB fused; the last two with
- *           KS_BCONV_TC added where ks_info.tc = 1 and (beta QP + L+1) alpha N is at least
+ *           KS_BCONV_TC added where ks_info.tc = 1 and (L+1) (QP + alpha) N is at least
  *           7 * 2^20 per conversion launch: 2 for DPOB, beta + 1 for DSOB, chunks times as
  *           many for DPOC and DSOC. KS_AUTO leaves that addition out when the scratch at
  *           hand, or the device, holds the plan only without it)

@@ -53,20 +53,26 @@ constexpr int kSchedMask = 0x3ff << KS_STAGE_SHIFT;
 // takes without a tuned one: per conversion launch (ModUp and ModDown, per digit and group
 // where the dataflow splits them), the products of a source and a target residue that leave
 // the integer pipes have to outweigh the launch's start-up and the wider intermediate.
-// Measured (integer / tensor-core, us; products per launch in 2^20):
-//   DPOB (2,2^15,10) 4.2 64.1 / 72.6, (3,2^14,18) 5.3 63.7 / 66.7, (4,2^16,35) level 7 7.0
-//   109.3 / 111.1, level 8 7.6 112.6 / 108.7, (4,2^15,19) 9.4 117.5 / 112.8, (7,2^14,30)
-//   11 112.9 / 107.1, (9,2^14,52) 27 216.6 / 184.1, (8,2^16,60) 153 905 / 693
+// Measured (integer / tensor-core, us; products per launch in 2^20, every digit with the limbs
+// it has at this level):
+//   DPOB (2,2^15,10) 4.0 64.1 / 72.6, (3,2^14,18) 4.9 63.7 / 66.7, (4,2^15,19) 9.4 117.5 /
+//   112.8, (7,2^14,30) 9.9 114.8 / 106.1, (9,2^14,52) 27 216.6 / 184.1, (8,2^16,60) 147
+//   905 / 693; (4,2^16,35) at level 7 6.5 101.5 / 104.4, 8 7.6 108.8 / 111.2, 9 8.8 127.8 /
+//   131.6, 11 11 140.4 / 137.4, 13 14 151.5 / 146.4; short last digits: (4,2^14,35) level 19
+//   5.9 67.1 / 74.5, (4,2^16,21) level 8 5.9 100.2 / 105.0, (10,2^17,40) level 6 7.4 163.7 /
+//   171.7, (7,2^14,36) level 24 7.2 86.7 / 85.6
 //   DSOB (2,2^15,17) 6.8 108.7 / 116.3, (3,2^15,26) 9.5 177 / 167.5
-//   DPOC (7,2^14,30) 5.5 125.3 / 135.0, (10,2^13,60) 9.2 147.9 / 143.4
+//   DPOC (7,2^14,30) 5.0 125.3 / 135.0, (10,2^13,60) 8.9 147.9 / 143.4
 //   DSOC (3,2^15,26) 4.7 199 / 233, (2,2^16,17) 6.8 233.8 / 227.7
+// Between 7 and 10 either side is ahead by up to 5%, by the size.
 constexpr double kTcWork = 7 << 20;
 int tc_rule(const ks_context *c, int base, int chunks) {
   const bool dp = base == KS_DPOB || base == KS_DPOC, oc = base == KS_DSOC || base == KS_DPOC;
   const int groups = oc ? (chunks ? chunks : 2) : 1;
-  const double targets = (double)c->beta * c->qp + c->nq;  // each digit's others, ModDown's
+  // each input limb onto the QP limbs, ModDown's alpha sources onto the L+1
+  const double products = (double)c->nq * (c->qp + c->alpha) * c->N;
   const double launches = (double)groups * ((dp ? 1 : c->beta) + 1);
-  return c->tc_ap > 0 && targets * c->alpha * c->N >= kTcWork * launches ? KS_BCONV_TC : 0;
+  return c->tc_ap > 0 && products >= kTcWork * launches ? KS_BCONV_TC : 0;
 }
 
 // The cluster kernels (ks_fused.cuh) serve the plain fused DPOB plan when they have the
