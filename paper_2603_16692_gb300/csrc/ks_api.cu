@@ -861,11 +861,34 @@ int with_workspace(ks_context *c, void *ws, size_t ws_bytes, size_t need, F fn) 
   return fn((u64 *)c->ws);
 }
 
+// Whether the device has room for an arena of `need` bytes in the place of one of `have`.
+// Asked before a plan that can do with less (Plan::ruled) gives its arena up to grow it: an
+// allocation that fails then would cost a synchronisation, a release and two allocations on
+// every call, and no call could be captured.
+bool can_grow(size_t have, size_t need) {
+  size_t room = 0, total = 0;
+  if (have >= need) return true;
+  if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return need <= have + room;
+}
+
 // with_workspace for plan pl (made from variant, chunks) and `extra` words; when the arena
 // cannot grow to it, pl again without the tensor-core conversions that tc_rule added.
 template <class F>
 int with_plan(ks_context *c, int variant, int chunks, Plan &pl, void *ws, size_t ws_bytes,
               size_t extra, F fn) {
+  if (!ws && pl.ruled) {
+    std::unique_lock<std::mutex> lk(c->ws_mu);
+    const size_t have = c->ws_bytes;
+    lk.unlock();
+    if (!can_grow(have, (pl.total + extra) * 8)) {
+      const int rc = make_plan(c, variant, chunks, &pl, 0);
+      if (rc) return rc;
+    }
+  }
   int rc = with_workspace(c, ws, ws_bytes, (pl.total + extra) * 8, fn);
   if (rc != KS_ENOMEM || !pl.ruled) return rc;
   rc = make_plan(c, variant, chunks, &pl, 0);
@@ -1469,6 +1492,7 @@ int ks_switch_batch(const ks_job *jobs, int njobs, int flags, void *stream) {
   int prc = plan_groups(~(size_t)0);
   if (prc) return prc;
   std::lock_guard<std::mutex> lk(g_batch.mu);
+  if (!can_grow(g_batch.arena_bytes, total) && (prc = plan_groups(0))) return prc;
   if (g_batch.arena_bytes < total) {
     if (g_batch.arena) {
       cudaDeviceSynchronize();
