@@ -102,10 +102,11 @@ u64 neg_inv64(u64 m) {
   return (u64)0 - x;
 }
 
+// f(0..n-1), on the host's threads unless there is too little to do (`serial`).
 template <class F>
-void par_for(int n, F f) {
+void par_for(int n, bool serial, F f) {
   unsigned hw = std::thread::hardware_concurrency();
-  int nt = std::max(1, std::min<int>(n, hw ? (int)hw : 4));
+  int nt = serial ? 1 : std::max(1, std::min<int>(n, hw ? (int)hw : 4));
   if (nt <= 1) {
     for (int i = 0; i < n; ++i) f(i);
     return;
@@ -136,7 +137,7 @@ int build_tables(ks_context *c) {
   std::vector<ulonglong2> iscale_q(nq), iscale_p(np), pinv(nq), pmod(nq);
   std::vector<u64> cup((size_t)beta * QP * alpha, 0), cdown((size_t)nq * alpha, 0);
 
-  par_for(QP, [&](int t) {
+  par_for(QP, false, [&](int t) {
     const u64 m = c->mods[t];
     ModInfo mi;
     mi.m = m;
@@ -251,7 +252,9 @@ int build_tables(ks_context *c) {
     for (int t = 0; t < QP; ++t) fix[t] = invm(((u64)1 << 32) % c->mods[t], c->mods[t]);
     bup.assign((size_t)beta * QP * blk, 0);
     bdown.assign((size_t)nq * blk, 0);
-    par_for(QP, [&](int t) {
+    // starting 16 threads takes as long as some 2,000 constants: (2, 2^13, 7) context 1.95 ms
+    // with them, 1.40 without; (2, 2^15, 10) 5.9 and 4.75
+    par_for(QP, (size_t)beta * QP * alpha < 2048, [&](int t) {
       for (int j = 0; j < beta; ++j) {
         const int lo = j * alpha, ns = std::min(nq, lo + alpha) - lo;
         fill(&bup[((size_t)j * QP + t) * blk], &cup[((size_t)j * QP + t) * alpha], ns, fix[t],
