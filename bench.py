@@ -105,15 +105,30 @@ def measured_alu(ks, stream):
     return bf, mac
 
 
+def tensor_peak(peaks):
+    """The sustained cuBLAS bf16 rate (FLOP/s): the kernels run inside a long step."""
+    return float(peaks.get("bf16_tflops_sustained", 1700.0)) * 1e12
+
+
+def tensor_flops(stat):
+    """The tensor-core FLOPs of a kernel's launches. The library counts the 16 sums per
+    target of a full byte product; the MMAs form eight of them."""
+    return 0.5 * (stat.get("tensor_flops") or 0)
+
+
+def tensor_ceil_ms(stats, reps, peaks):
+    """Tensor-core time of a step at the peak rate, from `reps` profiled steps."""
+    return sum(tensor_flops(s) for s in stats) / reps / tensor_peak(peaks) * 1e3
+
+
 def tensor_roofline(dom, per_launch_ms, peaks):
     """The tensor-core part of a kernel (the basis conversions of KS_BCONV_TC plans), or
     None: its bf16 FLOPs against the measured sustained cuBLAS bf16 rate (the kernel runs
     inside a long step)."""
     if not dom.get("tensor_flops"):
         return None
-    # the library counts 16 sums per target; the MMAs form eight of them
-    fl = 0.5 * dom["tensor_flops"] / dom["launches"]
-    pk = float(peaks.get("bf16_tflops_sustained", 1700.0)) * 1e12
+    fl = tensor_flops(dom) / dom["launches"]
+    pk = tensor_peak(peaks)
     return {"flops_per_launch": fl, "achieved": fl / (per_launch_ms / 1e3) / 1e12,
             "peak": pk / 1e12, "unit": "TFLOP/s", "frac": fl / pk * 1e3 / per_launch_ms,
             "t_ceil_ms": fl / pk * 1e3,
@@ -973,8 +988,7 @@ def main():
         "ks_alu_roofline": {"bound": "alu", "t_ceil_ms": t_ceil_step, "ms_per_step": step_ms,
                             "frac": t_ceil_step / step_ms,
                             "one_stream_frac": t_ceil_step / one_stream_ms,
-                            "tensor_t_ceil_ms": sum(x.get("tensor_flops", 0) for x in stats)
-                            / kprof / (float(peaks.get("bf16_tflops_sustained", 1700.0)) * 1e9),
+                            "tensor_t_ceil_ms": tensor_ceil_ms(stats, kprof, peaks),
                             "what": "the whole KeySwitch's integer arithmetic at the measured "
                                     "ceiling (the products of tensor-core conversions apart: "
                                     "tensor_t_ceil_ms at the sustained bf16 rate)"},
