@@ -2,29 +2,26 @@
 // arithmetic on this GPU, measured with every SM busy and no memory traffic. They
 // give a measured denominator for the integer-bound kernels beside the one derived
 // from unit counts and clocks.
-//   KS_CAL_BUTTERFLY: forward lazy butterflies with the approximate Shoup product
-//                     (the NTT inner operation for moduli below 2^51).
-//   KS_CAL_MAC:       exact 64x64->128-bit multiply-accumulates (the basis-conversion
-//                     and key-multiply inner operation), one REDC per 8 terms.
+//   KS_CAL_BUTTERFLY: the forward butterfly of the moduli below 2^51 (bfly_fwd_c), nothing
+//                     between stages.
+//   KS_CAL_MAC:       the exact multiply-accumulates of the basis conversions and the key
+//                     multiply (Mac3), one reduction per 8 terms.
+// (Before, with a conditional subtraction per butterfly and the 128-bit carry chain of the
+// single-pass kernels, they read 0.905 T butterflies and 1.33 T terms a second, which the
+// two-pass kernels exceed; now 1.126 T and 1.909 T on a GB300 at 2070 MHz.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "ks_arith.cuh"
 #include "ks_internal.h"
+#include "ks_ntt.cuh"
 
 namespace ks {
 namespace {
 
 constexpr int kCalThreads = 256;
 constexpr int kChains = 8;  // independent dependency chains per thread
-
-__device__ __forceinline__ void bfly(u64 &a, u64 &b, u64 w, u64 wp, u64 m, u64 m4) {
-  const u64 t = shoup4(b, w, wp, m);
-  const u64 x = a;
-  a = x + t;
-  b = x - t + m4;
-}
 
 __global__ void __launch_bounds__(kCalThreads) k_cal_butterfly(u64 m, u64 w, u64 wp, int iters,
                                                                u64 *sink) {
@@ -34,14 +31,10 @@ __global__ void __launch_bounds__(kCalThreads) k_cal_butterfly(u64 m, u64 w, u64
     a[c] = (threadIdx.x * 7919ull + c * 104729ull + blockIdx.x) % m;
     b[c] = (threadIdx.x * 15485863ull + c * 32452843ull) % m;
   }
-  const u64 m4 = 4 * m;
+  const ulonglong2 tw = make_ulonglong2(w, wp);
   for (int it = 0; it < iters; ++it) {
 #pragma unroll
-    for (int c = 0; c < kChains; ++c) {
-      bfly(a[c], b[c], w, wp, m, m4);
-      // keep the values bounded like a transform does between stages
-      a[c] = a[c] >= m4 ? a[c] - m4 : a[c];
-    }
+    for (int c = 0; c < kChains; ++c) bfly_fwd_c<CLS_FAST>(a[c], b[c], tw, m, 0);
   }
   u64 acc = 0;
 #pragma unroll
@@ -57,13 +50,14 @@ __global__ void __launch_bounds__(kCalThreads) k_cal_mac(u64 m, u64 minv, u64 c0
     x[c] = (threadIdx.x * 7919ull + c * 104729ull + blockIdx.x) % m;
     z[c] = 0;
   }
+  const uint32_t inv = 0u - (uint32_t)minv;
   for (int it = 0; it < iters; ++it) {
 #pragma unroll
     for (int c = 0; c < kChains; ++c) {
-      U128 acc = {0, 0};
+      Mac3 acc = {};
 #pragma unroll
-      for (int k = 0; k < 8; ++k) mac128(acc, x[c] + k, c0 + k);
-      z[c] += redc(acc, m, minv);
+      for (int k = 0; k < 8; ++k) acc.add(x[c] + k, c0 + k);
+      z[c] += acc.reduce(m, inv);
       x[c] = z[c] & ((1ull << 49) - 1);
     }
   }
