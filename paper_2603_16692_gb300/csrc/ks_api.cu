@@ -83,7 +83,7 @@ int tc_rule(const ks_context *c, int base, int chunks) {
 // 31.9 / 33.2, (2, 2^13, 11) 36.0 / 37.3; beyond: (4, 2^13, 15) 44.7 / 39.7,
 // (6, 2^13, 44) 119 / 87; (7, 2^14, 30) 154 / 130, (2, 2^15, 10) 88 / 64.
 bool fused_rule(const ks_context *c, int jobs) {
-  return c->fu && c->fu->fits(c->beta) && 8 * c->qp * jobs <= 152;
+  return c->fu && c->fu->fits(c->beta) && 8 * c->qp * jobs <= kSms;
 }
 
 // room: words of scratch there are. A KS_AUTO plan whose tensor-core conversions tc_rule

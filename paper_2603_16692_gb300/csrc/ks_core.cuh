@@ -1,4 +1,4 @@
-// Register-tile NTT core of the two-pass sizes (N >= 2^13, device side).
+// Register-tile NTT core of the two-pass sizes (N >= 2^12, device side).
 //
 // A thread holds E = 2^RL points of one sub-transform (a row or a column) of M = 2^LOGM
 // points; T = M / E threads share it. The LOGM stages run as RL stages in registers, one

@@ -16,6 +16,8 @@ namespace ks {
 
 struct FusedTable;
 
+// SMs of a GB300: the launch rules' lines (fused_rule, early_rule) are a wave on them.
+constexpr int kSms = 152;
 constexpr int kMaxLimbs = 256;   // QP limit (L+1 <= 128, alpha <= 128)
 
 // Per-modulus constants (device).

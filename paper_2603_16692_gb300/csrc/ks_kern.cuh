@@ -1087,7 +1087,7 @@ inline KArgs args_of(const ks_context *c) { return make_args(c); }
 // have all started (see pdl_trigger): when it is more than a wave at the kernels' 768
 // threads per SM. (Half of that: (4, 2^16, 35) in four chunks 672 -> 716 us, whose launches
 // are about a wave; twice: (4, 2^16, 35) 344 -> 349 us.)
-inline int early_rule(size_t threads) { return threads > (size_t)152 * 768 ? 1 : 0; }
+inline int early_rule(size_t threads) { return threads > (size_t)kSms * 768 ? 1 : 0; }
 
 // launch_pdl of a kernel whose first argument is its KArgs, with the early rule applied.
 template <class... KT, class... AT>

@@ -43,9 +43,6 @@ __host__ __device__ constexpr int geo_tile_log_col(int logn) {
 __host__ __device__ constexpr int geo_tile_log_row(int logn) {
   return logn <= 11 ? logn : (logn <= 15 ? 9 : 10);
 }
-__host__ __device__ constexpr int geo_loggr(int logn) {
-  return geo_tile_log_row(logn) - (logn - geo_loga(logn));
-}
 
 // Entry of (local stage ls, block c) in a row's twiddle slab of the two-pass sizes: the
 // first kRowHead stages stage-major, then, for the 2^kRowHead sub-blocks of a row that one
@@ -186,14 +183,11 @@ __device__ __forceinline__ u64 mac_reduce(Mac3 &s, const ModInfo &mi, u64 m, uin
   return csub(redc(U128{s.lo, s.hi}, m, mi.minv), m);
 }
 
-// SPLIT: the block runs several tiles side by side, NT threads each (NT a power of
-// two); a thread works on the tile of its group of NT (the caller picks s, tw, m).
-template <int LOGM, int LOGG, int P, int NT, bool ROW, bool INV, int LS0, int R, int CLS,
-          bool SPLIT = false>
+template <int LOGM, int LOGG, int P, int NT, bool ROW, bool INV, int LS0, int R, int CLS>
 __device__ __forceinline__ void ntt_round(u64 *s, const ulonglong2 *tw, u64 m) {
   constexpr int SUB = LOGM - LS0 - R;
   constexpr int NG = 1 << (LOGM - R + LOGG);
-  const int tid = SPLIT ? (int)(threadIdx.x & (NT - 1)) : (int)threadIdx.x;
+  const int tid = threadIdx.x;
 #pragma unroll
   for (int it = 0; it < (NG + NT - 1) / NT; ++it) {
     const int grp = tid + it * NT;
@@ -254,27 +248,22 @@ __device__ __forceinline__ void ntt_round(u64 *s, const ulonglong2 *tw, u64 m) {
   }
 }
 
+// Barrier of BARN threads of the block (the others run another role or another group).
+template <int BARN>
+__device__ __forceinline__ void round_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(BARN) : "memory");
+}
+
 // Forward stages 0..LOGM-1 of every sub-transform in the tile, in rounds of at
 // most RM stages (bounds: see the butterflies). Caller syncs before; each round syncs
 // after.
-// Barrier after a round: the whole block (BARN = 0), or named barrier `id` over BARN
-// threads (a group of the block; the others run another role or another group).
-template <int BARN>
-__device__ __forceinline__ void round_sync(int id = 1) {
-  if constexpr (BARN == 0)
-    __syncthreads();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(BARN) : "memory");
-}
-
-template <int LOGM, int LOGG, int P, int NT, bool ROW, int RM, int CLS, int LS0 = 0,
-          bool SPLIT = false, int BARN = 0>
-__device__ __forceinline__ void tile_fwd_t(u64 *s, const ulonglong2 *tw, u64 m, int bar_id = 1) {
+template <int LOGM, int LOGG, int P, int NT, bool ROW, int RM, int CLS, int LS0 = 0>
+__device__ __forceinline__ void tile_fwd_t(u64 *s, const ulonglong2 *tw, u64 m) {
   if constexpr (LS0 < LOGM) {
     constexpr int R = (LOGM - LS0) >= RM ? RM : (LOGM - LS0);
-    ntt_round<LOGM, LOGG, P, NT, ROW, false, LS0, R, CLS, SPLIT>(s, tw, m);
-    round_sync<BARN>(bar_id);
-    tile_fwd_t<LOGM, LOGG, P, NT, ROW, RM, CLS, LS0 + R, SPLIT, BARN>(s, tw, m, bar_id);
+    ntt_round<LOGM, LOGG, P, NT, ROW, false, LS0, R, CLS>(s, tw, m);
+    __syncthreads();
+    tile_fwd_t<LOGM, LOGG, P, NT, ROW, RM, CLS, LS0 + R>(s, tw, m);
   }
 }
 

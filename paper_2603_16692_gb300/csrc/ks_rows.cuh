@@ -131,8 +131,8 @@ __device__ __forceinline__ u64 inv_between(u64 x, u64 m, u64 mu, int cls) {
 
 // ---------------------------------------------------------------------------
 // Inverse row pass: d -> v (which 0, one polynomial) or the P-limbs of acc -> vp (which 1,
-// both polynomials, one group of 64 threads each, sharing the twiddle slab). Canonical
-// output for the column pass. Bound by the integer pipe and the twiddle slab's traffic
+// both polynomials, one group of 64 threads each, sharing the twiddle slab). Lazy output
+// (inv_between), within the bounds that col_inv starts from. Bound by the integer pipe and the twiddle slab's traffic
 // (16 bytes per point against 8 in and 8 out).
 template <int LOGN>
 __global__ void __launch_bounds__(128, row_blocks(LOGN))

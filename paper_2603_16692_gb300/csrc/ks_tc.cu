@@ -490,11 +490,11 @@ bool build_items(const ks_context *c, const Tasks &tk, bool up, TcItems &ti) {
 
 int sm_count(int dev) {
   static int cached[64] = {};
-  if (dev < 0 || dev >= 64) return 148;
+  if (dev < 0 || dev >= 64) return kSms;
   if (!cached[dev]) {
     int n = 0;
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cached[dev] = n > 0 ? n : 148;
+    cached[dev] = n > 0 ? n : kSms;
   }
   return cached[dev];
 }
