@@ -451,15 +451,18 @@ int run_plan(ks_context *c, const Plan &pl, const JobSet &js, cudaStream_t s,
 // capture apart from the same stream outside it; operations before the last have completed
 // by then); an input that it overlaps, or a stream without an entry, is waited for.
 class InputOrder {
-  // A stream by its handle (the two names of the legacy stream as one, the per-thread stream
-  // by its thread too) and, under capture, the capture. (cudaStreamGetId would invalidate a
-  // capture. A handle that names a new stream finds the old one's entry, to no harm: what
-  // another stream has queued is waited for through events, which the launches keep.)
+  // A stream by its handle (the two names of the legacy stream as one; it and the per-thread
+  // stream by the device too, the latter by its thread) and, under capture, the capture.
+  // (cudaStreamGetId would invalidate a capture. A handle that names a new stream finds the
+  // old one's entry, to no harm: what another stream has queued is waited for through events,
+  // which the launches keep.)
   struct Key {
     uintptr_t stream = 0, thread = 0;
+    int device = 0;
     unsigned long long capture = 0;
     bool operator==(const Key &o) const {
-      return stream == o.stream && thread == o.thread && capture == o.capture;
+      return stream == o.stream && thread == o.thread && device == o.device &&
+             capture == o.capture;
     }
   };
   struct Slot {
@@ -482,6 +485,10 @@ class InputOrder {
     if (st == cudaStreamCaptureStatusNone) k->capture = 0;
     k->stream = s == cudaStreamLegacy ? 0 : (uintptr_t)s;
     k->thread = s == cudaStreamPerThread ? (uintptr_t)&tag : 0;
+    if ((k->stream == 0 || k->thread) && cudaGetDevice(&k->device) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
     return true;
   }
   Slot *find(const Key &k) {
