@@ -328,7 +328,10 @@ typedef struct {
 #define KS_BATCH_AUTOTUNE 0x2 /* ks_tune each context first (once per group size) */
 #define KS_BATCH_PERSISTENT 0x4 /* run the whole batch in persistent kernels, one per
                                    stage over every job (every job's N in
-                                   2^13..2^17; plans DPOB, fused) */
+                                   2^13..2^17; plans DPOB, fused). On kernels of its own, with
+                                   integer conversions: slower than one ks_switch per job
+                                   (64 uneven jobs 21.4 ms against 18.5, and 15.8 with
+                                   KS_BATCH_GRAPH on tuned plans) */
 #define KS_BATCH_SELECT 0x8  /* jobs naming KS_AUTO run the plan of the installed selector
                                 network (ks_select, run once per context and selector);
                                 not with KS_BATCH_AUTOTUNE or KS_BATCH_PERSISTENT */
@@ -439,7 +442,9 @@ int ks_select(ks_context *ctx, int *variant, int *chunks, void *stream);
  * ks_profile_end every kernel launch made by ks_switch on this thread is bracketed
  * by an event pair on its stream and tagged with its algorithmic traffic (the
  * bytes it must read and write at least: each input and output once) and its
- * modular operation count (butterflies, multiply-accumulates, scalings).
+ * modular operation count (butterflies, multiply-accumulates, scalings). The names are
+ * those of the stages that the launched kernels do: "fused_..." where a cluster kernel
+ * does a whole step (N = 2^12..2^14).
  * ks_profile_end synchronizes those events and aggregates them by kernel name. */
 typedef struct {
   char name[40];

@@ -4,7 +4,9 @@ A 6 -> 64 -> 64 -> 4 FP32 MLP predicts the latency of four candidate plans from
 workload features; the selected plan is the argmin. The candidates are the plans
 that compete on GB300 in the library's own sweep of ten plans (four dataflows x
 radix 8 / radix 4, OutputChunked with 2 and 4 chunks): DPOB, DSOB, DPOB with
-radix-4 rounds, and DPOC with 2 chunks. Output 0 is the log-latency of DPOB,
+radix-4 rounds, and DPOC with 2 chunks. (The committed sweep was taken when the radix named
+different kernels at every N; at N >= 2^12 DPOB and DPOB with radix-4 rounds are the same
+kernels now, and a pick of either runs them.) Output 0 is the log-latency of DPOB,
 outputs 1-3 the log-ratios of the other candidates to it (each output standardised
 over the training rows): the latencies span three orders of magnitude across
 workloads while the choice depends on differences of a few percent, which an
